@@ -33,6 +33,24 @@ def test_stack_stats_bit_exact(ctx, n, w, h):
     np.testing.assert_array_equal(var.cpu().numpy(), ov)
 
 
+@pytest.mark.parametrize("n,w,h", [(257, 10, 3), (512, 17, 2), (3, 4096, 9)])
+def test_stack_stats_blocks(ctx, n, w, h):
+    """More frames than one block of 32-bit partial sums (with an odd last frame), rows of even and
+    odd width, full-scale samples, a constant pixel (variance 0) and
+    one that is 1 once: bit-exact like the rest."""
+    r = np.random.default_rng(n)
+    frames = np.zeros((n, h, synth.pitch_for(w)), np.uint16)
+    frames[:, :, :w] = r.integers(65400, 65536, (n, h, w))
+    frames[:, 0, 0] = 65535
+    frames[:, 0, 1] = r.integers(0, 4096, n)
+    frames[:, 1, 2] = 0
+    frames[0, 1, 2] = 1
+    mean, var = ctx.calib_stack_stats(torch.from_numpy(frames).cuda(), w)
+    om, ov = calib.stack_stats(frames, w)
+    np.testing.assert_array_equal(mean.cpu().numpy(), om)
+    np.testing.assert_array_equal(var.cpu().numpy(), ov)
+
+
 def test_gain_and_exposure_match_the_oracle(ctx):
     g = 2.0
     prnu = (1.0 + 0.02 * np.random.default_rng(3).standard_normal((96, 128))).clip(0.9, 1.1)
