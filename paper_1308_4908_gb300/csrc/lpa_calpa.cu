@@ -3,6 +3,7 @@
 // modes of the reconstruction kernel (lpa_kernel.cuh).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -19,69 +20,162 @@ struct MetricArgs {
   const float2 *grad;
   float *metric;
   int W, H, r;
+  int cells;                       // cells of the disc (pixels whose disc lies inside the image)
   int rw[2 * kRmax + 1];           // half width of the disc in row offset dj (|di| <= rw)
-  double w[2 * kRmax * kRmax + 1];  // Gaussian weight by di^2 + dj^2
-  double scale2;                    // grad_scale^2: T of the scaled gradients
+  float2 w[2 * kRmax * kRmax + 1];  // Gaussian weight by di^2 + dj^2, as a pair
+  // grad_scale = unit m with unit a power of two (the gradients are staged times it, exactly) and
+  // m in [1, 2): T of the scaled gradients is m^2 (a pair) times the sums
+  float unit;
+  float2 m2;
   float alpha, lambda1, lambda2, min_eig, max_eig;
 };
 
+// Pairs of FP32 numbers (x + y unevaluated, |y| <= ulp(x) / 2): about 46 significant bits, from the
+// error-free sum (Knuth) and product (FMA residual). An FP64 instruction takes 16 cycles of an SM
+// here, a pair operation a handful of FP32 issue slots.
+__device__ __forceinline__ float2 pair_norm(float h, float l) {
+  const float s = __fadd_rn(h, l);
+  return make_float2(s, __fsub_rn(l, __fsub_rn(s, h)));
+}
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x), z = __fsub_rn(s, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, z)), __fsub_rn(b.x, z));
+  const float t = __fadd_rn(a.y, b.y), y = __fsub_rn(t, a.y);
+  const float f = __fadd_rn(__fsub_rn(a.y, __fsub_rn(t, y)), __fsub_rn(b.y, y));
+  const float2 u = pair_norm(s, __fadd_rn(e, t));
+  return pair_norm(u.x, __fadd_rn(u.y, f));
+}
+__device__ __forceinline__ float2 pair_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  return pair_norm(p, fmaf(a.x, b.y, fmaf(a.y, b.x, __fmaf_rn(a.x, b.x, -p))));
+}
+__device__ __forceinline__ float2 pair_sqrt(float2 a) {  // a >= 0
+  if (!(a.x > 0.f)) return make_float2(a.x, 0.f);
+  const float s = sqrtf(a.x);
+  return pair_norm(s, (__fmaf_rn(-s, s, a.x) + a.y) / (2.f * s));
+}
+
 // One thread per output pixel. The gradients of the block and its halo are staged in shared
-// memory as the FP64 products gx^2, gx gy, gy^2 (exact: products of two FP32 values), so each
-// neighbour costs three FP64 FMAs. T = sum_i w_i g_i g_i^T over the disc is summed in FP64: T of
-// a straight edge is nearly rank one, and its small eigenvalue is the difference of large sums.
-// The eigenvalues l1,2 = h +- sqrt(((a - c) / 2)^2 + b^2) and the components of the eigenvector
-// of l1 ((b, l1 - a) or (l1 - c, b), the longer) are formed in FP64 too; what follows them (square
-// roots, the direction's normalisation, elongation, the power and the matrix) has no cancellation
-// and runs in FP32.
+// memory as the products gx^2, gx gy, gy^2, each an exact FP32 pair, and T = sum_i w_i g_i g_i^T
+// over the disc is summed in pairs: T of a straight edge is nearly rank one, and its small
+// eigenvalue is the difference of large sums. The eigenvalues l1,2 = h +- sqrt(((a - c) / 2)^2 + b^2)
+// and the components of the eigenvector of l1 ((b, l1 - a) or (l1 - c, b), the longer) are formed in
+// pairs too; what follows them (square roots, the direction's normalisation, elongation, the power
+// and the matrix) has no cancellation and runs in FP32.
+//
+// Bound by the FP32 pipe: 36 pipe cycles per warp and disc cell (12 operations on each of three
+// sums, gx^2 and gy^2 side by side in paired instructions). The same sums in FP64 kept the FP64
+// pipe 84 % busy: gradients and matrices of 1920 x 1080 with 29 cells took 751 us, with this kernel
+// 324 us.
 __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__ MetricArgs A) {
-  constexpr int kTile = (kBY + 2 * kRmax) * (kBX + 2 * kRmax);
-  __shared__ double sxx[kTile], sxy[kTile], syy[kTile];
+  extern __shared__ __align__(16) float4 sm[];
   const int r = A.r, TW = kBX + 2 * r, TH = kBY + 2 * r;
+  float4 *sd = sm;                                        // (gx^2, gy^2, their residuals)
+  float2 *sx = reinterpret_cast<float2 *>(sm + TW * TH);  // (gx gy, its residual)
   // one-dimensional grid over the 32 x 8 blocks (any output height)
   const int nbx = (A.W + kBX - 1) / kBX;
   const int bx0 = (int)(blockIdx.x % nbx) * kBX, by0 = (int)(blockIdx.x / nbx) * kBY;
-  const int tid = threadIdx.y * kBX + threadIdx.x;
-  for (int e = tid; e < TW * TH; e += kBX * kBY) {
-    const int X = bx0 - r + e % TW, Y = by0 - r + e / TW;
-    const float2 g = (X >= 0 && X < A.W && Y >= 0 && Y < A.H) ? A.grad[(size_t)Y * A.W + X] : make_float2(0.f, 0.f);
-    const double gx = g.x, gy = g.y;
-    sxx[e] = gx * gx;
-    sxy[e] = gx * gy;
-    syy[e] = gy * gy;
+  for (int ty = threadIdx.y; ty < TH; ty += kBY) {
+    const int Y = by0 - r + ty;
+    const float2 *row = A.grad + (size_t)max(Y, 0) * A.W;
+    for (int tx = threadIdx.x; tx < TW; tx += kBX) {
+      const int X = bx0 - r + tx;
+      float2 g = (X >= 0 && X < A.W && Y >= 0 && Y < A.H) ? row[X] : make_float2(0.f, 0.f);
+      g = make_float2(g.x * A.unit, g.y * A.unit);
+      const float xx = __fmul_rn(g.x, g.x), yy = __fmul_rn(g.y, g.y), xy = __fmul_rn(g.x, g.y);
+      sd[ty * TW + tx] = make_float4(xx, yy, __fmaf_rn(g.x, g.x, -xx), __fmaf_rn(g.y, g.y, -yy));
+      sx[ty * TW + tx] = make_float2(xy, __fmaf_rn(g.x, g.y, -xy));
+    }
   }
   __syncthreads();
   const int u = bx0 + threadIdx.x, v = by0 + threadIdx.y;
   if (u >= A.W || v >= A.H) return;
-  double a = 0.0, b = 0.0, c = 0.0;
-  int M = 0;
+  const float2 minus = make_float2(-1.f, -1.f);
+  float2 S = make_float2(0.f, 0.f), E = S;  // (sum w gx^2, sum w gy^2) and what rounding dropped
+  float s = 0.f, e = 0.f;                   // the same of sum w gx gy
   for (int dj = -r; dj <= r; dj++) {
-    const int vv = v + dj;
-    if (vv < 0 || vv >= A.H) continue;
     const int rw = A.rw[dj + r];
-    M += min(u + rw, A.W - 1) - max(u - rw, 0) + 1;  // disc cells of this row inside the image
-    const int row = (threadIdx.y + r + dj) * TW + threadIdx.x + r;
+    const int at = (threadIdx.y + r + dj) * TW + threadIdx.x + r;
+#pragma unroll 2
     for (int di = -rw; di <= rw; di++) {
-      const double wt = A.w[di * di + dj * dj];
-      a = fma(wt, sxx[row + di], a);
-      b = fma(wt, sxy[row + di], b);
-      c = fma(wt, syy[row + di], c);
+      const float2 w = A.w[di * di + dj * dj];
+      const float4 d = sd[at + di];
+      const float2 x = sx[at + di];
+      {
+        const float2 X = make_float2(d.x, d.y), W = make_float2(w.x, w.x);
+        const float2 P = __fmul2_rn(W, X);
+        float2 q = __ffma2_rn(W, X, make_float2(-P.x, -P.y));
+        q = __ffma2_rn(W, make_float2(d.z, d.w), q);
+        q = __ffma2_rn(make_float2(w.y, w.y), X, q);
+        const float2 t = __fadd2_rn(S, P), z = __ffma2_rn(S, minus, t);
+        const float2 k = __ffma2_rn(__ffma2_rn(z, minus, t), minus, S);  // S - (t - z)
+        E = __fadd2_rn(E, __fadd2_rn(__fadd2_rn(k, __ffma2_rn(z, minus, P)), q));
+        S = t;
+      }
+      {
+        const float p = __fmul_rn(w.x, x.x);
+        const float q = fmaf(w.y, x.x, fmaf(w.x, x.y, __fmaf_rn(w.x, x.x, -p)));
+        const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+        const float k = __fsub_rn(s, __fsub_rn(t, z));
+        e = __fadd_rn(e, __fadd_rn(__fadd_rn(k, __fsub_rn(p, z)), q));
+        s = t;
+      }
     }
   }
-  a *= A.scale2;
-  b *= A.scale2;
-  c *= A.scale2;
-  const double h = 0.5 * (a + c), d = sqrt(0.25 * (a - c) * (a - c) + b * b);
-  const double l1 = h + d, l2 = fmax(h - d, 0.0);
-  double vx = b, vy = l1 - a;
-  const double fx = l1 - c, fy = b;
-  if (fx * fx + fy * fy > vx * vx + vy * vy) {
-    vx = fx;
-    vy = fy;
+  int M = A.cells;
+  if (u < r || v < r || u + r >= A.W || v + r >= A.H) {  // disc cells inside the image
+    M = 0;
+    for (int dj = -r; dj <= r; dj++) {
+      const int rw = A.rw[dj + r];
+      if (v + dj >= 0 && v + dj < A.H) M += min(u + rw, A.W - 1) - max(u - rw, 0) + 1;
+    }
   }
-  // the direction to FP32 with its exponent removed exactly (no underflow for tiny T)
-  int ex = 0;
-  frexp(fmax(fabs(vx), fabs(vy)), &ex);
-  float ux = (float)ldexp(vx, -ex), uy = (float)ldexp(vy, -ex);
+  // T brought to [1, 2) by a power of two, so that the squares below neither overflow nor underflow
+  const int et = min(max((__float_as_int(fmaxf(S.x, S.y)) >> 23) & 255, 1), 253);
+  const float up = __int_as_float(et << 23), down = __int_as_float((254 - et) << 23);
+  const float2 a = pair_mul(pair_norm(S.x * down, E.x * down), A.m2);
+  const float2 c = pair_mul(pair_norm(S.y * down, E.y * down), A.m2);
+  const float2 b = pair_mul(pair_norm(s * down, e * down), A.m2);
+  const float2 sum = pair_add(a, c), dif = pair_add(a, pair_neg(c));
+  const float2 h = make_float2(0.5f * sum.x, 0.5f * sum.y), t = make_float2(0.5f * dif.x, 0.5f * dif.y);
+  const float2 d = pair_sqrt(pair_add(pair_mul(t, t), pair_mul(b, b)));
+  const float2 l1 = pair_add(h, d), l2 = pair_add(h, pair_neg(d));
+  // the eigenvector's longer form: |l1 - c| > |l1 - a| where a > c
+  float ux = b.x, uy = b.x;
+  if (dif.x > 0.f) ux = pair_add(l1, pair_neg(c)).x;
+  else uy = pair_add(l1, pair_neg(a)).x;
+  float L1 = l1.x * up, L2 = fmaxf(l2.x, 0.f) * up;
+  // Nearly rank one: the pairs hold l2 to about 2^-45 l1, less than an FP32 value needs below this
+  // ratio (noise keeps it above in camera frames; a lone gradient or a clean ramp is below), so T and
+  // its eigenvalues are formed again in FP64.
+  if (l2.x < 0x1p-18f * l1.x) {
+    double da = 0.0, db = 0.0, dc = 0.0;
+    for (int dj = -r; dj <= r; dj++) {
+      const int rw = A.rw[dj + r], at = (threadIdx.y + r + dj) * TW + threadIdx.x + r;
+      for (int di = -rw; di <= rw; di++) {
+        const float2 wp = A.w[di * di + dj * dj], x = sx[at + di];
+        const float4 q = sd[at + di];
+        const double w = (double)wp.x + (double)wp.y;
+        da = fma(w, (double)q.x + (double)q.z, da);
+        db = fma(w, (double)x.x + (double)x.y, db);
+        dc = fma(w, (double)q.y + (double)q.w, dc);
+      }
+    }
+    const double m2 = ((double)A.m2.x + (double)A.m2.y) * (double)down;
+    da *= m2;
+    db *= m2;
+    dc *= m2;
+    const double dh = 0.5 * (da + dc), dd = sqrt(0.25 * (da - dc) * (da - dc) + db * db);
+    L1 = (float)(dh + dd) * up;
+    L2 = (float)fmax(dh - dd, 0.0) * up;
+    ux = da > dc ? (float)(dh + dd - dc) : (float)db;
+    uy = da > dc ? (float)db : (float)(dh + dd - da);
+  }
+  const int ex = (__float_as_int(fmaxf(fabsf(ux), fabsf(uy))) >> 23) & 255;  // its exponent removed, exactly
+  const float unit = __int_as_float(min(max(253 - ex, 1), 254) << 23);
+  ux *= unit;
+  uy *= unit;
   const float n2 = ux * ux + uy * uy;
   if (n2 == 0.f) {  // T = 0
     ux = 1.f;
@@ -91,7 +185,7 @@ __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__
     ux /= nrm;
     uy /= nrm;
   }
-  const float s1 = sqrtf((float)l1), s2 = sqrtf((float)l2);
+  const float s1 = sqrtf(L1), s2 = sqrtf(L2);
   const float elong = (s1 + A.lambda1) / (s2 + A.lambda1);
   const float gamma = powf((s1 * s2 + A.lambda2) / (float)M, A.alpha);
   const float ea = fminf(fmaxf(gamma * elong, A.min_eig), A.max_eig);  // along u1: across the edge
@@ -194,16 +288,21 @@ hdr_status hdr_calpa_metric(hdr_ctx *ctx, int32_t out_w, int32_t out_h, const hd
     while (rw + 1 <= A.r && (double)((rw + 1) * (rw + 1) + dj * dj) <= R * R) rw++;
     A.rw[dj + A.r] = rw;
   }
-  for (int k = 0; k <= 2 * A.r * A.r; k++) A.w[k] = std::exp(-(double)k / (2.0 * ws * ws));
-  A.scale2 = calpa->grad_scale * calpa->grad_scale;
+  auto pair = [](double x) { return make_float2((float)x, (float)(x - (double)(float)x)); };
+  A.cells = 0;
+  for (int dj = -A.r; dj <= A.r; dj++) A.cells += 2 * A.rw[dj + A.r] + 1;
+  for (int k = 0; k <= 2 * A.r * A.r; k++) A.w[k] = pair(std::exp(-(double)k / (2.0 * ws * ws)));
+  A.unit = (float)std::ldexp(1.0, std::max(std::ilogb(calpa->grad_scale), -100));
+  const double m = calpa->grad_scale / (double)A.unit;
+  A.m2 = pair(m * m);
   A.alpha = (float)calpa->alpha;
   A.lambda1 = (float)calpa->lambda1;
   A.lambda2 = (float)calpa->lambda2;
   A.min_eig = (float)calpa->min_eig;
   A.max_eig = (float)calpa->max_eig;
   const unsigned blocks = (unsigned)(((long long)out_w + kBX - 1) / kBX * (((long long)out_h + kBY - 1) / kBY));
-  calpa_metric<<<blocks, dim3(kBX, kBY), 0,
-                 (cudaStream_t)cuda_stream>>>(A);
+  const size_t smem = (size_t)(kBX + 2 * A.r) * (kBY + 2 * A.r) * (sizeof(float4) + sizeof(float2));  // at most 35 KB
+  calpa_metric<<<blocks, dim3(kBX, kBY), smem, (cudaStream_t)cuda_stream>>>(A);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return lpa_fail(HDR_E_CUDA, cudaGetErrorString(e));
   return HDR_OK;

@@ -295,3 +295,23 @@ def test_metric_of_a_tall_thin_output(ctx):
     ctx.check()
     check_metric(q, oracle.steering_metric(g.astype(np.float64), c.window_sigma, c.alpha, c.lambda1, c.lambda2,
                                            c.min_eig, c.max_eig, c.grad_scale))
+
+
+@pytest.mark.parametrize("window_sigma,grad_scale", [(0.34, 1.0), (1.0, 0.1), (1.06, 3e-3), (3.6, 0.1)])
+def test_metric_windows_and_near_rank_one(ctx, window_sigma, grad_scale):
+    """Discs of radius 1, 3 (two memberships) and 10 on a ragged 45 x 37 plane: gradients spanning two
+    decades, a ramp with 1e-4 relative noise (its matrix is of rank one to about 1e-8, where the
+    kernel sums in FP64), a lone gradient along x (exactly rank one) and none at all. Discs of
+    radius 1 keep gradients everywhere: beside an empty block they would hold one oblique gradient,
+    where FP64 itself (the oracle included: 7e-4 against long double) does not resolve the zero
+    eigenvalue."""
+    r = np.random.default_rng(int(1000 * window_sigma))
+    g = (10.0 ** r.uniform(0.0, 2.0, (37, 45, 1)) * r.standard_normal((37, 45, 2))).astype(np.float32)
+    g[:14, :14] = np.array([300.0, 170.0]) * (1.0 + 1e-4 * r.standard_normal((14, 14, 2)))
+    if window_sigma > 0.5:
+        g[16:, 20:] = 0.0
+        g[30, 35] = (2048.0, 0.0)
+    c = _calpa(window_sigma=window_sigma, grad_scale=grad_scale)
+    q = ctx.calpa_metric(c, torch.from_numpy(g).cuda()).cpu().numpy()
+    check_metric(q, oracle.steering_metric(g.astype(np.float64), c.window_sigma, c.alpha, c.lambda1, c.lambda2,
+                                           c.min_eig, c.max_eig, c.grad_scale))
