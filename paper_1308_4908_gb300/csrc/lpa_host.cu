@@ -283,6 +283,7 @@ struct PlanEnv {
   int device;
   PlanCache *tabs;  // NULL: no caches (the entry point may not allocate): nothing tabulated
   bool tabulate;    // tabulated weights allowed (the persistent batch kernels search every window)
+  bool single = true;  // frames with one scale may leave the variance sums out (LPA_ONE)
 };
 
 bool is_identity_linear(const double *a) {
@@ -318,7 +319,8 @@ size_t conv_elems(const Rig &rig) {
   return n;
 }
 
-hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p, bool f64_possible, LpaLaunch &L) {
+hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p, bool f64_possible, bool one,
+                        LpaLaunch &L) {
   L.tab_hdr = nullptr;
   L.tab_cells = nullptr;
   L.tab_nsp = 0;
@@ -330,7 +332,8 @@ hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p,
   for (int s = 0; s < rig.n; s++)
     if (!is_identity_linear(rig.s[s].d.affine)) return HDR_OK;
   const int J = p->n_scales;
-  const int nsp = lpa_scales_per_walk(p->order, p->accum != 0, f64_possible ? LPA_TABULATED : LPA_TABULATED_F32);
+  const int tab_mode = one ? LPA_TABULATED_ONE : LPA_TABULATED;
+  const int nsp = lpa_scales_per_walk(p->order, p->accum != 0, f64_possible ? tab_mode : lpa_mode_to_f32(tab_mode));
   const int npass = lpa_n_passes(J, nsp);
   std::vector<double> inputs = {(double)rig.n, (double)J, p->trunc_k, p->green_ratio, (double)nsp};
   for (int j = 0; j < J; j++) inputs.push_back(p->sigma[j]);
@@ -346,7 +349,7 @@ hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p,
     L.tab_hdr = static_cast<const int4 *>(known->second);
     L.tab_cells = reinterpret_cast<const float4 *>(static_cast<const int4 *>(known->second) + n_hdr);
     L.tab_nsp = nsp;
-    L.mode = LPA_TABULATED;
+    L.mode = tab_mode;
     return HDR_OK;
   }
   const double taper = std::exp(-0.5 * p->trunc_k * p->trunc_k);
@@ -474,7 +477,7 @@ hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p,
   L.tab_hdr = static_cast<const int4 *>(it->second);
   L.tab_cells = reinterpret_cast<const float4 *>(static_cast<const int4 *>(it->second) + hdr.size());
   L.tab_nsp = nsp;
-  L.mode = LPA_TABULATED;
+  L.mode = tab_mode;
   return HDR_OK;
 }
 
@@ -630,8 +633,10 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   if (p->weight_mode == 1) {  // the printed noise weight K / s: searched window, its own kernel
     L.mode = LPA_LITERAL;
   } else {
-    hdr_status st = build_tables(env, rig, p, f64_possible, L);
+    const bool one = env.single && stages != 2 && p->n_scales == 1;
+    hdr_status st = build_tables(env, rig, p, f64_possible, one, L);
     if (st) return st;
+    if (one && L.mode == LPA_SEARCHED) L.mode = LPA_ONE;
   }
   if (!f64_possible) L.mode = lpa_mode_to_f32(L.mode);
   if (!lpa_mode_tab(L.mode)) {  // each thread's sample cell in each sensor (tables need none)
@@ -664,8 +669,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
 }
 
 hdr_status plan(hdr_ctx *ctx, const Rig &rig, const hdr_params *p, const uint16_t *const *raw, LpaLaunch &L,
-                double reach = 1.0, bool tabulate = true, int stages = 1, float2 *conv = nullptr) {
-  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, tabulate}, rig, p, raw, L,
+                double reach = 1.0, bool levels = false, int stages = 1, float2 *conv = nullptr) {
+  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels}, rig, p, raw, L,
                   LPA_FRAME_TILE_H, reach, stages, conv);
 }
 
@@ -719,7 +724,7 @@ hdr_status convert_rows(hdr_ctx *ctx, const LpaLaunch &L, const LpaRows &rows, b
 
 // plan() of a single-frame call through the context's plan cache.
 hdr_status cached_plan(hdr_ctx *ctx, int32_t rig_id, const hdr_params *p, const uint16_t *const *raw, LpaLaunch &L,
-                       bool tabulate, int stages, float2 *conv) {
+                       bool levels, int stages, float2 *conv) {
   const Rig &rig = ctx->rigs[rig_id];
   std::vector<uint8_t> key(sizeof(int32_t) + 2 * sizeof(uint64_t) + sizeof(hdr_params) + 2 + (rig.n + 1) * sizeof(void *));
   uint8_t *k = key.data();
@@ -731,7 +736,7 @@ hdr_status cached_plan(hdr_ctx *ctx, int32_t rig_id, const hdr_params *p, const 
   k += sizeof(uint64_t);
   memcpy(k, p, sizeof(hdr_params));
   k += sizeof(hdr_params);
-  *k++ = tabulate ? 1 : 0;
+  *k++ = levels ? 1 : 0;
   *k++ = (uint8_t)stages;
   memcpy(k, &conv, sizeof(void *));
   k += sizeof(void *);
@@ -741,7 +746,7 @@ hdr_status cached_plan(hdr_ctx *ctx, int32_t rig_id, const hdr_params *p, const 
     L = it->second;
     return HDR_OK;
   }
-  hdr_status st = plan(ctx, rig, p, raw, L, 1.0, tabulate, stages, conv);
+  hdr_status st = plan(ctx, rig, p, raw, L, 1.0, levels, stages, conv);
   if (st) return st;
   if (ctx->plans.size() >= 256) ctx->plans.clear();
   ctx->plans.emplace(std::move(key), L);
@@ -783,7 +788,7 @@ hdr_status reconstruct_impl(hdr_ctx *ctx, int32_t rig_id, const hdr_params *para
   st = conv_buffer(ctx, ctx->rigs[rig_id], params, &conv);
   if (st) return st;
   // the diagnostic (level maps) kernel searches every window
-  st = cached_plan(ctx, rig_id, params, raw_dev, L, levels_dev == nullptr, levels_dev ? 1 : LPA_FRAME_STAGES, conv);
+  st = cached_plan(ctx, rig_id, params, raw_dev, L, levels_dev != nullptr, levels_dev ? 1 : LPA_FRAME_STAGES, conv);
   if (st) return st;
   L.out = out_dev;
   L.choice = choice_dev;
@@ -1038,7 +1043,7 @@ hdr_status hdr_reconstruct_host(hdr_ctx *ctx, int32_t rig_id, const hdr_params *
   float2 *conv = nullptr;
   st = conv_buffer(ctx, rig, params, &conv);
   if (st) return st;
-  st = cached_plan(ctx, rig_id, params, raw_dev, L, true, LPA_FRAME_STAGES, conv);
+  st = cached_plan(ctx, rig_id, params, raw_dev, L, false, LPA_FRAME_STAGES, conv);
   if (st) return st;
   L.out = ctx->out_stage;
   L.choice = choice_host ? ctx->choice_stage : nullptr;
@@ -1270,7 +1275,7 @@ hdr_status batch_plan(hdr_ctx *ctx, int n, const hdr_frame *frames, const int2 *
   for (int f = 0; f < n; f++) {
     const hdr_frame &F = frames[f];
     // no tables: the persistent kernels search every window
-    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, false}, ctx->rigs[F.rig_id],
+    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, false, false}, ctx->rigs[F.rig_id],
                              F.params, F.raw_dev, plans[f], cfg.tile_h);
     if (st) return fail(st, "frame %d: %s", f, g_err.c_str());
     if (plans[f].mode != LPA_SEARCHED && plans[f].mode != LPA_SEARCHED_F32)
@@ -1390,7 +1395,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       pp = &sp;
     }
     const int px = (cfg.px_per_thread == 2 && !F.calpa) ? 2 : 1;
-    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !F.calpa}, ctx->rigs[F.rig_id],
+    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !F.calpa, px == 1}, ctx->rigs[F.rig_id],
                              pp, F.raw_dev, plans[f], F.calpa ? 16 : cfg.tile_h,
                              F.calpa ? lpa_calpa_reach(F.calpa) : 1.0, (F.calpa || px != 1) ? 1 : cfg.stages,
                              F.calpa ? nullptr : cv[f]);
@@ -1672,7 +1677,7 @@ hdr_status lpa_launch_mode(hdr_ctx *ctx, int32_t rig_id, const hdr_params *param
     if (s) return s;
   }
   LpaLaunch L;
-  s = plan(ctx, ctx->rigs[rig_id], &p, raw_dev, L, reach, true, 1, conv);
+  s = plan(ctx, ctx->rigs[rig_id], &p, raw_dev, L, reach, false, 1, conv);
   if (s) return s;
   if (L.conv) {  // the frame converted once, then the pass
     s = convert_rows(ctx, L, all_rows(L), true, st);

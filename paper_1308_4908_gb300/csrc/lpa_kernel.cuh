@@ -54,8 +54,11 @@ __device__ __forceinline__ void comp_add(float &hi, float &lo, float a, float b)
   lo = __fadd_rn(lo, __fadd_rn(e, pe));
 }
 
-template <int ORDER, bool COMP>
+// VAR: the variance sums are kept (they are not where no interval is formed: one window scale, the
+// gradient pass).
+template <int ORDER, bool COMP, bool VAR = true>
 struct Moments {
+  static constexpr bool HAS_VAR = VAR;
   static constexpr int NA = n_monos(ORDER);     // sum w d^a d^b, a+b <= 2M
   static constexpr int NB = n_unknowns(ORDER);  // sum w f phi
   float a[NA], b[NB], k[NA];                    // k: sum w K d^a d^b (variance of C_0)
@@ -81,11 +84,11 @@ struct Moments {
   __device__ __forceinline__ void add0(float w, float wf, float wk, float one) {
     if (COMP) {
       comp_add(a[0], al[0], w, 1.f);
-      comp_add(k[0], kl[0], wk, 1.f);
+      if (VAR) comp_add(k[0], kl[0], wk, 1.f);
       comp_add(b[0], bl[0], wf, 1.f);
     } else {
       a[0] += w;
-      k[0] += wk;
+      if (VAR) k[0] += wk;
       b[0] += wf;
     }
     cnt += one;
@@ -116,18 +119,18 @@ struct Moments {
 #pragma unroll
       for (int i = 0; i < NA; i++) {
         comp_add(a[i], al[i], w, m[i]);
-        comp_add(k[i], kl[i], wk, m[i]);
+        if (VAR) comp_add(k[i], kl[i], wk, m[i]);
       }
 #pragma unroll
       for (int i = 0; i < NB; i++) comp_add(b[i], bl[i], wf, m[i]);
     } else {
       a[0] += w;
-      k[0] += wk;
+      if (VAR) k[0] += wk;
       b[0] += wf;
 #pragma unroll
       for (int i = 1; i < NA; i++) {
         a[i] = fmaf(w, m[i], a[i]);
-        k[i] = fmaf(wk, m[i], k[i]);
+        if (VAR) k[i] = fmaf(wk, m[i], k[i]);
       }
 #pragma unroll
       for (int i = 1; i < NB; i++) b[i] = fmaf(wf, m[i], b[i]);
@@ -158,6 +161,7 @@ struct Moments {
 // Blackwell issues two FP32 operations per paired instruction, so fewer instructions are issued.
 template <int ORDER>
 struct MomentsPacked {
+  static constexpr bool HAS_VAR = true;
   static constexpr int NA = n_monos(ORDER);
   static constexpr int NB = n_unknowns(ORDER);
   float2 ak[NA];  // (sum w m_i, sum w K m_i)
@@ -229,14 +233,86 @@ struct MomentsPacked {
   __device__ __forceinline__ T Kv(int i) const { return (T)ak[i].y; }
 };
 
+// The plain FP32 sums without the variance sums: the Gram sums in the pairs the monomials come in
+// ((m_1, m_2) = D, (m_3, m_5) = D2, the paired products of degree 3 and 4; m_4 and m_12 alone), the
+// right-hand side as above. Every sum takes the same terms in the same order with the same
+// roundings as MomentsPacked, in 11 paired and 3 scalar operations a sample instead of 17 and 1 at
+// order 2.
+template <int ORDER>
+struct MomentsLean {
+  static constexpr bool HAS_VAR = false;
+  static constexpr int NA = n_monos(ORDER);
+  static constexpr int NB = n_unknowns(ORDER);
+  float2 a0n;                                  // (sum w, count)
+  float2 a12, a35, a69, a78, aAE, aBD;         // A, B, D, E: monomials 10, 11, 13, 14
+  float a4, aC;                                // C: monomial 12
+  float2 b12, b35;
+  float b0, b4;
+
+  __device__ __forceinline__ void zero() {
+    a0n = a12 = a35 = a69 = a78 = aAE = aBD = b12 = b35 = make_float2(0.f, 0.f);
+    a4 = aC = b0 = b4 = 0.f;
+  }
+  __device__ __forceinline__ float count() const { return a0n.y; }
+  __device__ __forceinline__ void add2(float2 D, float2 D2, float w, float wf, float) {
+    const float2 W = make_float2(w, w), F = make_float2(wf, wf);
+    const float m4 = D.x * D.y;
+    a0n = __fadd2_rn(a0n, make_float2(w, 1.f));
+    a12 = __ffma2_rn(W, D, a12);
+    a35 = __ffma2_rn(W, D2, a35);
+    a4 = fmaf(w, m4, a4);
+    b0 += wf;
+    b12 = __ffma2_rn(F, D, b12);
+    if (NB > 3) {
+      const float2 SW = make_float2(D.y, D.x);
+      const float2 P3 = __fmul2_rn(D2, D), P21 = __fmul2_rn(D2, SW);
+      a69 = __ffma2_rn(W, P3, a69);
+      a78 = __ffma2_rn(W, P21, a78);
+      aAE = __ffma2_rn(W, __fmul2_rn(D2, D2), aAE);
+      aBD = __ffma2_rn(W, __fmul2_rn(P3, SW), aBD);
+      aC = fmaf(w, m4 * m4, aC);
+      b35 = __ffma2_rn(F, D2, b35);
+      b4 = fmaf(wf, m4, b4);
+    }
+  }
+  template <typename T>
+  __device__ __forceinline__ T A(int i) const {
+    return (T)(i == 0    ? a0n.x
+               : i == 1  ? a12.x
+               : i == 2  ? a12.y
+               : i == 3  ? a35.x
+               : i == 4  ? a4
+               : i == 5  ? a35.y
+               : i == 6  ? a69.x
+               : i == 7  ? a78.x
+               : i == 8  ? a78.y
+               : i == 9  ? a69.y
+               : i == 10 ? aAE.x
+               : i == 11 ? aBD.x
+               : i == 12 ? aC
+               : i == 13 ? aBD.y
+                         : aAE.y);
+  }
+  template <typename T>
+  __device__ __forceinline__ T B(int i) const {
+    return (T)(i == 0 ? b0 : i == 1 ? b12.x : i == 2 ? b12.y : i == 3 ? b35.x : i == 4 ? b4 : b35.y);
+  }
+  template <typename T>
+  __device__ __forceinline__ T Kv(int) const { return T(0); }
+};
+
 // The accumulator a kernel uses: paired for plain FP32 sums of order >= 1.
-template <int ORDER, bool COMP, bool PACKED = (LPA_PACKED_MOMENTS != 0) && !COMP && ORDER >= 1>
+template <int ORDER, bool COMP, bool VAR = true, bool PACKED = (LPA_PACKED_MOMENTS != 0) && !COMP && ORDER >= 1>
 struct MomentsSel {
-  using type = Moments<ORDER, COMP>;
+  using type = Moments<ORDER, COMP, VAR>;
 };
 template <int ORDER>
-struct MomentsSel<ORDER, false, true> {
+struct MomentsSel<ORDER, false, true, true> {
   using type = MomentsPacked<ORDER>;
+};
+template <int ORDER>
+struct MomentsSel<ORDER, false, false, true> {
+  using type = MomentsLean<ORDER>;
 };
 
 // ---------------------------------------------------------------- solve
@@ -331,6 +407,7 @@ __device__ __forceinline__ FitOut solve(const MOM &m, float min_pivot) {
 #pragma unroll
   for (int i = 0; i < P; i++) {
     c0 += x[i] * m.template B<T>(i);
+    if (!MOM::HAS_VAR) continue;
     T row = T(0);
 #pragma unroll
     for (int j = 0; j < P; j++)
@@ -618,8 +695,8 @@ __device__ __forceinline__ void walk_sensor(const LpaSensorK &S, int4 pos, int c
   }
 }
 
-template <int ORDER, bool COMP, int MODE = LPA_SEARCHED>
-__device__ __forceinline__ void accumulate_sensor(typename MomentsSel<ORDER, COMP>::type &m, const LpaSensorK &S,
+template <int ORDER, int MODE, class MOM>
+__device__ __forceinline__ void accumulate_sensor(MOM &m, const LpaSensorK &S,
                                                   int4 pos, int c, float R, float R2,
                                                   float cexp, float taper, int x0, int y0,
                                                   const unsigned char *smem, bool active, unsigned *status,
@@ -898,7 +975,7 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
     if constexpr (STEER)
       if (pix) Q = make_float4(L.aux[opix * 3], L.aux[opix * 3 + 1], L.aux[opix * 3 + 2], 0.f);
 
-    using MOM = typename MomentsSel<ORDER, COMP>::type;
+    using MOM = typename MomentsSel<ORDER, COMP, lpa_mode_var(MODE)>::type;
     // the fit of one (channel, scale) from its moments: factorised unless no lane of the warp has as
     // many samples as unknowns (such a fit is not usable whatever its pivots; on near-translational
     // rigs the lanes share one sample layout, so whole warps qualify)
@@ -1016,7 +1093,7 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
         const bool act = DIAG ? pix : !ici.done;
   #pragma unroll 1
         for (int s = 0; s < S; s++)
-          accumulate_sensor<ORDER, COMP, MODE>(m, L.s[s], pos[s * NT], c, R, R2, cexp, RD(L.taper), fp_x0[s],
+          accumulate_sensor<ORDER, MODE>(m, L.s[s], pos[s * NT], c, R, R2, cexp, RD(L.taper), fp_x0[s],
                                                 fp_y0[s], smem, act, RD(L.status), Q);
         const FitOut f = fit_of(m);
         if constexpr (GRAD) {  // Section 5.4: the order-1 fit's linear coefficients; 0 if not usable
@@ -1042,9 +1119,17 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
 #ifndef LPA_M2_CTAS_256
 #define LPA_M2_CTAS_256 2  // resident 256-thread CTAs per SM the multi-scale order-2 kernel is built for
 #endif
+// One scale without variance sums (and the gradient pass): 59 to 64 registers at order 1, 74 at order
+// 2 with the FP64 re-solve compiled out; compensated sums take twice the registers (order 2 on 1024 x
+// 900 pixels of three sensors: 768 us at two CTAs per SM, 804 at three with 52 B of spills).
+template <int ORDER, bool COMP, int MODE>
+struct OneOccupancy {
+  static constexpr int value = ORDER == 1 ? (COMP ? 2 : 4) : !COMP && lpa_mode_f32(MODE) ? 3 : 2;
+};
 template <int ORDER, bool COMP, int TH, int MODE>
 struct FrameOccupancy {
-  static constexpr int value = (ORDER == 2 && MultiScale<ORDER, COMP, MODE>::value > 1) ? LPA_M2_CTAS_256 * 16 / TH
+  static constexpr int value = (!lpa_mode_var(MODE) && ORDER > 0) ? OneOccupancy<ORDER, COMP, MODE>::value * 16 / TH
+                               : (ORDER == 2 && MultiScale<ORDER, COMP, MODE>::value > 1) ? LPA_M2_CTAS_256 * 16 / TH
                                : ORDER == 0                                              ? LPA_M0_CTAS_256 * 16 / TH
                                                                                          : 16 / TH * 2;
 };

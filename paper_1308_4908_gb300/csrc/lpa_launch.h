@@ -102,6 +102,11 @@ struct LpaLaunch {
 // with every fit solved in FP32 only, for parameters under which the FP64 re-solve can never
 // trigger ((min_pivot - 1e-4) * cond_fallback >= 2: a usable fit's equilibrated pivots lie in
 // (min_pivot, 1], so their spread stays below cond_fallback).
+// LPA_ONE, LPA_TABULATED_ONE (and _F32): the searched or tabulated window of a frame with one scale,
+// without the variance sums (15 of the 36 sums of a sample at order 2, 6 of 15 at order 1): the
+// interval rule has nothing to compare, so Var C_0 is not used. The values are those of
+// LPA_SEARCHED and LPA_TABULATED bit for bit. Built for one pixel per thread and one staging buffer
+// (other launches, the level maps and the persistent kernels keep the variance sums).
 enum {
   LPA_SEARCHED = 0,
   LPA_TABULATED = 1,
@@ -110,19 +115,33 @@ enum {
   LPA_LITERAL = 4,
   LPA_SEARCHED_F32 = 5,
   LPA_STEERED_F32 = 6,
-  LPA_TABULATED_F32 = 7
+  LPA_TABULATED_F32 = 7,
+  LPA_ONE = 8,
+  LPA_ONE_F32 = 9,
+  LPA_TABULATED_ONE = 10,
+  LPA_TABULATED_ONE_F32 = 11
 };
 __host__ __device__ constexpr bool lpa_mode_steered(int mode) { return mode == LPA_STEERED || mode == LPA_STEERED_F32; }
-__host__ __device__ constexpr bool lpa_mode_tab(int mode) { return mode == LPA_TABULATED || mode == LPA_TABULATED_F32; }
-__host__ __device__ constexpr bool lpa_mode_f32(int mode) {
-  return mode == LPA_SEARCHED_F32 || mode == LPA_STEERED_F32 || mode == LPA_TABULATED_F32;
+__host__ __device__ constexpr bool lpa_mode_one(int mode) {
+  return mode == LPA_ONE || mode == LPA_ONE_F32 || mode == LPA_TABULATED_ONE || mode == LPA_TABULATED_ONE_F32;
 }
+__host__ __device__ constexpr bool lpa_mode_tab(int mode) {
+  return mode == LPA_TABULATED || mode == LPA_TABULATED_F32 || mode == LPA_TABULATED_ONE || mode == LPA_TABULATED_ONE_F32;
+}
+__host__ __device__ constexpr bool lpa_mode_f32(int mode) {
+  return mode == LPA_SEARCHED_F32 || mode == LPA_STEERED_F32 || mode == LPA_TABULATED_F32 || mode == LPA_ONE_F32 ||
+         mode == LPA_TABULATED_ONE_F32;
+}
+// whether the mode forms Var C_0
+__host__ __device__ constexpr bool lpa_mode_var(int mode) { return !lpa_mode_one(mode) && mode != LPA_GRADIENTS; }
 // the FP32-only variant of a mode, where it has one
 __host__ __device__ constexpr int lpa_mode_to_f32(int mode) {
-  return mode == LPA_SEARCHED    ? LPA_SEARCHED_F32
-         : mode == LPA_STEERED   ? LPA_STEERED_F32
-         : mode == LPA_TABULATED ? LPA_TABULATED_F32
-                                 : mode;
+  return mode == LPA_SEARCHED        ? LPA_SEARCHED_F32
+         : mode == LPA_STEERED       ? LPA_STEERED_F32
+         : mode == LPA_TABULATED     ? LPA_TABULATED_F32
+         : mode == LPA_ONE           ? LPA_ONE_F32
+         : mode == LPA_TABULATED_ONE ? LPA_TABULATED_ONE_F32
+                                     : mode;
 }
 
 // Scales per walk of the window cells: the searched, steered and tabulated windows with plain FP32
@@ -139,6 +158,7 @@ __host__ __device__ constexpr int lpa_mode_to_f32(int mode) {
 #endif
 __host__ __device__ constexpr int lpa_scales_per_walk(int order, bool comp, int mode) {
   return comp ? 1
+         : lpa_mode_one(mode) ? 1
          : lpa_mode_f32(mode)
              ? (order == 2 ? LPA_MULTI_SCALE : order == 1 ? LPA_MULTI_SCALE_LOW : LPA_MULTI_SCALE_M0)
          : (mode == LPA_SEARCHED || mode == LPA_STEERED || mode == LPA_TABULATED)
@@ -158,7 +178,7 @@ struct LpaRows {
 
 // The two-buffer single-frame kernel is built for plain sums with the searched or tabulated window.
 __host__ __device__ constexpr bool lpa_stages2_built(int mode, bool comp) {
-  return !comp && (mode == LPA_SEARCHED || mode == LPA_SEARCHED_F32 || lpa_mode_tab(mode));
+  return !comp && !lpa_mode_one(mode) && (mode == LPA_SEARCHED || mode == LPA_SEARCHED_F32 || lpa_mode_tab(mode));
 }
 // CTAs of a single-frame launch over `tiles` tiles: one per tile, or one per LPA_STAGED_TILES tiles
 // with two staging buffers.

@@ -2,8 +2,8 @@
 // lpa_m0.cu, lpa_m1.cu and lpa_m2.cu, which compile in parallel).
 //
 // Instantiated per order: the searched window (Eq. 8) with and without the level maps, the
-// tabulated window (Section 8), tile heights 8 and 16, and 16-row tiles with two pixels per
-// thread; the steered window (Section 5.4) and the printed noise weight K / s at tile height 16;
+// tabulated window (Section 8), both also for one scale without the variance sums, tile heights 8
+// and 16, and 16-row tiles with two pixels per thread; the steered window (Section 5.4) and the printed noise weight K / s at tile height 16;
 // the gradient pass (Section 5.4) for order 1 only.
 #pragma once
 #include "lpa_dispatch.h"
@@ -13,6 +13,7 @@ namespace lpa_orders {
 
 template <int ORDER, int MODE, int TH, int PX>
 constexpr bool instantiated() {
+  if (PX == 2 && lpa_mode_one(MODE)) return false;
   if (PX == 2)  // two pixels per thread: 16-row tiles of 8-row CTAs, the windows batches use
     return TH == 8 && (MODE == LPA_SEARCHED || MODE == LPA_SEARCHED_F32 || lpa_mode_tab(MODE));
   if (MODE == LPA_GRADIENTS) return ORDER == 1 && TH == 16;
@@ -40,6 +41,10 @@ const void *kernel_mode(int mode) {
     case LPA_SEARCHED_F32: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_SEARCHED_F32, PX, STAGES>();
     case LPA_STEERED_F32: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_STEERED_F32, PX, STAGES>();
     case LPA_TABULATED_F32: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_TABULATED_F32, PX, STAGES>();
+    case LPA_ONE: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_ONE, PX, STAGES>();
+    case LPA_TABULATED_ONE: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_TABULATED_ONE, PX, STAGES>();
+    case LPA_TABULATED_ONE_F32: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_TABULATED_ONE_F32, PX, STAGES>();
+    case LPA_ONE_F32: return kernel_fn<ORDER, COMP, DIAG, TH, LPA_ONE_F32, PX, STAGES>();
     default: return nullptr;
   }
 }
