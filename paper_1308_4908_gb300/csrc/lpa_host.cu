@@ -1457,7 +1457,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 8 + L.mode, comp ? 1 : 0, L.tile_h, L.px, L.stages + 4 * (d >= 0 ? 1 : 0)});
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, L.px, L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};
     r.func = const_cast<void *>(fn);
