@@ -284,6 +284,8 @@ struct PlanEnv {
   PlanCache *tabs;  // NULL: no caches (the entry point may not allocate): nothing tabulated
   bool tabulate;    // tabulated weights allowed (the persistent batch kernels search every window)
   bool single = true;  // frames with one scale may leave the variance sums out (LPA_ONE)
+  bool mean = true;    // small windows of order 0 may run lpa_mean (not the level maps, whose kernel also
+                       // writes Var C_0, nor the persistent batch kernels)
 };
 
 bool is_identity_linear(const double *a) {
@@ -302,9 +304,93 @@ int floor_div2_parity(long long v) { return (int)(((v % 2) + 2) % 2); }
 
 // Frames converted in a pass of their own before the reconstruction: at least one wave of 16x16
 // tiles on the GPU's 152 SMs (smaller frames cost their launches, not the repeated conversion of
-// overlapping footprints), outside the adaptive passes (their kernels convert footprints).
-bool lpa_conv_eligible(const hdr_params *p, bool adaptive) {
-  return LPA_FRAME_CONV && !adaptive && (long long)p->out_w * p->out_h >= 152LL * 256;
+// overlapping footprints), outside the adaptive passes of a batch (their kernels convert footprints)
+// and outside lpa_mean, which reads the raw frames.
+namespace {
+
+struct MeanPlan {
+  int size = -1;      // kernel template, -1: another kernel
+  bool axis = true;   // every sensor's axes are parallel to the output's
+  int p = 1;          // output rows per thread
+  double rb = 0, g = 0;  // window radius of R and B, and of G (reference px)
+};
+// Whether a frame runs lpa_mean: order 0, one scale, plain sums, the inverse-variance weight, and
+// windows of at most 4 x 4 (R, B) and 3 x 3 (G) cells of a colour phase. A fit of one unknown has the
+// equilibrated pivot 1, so it is usable with any sample (min_pivot below 1) and never solved again
+// in FP64 (cond_fallback at least 1, or none); other parameters keep the general kernel.
+// Rows per thread: four once 64 x 32 tiles fill the SMs' two resident CTAs twice (less halo converted
+// per pixel), fewer for smaller frames (more CTAs).
+MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
+  MeanPlan m;
+  if (p->order != 0 || p->n_scales != 1 || p->accum != 0 || p->weight_mode != 0 || !(p->min_pivot < 0.99) ||
+      !(p->cond_fallback <= 0.0 || p->cond_fallback >= 1.0))
+    return m;
+  m.rb = p->trunc_k * p->sigma[0];
+  m.g = m.rb * p->green_ratio;
+  m.axis = p->out_affine[1] == 0.0 && p->out_affine[3] == 0.0;
+  double most = 0.0;
+  for (int s = 0; s < rig.n; s++) {
+    double t[6];
+    invert_affine(rig.s[s].d.affine, t);
+    most = std::max(most, std::max(std::hypot(t[0], t[1]), std::hypot(t[3], t[4])));
+    m.axis = m.axis && t[1] == 0.0 && t[3] == 0.0;
+  }
+  m.size = lpa_mean_size(m.rb * most + 2e-3, m.g * most + 2e-3);
+  const long long px = (long long)p->out_w * p->out_h;
+  m.p = px >= 4LL * 152 * 64 * 32 ? 4 : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
+  return m;
+}
+
+// Staging box of lpa_mean for sensor transform G: the tile's points, `left` px before the first one (the
+// window's reach) and up to the last candidate cell after the last, one px of margin on each side, and
+// the alignment of its origin (x to 8, y to 2).
+void mean_box(const MeanPlan &m, const double G[6], double hxu, double hyu, int *bw, int *bh, float *ext_x, float *ext_y) {
+  const int nr = lpa_mean_cells(m.size, false), ng = lpa_mean_cells(m.size, true);
+  const double w = LPA_MEAN_TILE_W - 1, h = 8 * m.p - 1;
+  auto sides = [&](double unit, float *ext) {
+    const double rb = m.rb * unit + 2e-3, g = m.g * unit + 2e-3;
+    *ext = (float)(std::max(rb, g) + 1.0);
+    return *ext + std::max(2.0 * nr - rb, 2.0 * ng - g) + 1.0;
+  };
+  *bw = ((int)std::ceil(std::fabs(G[0]) * w + std::fabs(G[1]) * h + sides(hxu, ext_x)) + 8 + 7) / 8 * 8;
+  *bh = ((int)std::ceil(std::fabs(G[3]) * w + std::fabs(G[4]) * h + sides(hyu, ext_y)) + 2 + 1) / 2 * 2;
+}
+
+// lpa_mean's shared memory for a rig (two buffers of the largest box's planes, then the tables), or 0
+// where it would leave fewer than two CTAs on an SM.
+uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, uint32_t *plane, uint32_t *tab) {
+  double need = 0.0;
+  for (int s = 0; s < rig.n; s++) {
+    double t[6], G[6];
+    invert_affine(rig.s[s].d.affine, t);
+    compose_affine(t, p->out_affine, G);
+    if (!(std::fabs(G[0]) + std::fabs(G[1]) + std::fabs(G[3]) + std::fabs(G[4]) < 16.0)) return 0;
+    int bw, bh;
+    float ex, ey;
+    mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);
+    need = std::max(need, 8.0 * bw * bh);
+  }
+  const double all = 2.0 * need + lpa_mean_tab_bytes(m.size, m.axis, m.p, rig.n);
+  if (all > 110.0 * 1024) return 0;
+  *plane = (uint32_t)need;
+  *tab = 2u * *plane;
+  return (uint32_t)all;
+}
+
+bool runs_mean(const Rig &rig, const hdr_params *p) {
+  const MeanPlan m = mean_plan(rig, p);
+  uint32_t plane, tab;
+  return m.size >= 0 && mean_smem(rig, p, m, &plane, &tab) > 0;
+}
+
+bool conv_eligible(const Rig &rig, const hdr_params *p, bool adaptive, bool mean = true) {
+  return LPA_FRAME_CONV && !adaptive && (long long)p->out_w * p->out_h >= 152LL * 256 && !(mean && runs_mean(rig, p));
+}
+
+}  // namespace
+
+bool lpa_conv_eligible(const hdr_ctx *ctx, int rig_id, const hdr_params *p, bool adaptive) {
+  return conv_eligible(ctx->rigs[rig_id], p, adaptive);
 }
 
 namespace {
@@ -516,6 +602,13 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   const double rmax = reach * p->trunc_k * p->sigma[p->n_scales - 1] * std::fmax(1.0, p->green_ratio);
   uint32_t off = 0, tx = 0;
   size_t conv_off = 0;
+  MeanPlan mean;
+  if (env.mean) mean = mean_plan(rig, p);
+  if (mean.size >= 0) {
+    L.smem_bytes = mean_smem(rig, p, mean, &L.mean_plane, &L.mean_tab);
+    if (L.smem_bytes == 0) mean.size = -1;
+  }
+  if (mean.size >= 0) conv = nullptr;  // lpa_mean reads the raw frames
   L.conv = conv ? 1 : 0;
   for (int s = 0; s < rig.n; s++) {
     const hdr_sensor_desc &d = rig.s[s].d;
@@ -526,6 +619,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     invert_affine(d.affine, tinv);
     compose_affine(tinv, p->out_affine, K.G);
     for (int i = 0; i < 4; i++) K.Gf[i] = (float)K.G[i < 2 ? i : i + 1];
+    K.Gt[0] = (float)K.G[2];
+    K.Gt[1] = (float)K.G[5];
     K.A[0] = (float)d.affine[0];
     K.A[1] = (float)d.affine[1];
     K.A[2] = (float)d.affine[3];
@@ -547,6 +642,12 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     K.prnu = rig.s[s].prnu;
     K.rvar = rig.s[s].rvar;
     K.satf = rig.s[s].satf;
+    K.raw = raw[s];
+    K.raw_pitch = d.pitch_elems;
+    if (mean.size >= 0) {
+      mean_box(mean, K.G, hxu, hyu, &K.box_w, &K.box_h, &K.ext_x, &K.ext_y);
+      continue;
+    }
     // staging box: the tile's pixel points span |G_lin| * (TILE-1) in sensor space; add the
     // largest window's half extent plus margin on both sides, the floor of the origin and
     // the alignment of the origin (x to 8 elements = 16 bytes, y to 2)
@@ -562,8 +663,6 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
       return fail(HDR_E_UNSUPPORTED, "sensor %d staging box %dx%d exceeds 256 (window or output scale too large)", s, bw, bh);
     K.box_w = bw;
     K.box_h = bh;
-    K.raw = raw[s];
-    K.raw_pitch = d.pitch_elems;
     if (conv) {
       // the converted frame's colour-phase planes, copied straight into the staged planes
       K.conv_pitch = conv_pitch_of(d.width);
@@ -626,6 +725,14 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
       }
     }
   }
+  if (mean.size >= 0) {
+    L.mode = LPA_MEAN;
+    L.mean_p = mean.p;
+    L.mean_size = mean.size;
+    L.mean_axis = mean.axis ? 1 : 0;
+    L.stages = 1;
+    return HDR_OK;
+  }
   L.tx_bytes = tx;
   // a usable fit's equilibrated pivots lie in (min_pivot, 1]: when min_pivot * cond_fallback >= 2
   // their spread never exceeds cond_fallback and the FP64 re-solve cannot trigger
@@ -670,7 +777,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
 
 hdr_status plan(hdr_ctx *ctx, const Rig &rig, const hdr_params *p, const uint16_t *const *raw, LpaLaunch &L,
                 double reach = 1.0, bool levels = false, int stages = 1, float2 *conv = nullptr) {
-  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels}, rig, p, raw, L,
+  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels, !levels}, rig, p, raw, L,
                   LPA_FRAME_TILE_H, reach, stages, conv);
 }
 
@@ -691,9 +798,9 @@ hdr_status conv_capacity(hdr_ctx *ctx, size_t need) {
 
 // The conversion buffer of a single-frame call for this rig, or nullptr when the frame is
 // converted in the kernel (lpa_conv_eligible).
-hdr_status conv_buffer(hdr_ctx *ctx, const Rig &rig, const hdr_params *p, float2 **buf) {
+hdr_status conv_buffer(hdr_ctx *ctx, const Rig &rig, const hdr_params *p, bool levels, float2 **buf) {
   *buf = nullptr;
-  if (!lpa_conv_eligible(p, false)) return HDR_OK;
+  if (!conv_eligible(rig, p, false, !levels)) return HDR_OK;
   hdr_status st = conv_capacity(ctx, conv_elems(rig));
   if (st) return st;
   *buf = ctx->conv_buf;
@@ -756,6 +863,11 @@ hdr_status cached_plan(hdr_ctx *ctx, int32_t rig_id, const hdr_params *p, const 
 hdr_status launch(const LpaLaunch &L, int accum, bool diag, cudaStream_t st) {
   if (L.tiles_x == 0 || L.tiles_y == 0) return HDR_OK;
   cudaError_t e;
+  if (L.mode == LPA_MEAN) {
+    e = lpa_launch_mean(L, st);
+    if (e != cudaSuccess) return fail(HDR_E_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+    return HDR_OK;
+  }
   switch (L.order) {
     case 0: e = lpa_launch_order0(L, accum != 0, diag, st); break;
     case 1: e = lpa_launch_order1(L, accum != 0, diag, st); break;
@@ -785,7 +897,7 @@ hdr_status reconstruct_impl(hdr_ctx *ctx, int32_t rig_id, const hdr_params *para
     return fail(HDR_E_UNSUPPORTED, "the level maps are computed with the inverse-variance weight (weight_mode 0)");
   LpaLaunch L;
   float2 *conv = nullptr;
-  st = conv_buffer(ctx, ctx->rigs[rig_id], params, &conv);
+  st = conv_buffer(ctx, ctx->rigs[rig_id], params, levels_dev != nullptr, &conv);
   if (st) return st;
   // the diagnostic (level maps) kernel searches every window
   st = cached_plan(ctx, rig_id, params, raw_dev, L, levels_dev != nullptr, levels_dev ? 1 : LPA_FRAME_STAGES, conv);
@@ -1041,7 +1153,7 @@ hdr_status hdr_reconstruct_host(hdr_ctx *ctx, int32_t rig_id, const hdr_params *
   const size_t esize = params->out_dtype ? 2 : 4;
   LpaLaunch L;
   float2 *conv = nullptr;
-  st = conv_buffer(ctx, rig, params, &conv);
+  st = conv_buffer(ctx, rig, params, false, &conv);
   if (st) return st;
   st = cached_plan(ctx, rig_id, params, raw_dev, L, false, LPA_FRAME_STAGES, conv);
   if (st) return st;
@@ -1275,7 +1387,7 @@ hdr_status batch_plan(hdr_ctx *ctx, int n, const hdr_frame *frames, const int2 *
   for (int f = 0; f < n; f++) {
     const hdr_frame &F = frames[f];
     // no tables: the persistent kernels search every window
-    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, false, false}, ctx->rigs[F.rig_id],
+    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, false, false, false}, ctx->rigs[F.rig_id],
                              F.params, F.raw_dev, plans[f], cfg.tile_h);
     if (st) return fail(st, "frame %d: %s", f, g_err.c_str());
     if (plans[f].mode != LPA_SEARCHED && plans[f].mode != LPA_SEARCHED_F32)
@@ -1343,13 +1455,13 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
     } else {
       size_t total = 0;
       for (int f = 0; f < n; f++)
-        if (lpa_conv_eligible(frames[f].params, frames[f].calpa != nullptr)) total += conv_elems(ctx->rigs[frames[f].rig_id]);
+        if (conv_eligible(ctx->rigs[frames[f].rig_id], frames[f].params, frames[f].calpa != nullptr)) total += conv_elems(ctx->rigs[frames[f].rig_id]);
       if (total) {
         hdr_status st = conv_capacity(ctx, total);
         if (st) return st;
         float2 *p = ctx->conv_buf;
         for (int f = 0; f < n; f++)
-          if (lpa_conv_eligible(frames[f].params, frames[f].calpa != nullptr)) {
+          if (conv_eligible(ctx->rigs[frames[f].rig_id], frames[f].params, frames[f].calpa != nullptr)) {
             cv[f] = p;
             p += conv_elems(ctx->rigs[frames[f].rig_id]);
           }
@@ -1395,7 +1507,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       pp = &sp;
     }
     const int px = (cfg.px_per_thread == 2 && !F.calpa) ? 2 : 1;
-    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !F.calpa, px == 1}, ctx->rigs[F.rig_id],
+    hdr_status st = plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !F.calpa, px == 1, !F.calpa}, ctx->rigs[F.rig_id],
                              pp, F.raw_dev, plans[f], F.calpa ? 16 : cfg.tile_h,
                              F.calpa ? lpa_calpa_reach(F.calpa) : 1.0, (F.calpa || px != 1) ? 1 : cfg.stages,
                              F.calpa ? nullptr : cv[f]);
@@ -1404,7 +1516,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       plans[f].mode = lpa_mode_f32(plans[f].mode) ? LPA_STEERED_F32 : LPA_STEERED;
       plans[f].aux = aux[f] + npx * 2;  // the steering matrices
     }
-    plans[f].px = px;
+    plans[f].px = plans[f].mode == LPA_MEAN ? 1 : px;
     plans[f].out = F.out_dev;
     plans[f].choice = F.choice_dev;
     plans[f].levels = nullptr;
@@ -1413,6 +1525,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       return fail(HDR_E_INVALID, "frame %d: tile range [%d, %d) outside [0, %d)", f, ranges[f].x, ranges[f].y, nt);
     plans[f].tile0 = ranges ? ranges[f].x : 0;
     grid[f] = ranges ? ranges[f].y - ranges[f].x : nt;
+    if (plans[f].mode == LPA_MEAN) plans[f].tile_count = grid[f];
   }
   std::vector<int> order;
   for (int f = 0; f < n; f++)
@@ -1451,18 +1564,20 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       kp.push_back(c);
       dep.push_back(-1);
     }
-    const void *fn = lpa_kernel(L.order, comp, false, L.mode, L.tile_h, L.px, L.stages);
+    const bool mean = L.mode == LPA_MEAN;
+    const void *fn = mean ? lpa_mean_kernel(L) : lpa_kernel(L.order, comp, false, L.mode, L.tile_h, L.px, L.stages);
     if (!fn)
       return fail(HDR_E_INTERNAL, "no kernel for order %d, mode %d, tile height %d, %d pixels per thread, %d stages",
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, L.px, L.stages + 4 * (d >= 0 ? 1 : 0)});
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis : L.px,
+                   L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};
     r.func = const_cast<void *>(fn);
-    r.gridDim = dim3((unsigned)lpa_grid_ctas(grid[f], L.stages));
-    r.blockDim = dim3((unsigned)(LPA_TILE * L.tile_h / L.px));
+    r.gridDim = dim3(mean ? lpa_mean_grid(L) : (unsigned)lpa_grid_ctas(grid[f], L.stages));
+    r.blockDim = dim3(mean ? (unsigned)LPA_MEAN_THREADS : (unsigned)(LPA_TILE * L.tile_h / L.px));
     r.sharedMemBytes = L.smem_bytes;
     r.kernelParams = args.back().data();
     kp.push_back(r);
@@ -1673,11 +1788,12 @@ hdr_status lpa_launch_mode(hdr_ctx *ctx, int32_t rig_id, const hdr_params *param
   p.tab_weights = 0;  // the window is searched: offsets or weights differ per pixel
   float2 *conv = nullptr;
   if (ahead) {
-    s = conv_buffer(ctx, ctx->rigs[rig_id], &p, &conv);
+    s = conv_buffer(ctx, ctx->rigs[rig_id], &p, true, &conv);
     if (s) return s;
   }
   LpaLaunch L;
-  s = plan(ctx, ctx->rigs[rig_id], &p, raw_dev, L, reach, false, 1, conv);
+  // (planned as for the level maps: the kernel of `mode` is the general one, with its variance sums)
+  s = plan(ctx, ctx->rigs[rig_id], &p, raw_dev, L, reach, true, 1, conv);
   if (s) return s;
   if (L.conv) {  // the frame converted once, then the pass
     s = convert_rows(ctx, L, all_rows(L), true, st);

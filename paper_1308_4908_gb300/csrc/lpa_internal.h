@@ -21,7 +21,7 @@ hdr_status lpa_convert_frame(hdr_ctx *ctx, int32_t rig_id, const hdr_params *par
                              float2 *conv, cudaStream_t st);
 // Whether a frame with these parameters is converted in a pass of its own before its
 // reconstruction, and the float2 elements of its converted planes for a rig.
-bool lpa_conv_eligible(const hdr_params *p, bool adaptive);
+bool lpa_conv_eligible(const hdr_ctx *ctx, int rig_id, const hdr_params *p, bool adaptive);
 size_t lpa_conv_elems(const hdr_ctx *ctx, int rig_id);
 // Validate adaptive-reconstruction parameters.
 hdr_status lpa_check_calpa(const hdr_calpa_params *c);

@@ -9,6 +9,8 @@
 #define LPA_TILE 16         // output tile width in pixels; the height TH is 8 or 16 (one thread per pixel)
 #define LPA_ANCHOR 8        // edge of the output blocks whose sensor positions are anchored in FP64
 #define LPA_MARGIN 4        // staging margin in sensor px around every window box
+#define LPA_MEAN_THREADS 512
+#define LPA_MEAN_TILE_W 64
 #define LPA_STAGED_TILES 4  // tiles per CTA of the single-frame kernel with two staging buffers
 
 // Device status word bits (read and cleared by hdr_check).
@@ -19,6 +21,7 @@ struct alignas(64) LpaSensorK {
   CUtensorMap tmap;         // 2-D tiled map of the raw frame (uint16, dims width x height)
   double G[6];              // output px -> sensor px: T_s^{-1} composed with the output mapping
   float Gf[4];              // linear part of G in FP32 (steps between neighbouring output pixels)
+  float Gt[2];              // translation of G in FP32
   float A[4];               // linear part of T_s (sensor px -> reference px), row-major
   float hx_unit, hy_unit;   // sensor-space half extent of a reference disc of radius 1
   float inv_gtn;            // 1 / (g t n)
@@ -96,7 +99,20 @@ struct LpaLaunch {
   // LPA_LITERAL: the searched window with the noise weight printed in Eq. 6 (K / s, not K / s2).
   int mode;
   float *aux;
+  // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, whether every sensor's axes are
+  // parallel to the output's, bytes of one buffer of colour-phase planes (two from offset 0) and
+  // the offset of the position tables
+  int mean_p, mean_size, mean_axis;
+  uint32_t mean_plane, mean_tab;
 };
+
+// Output rows [first, end) of a launch's unit tiles (whole tile rows).
+__host__ __device__ inline int lpa_first_row(const LpaLaunch &L) { return L.tile0 / L.tiles_x * L.tile_h; }
+__host__ __device__ inline int lpa_end_row(const LpaLaunch &L) {
+  const int count = L.tile_count > 0 ? L.tile_count : L.tiles_x * L.tiles_y - L.tile0;
+  const int end = ((L.tile0 + count - 1) / L.tiles_x + 1) * L.tile_h;
+  return end < L.out_h ? end : L.out_h;
+}
 
 // LPA_SEARCHED_F32, LPA_STEERED_F32, LPA_TABULATED_F32: the searched, steered or tabulated window
 // with every fit solved in FP32 only, for parameters under which the FP64 re-solve can never
@@ -107,6 +123,8 @@ struct LpaLaunch {
 // interval rule has nothing to compare, so Var C_0 is not used. The values are those of
 // LPA_SEARCHED and LPA_TABULATED bit for bit. Built for one pixel per thread and one staging buffer
 // (other launches, the level maps and the persistent kernels keep the variance sums).
+// LPA_MEAN: order 0 with one small window, a kernel of its own (lpa_mean.cu) whose tiles are 64 pixels wide;
+// tile ranges are given in the same unit tiles as the other modes' and cover whole tile rows.
 enum {
   LPA_SEARCHED = 0,
   LPA_TABULATED = 1,
@@ -119,7 +137,8 @@ enum {
   LPA_ONE = 8,
   LPA_ONE_F32 = 9,
   LPA_TABULATED_ONE = 10,
-  LPA_TABULATED_ONE_F32 = 11
+  LPA_TABULATED_ONE_F32 = 11,
+  LPA_MEAN = 12
 };
 __host__ __device__ constexpr bool lpa_mode_steered(int mode) { return mode == LPA_STEERED || mode == LPA_STEERED_F32; }
 __host__ __device__ constexpr bool lpa_mode_one(int mode) {

@@ -1,0 +1,327 @@
+// Order 0 with one window scale: the local constant fit of Eq. 7, sum K f / s2 over sum K / s2.
+//
+// With one sum and one weight per sample the general kernel spends its instructions on finding the
+// window (its bounding box, warp-wide maxima, rows, a test per cell): 2420 warp instructions per 32
+// pixels of a two-sensor frame enlarged twofold, 300 per walk of a 9-cell window. Here the candidate
+// cells of a window are a fixed N x N block of its colour phase (N = cells that a row or column of
+// the window can hold), so the loops unroll, and a cell outside the window needs no test: its value
+// exp(-r^2 / 2 sigma^2) - exp(-k^2 / 2) (Eq. 8) is not positive there and is cut at 0.
+//
+// A CTA of 512 threads reconstructs 64 x 8 P pixels, P rows per thread; lanes are consecutive
+// pixels of a row, so stores coalesce and neighbours read the same cells. Sensors come one after the
+// other: their raw footprint is read straight from global memory (16-byte loads, the next sensor's
+// in flight during this one's sums), converted once per sample (Eqs. 18 and 20) into colour-phase
+// planes of (1 / s2, f / s2) in shared memory, double-buffered: one barrier per sensor. Each cell is
+// then one shared load and one paired FMA into (sum K / s2, sum K f / s2). No conversion pass goes
+// ahead of the kernel: with 64 x 32 tiles a sample is converted about 1.5 times, and the pass cost
+// 47 us of 517 on four 2336 x 1752 sensors. Measured against the general kernel with that pass: 2 x 2048^2 ->
+// 4096^2 FP16 1226 -> 303 us, the four sensors (tabulated windows before) 517 -> 172 us, 64^2 14.4 -> 10.3 us a call;
+// 1024 x 900, three rotated sensors 147 -> 78 us.
+//
+// AXIS: every sensor's axes are parallel to the output's, so the Gaussian factors into a column and
+// a row factor, tabulated per tile: a cell is one FMA, one maximum, the load and the paired FMA.
+// Otherwise each cell forms its offset and one exponential.
+#include <cuda_fp16.h>
+
+#include <cmath>
+#include <type_traits>
+
+#include "lpa_dispatch.h"
+#include "lpa_launch.h"
+#include "lpa_convert.cuh"
+#include "lpa_ptx.cuh"
+
+namespace lpa {
+namespace {
+
+constexpr int kThreads = LPA_MEAN_THREADS;
+constexpr int kBW = LPA_MEAN_TILE_W;
+
+// First candidate cell of a window along one axis of one colour phase: the position is cell `l` (from
+// the box origin, even) plus fraction f; the window reaches h (m = floor(h / 2)). Returns the
+// lattice index (cell o + 2 i) and its offset from the position.
+__device__ __forceinline__ int first_cell(int l, float f, int o, float h, float m, float &delta) {
+  const int e = l - o;
+  const float r = (e & 1) ? f + 1.f : f;             // position from the even lattice cell below, in [0, 2)
+  const float n = (h - r) * 0.5f < m ? m - 1.f : m;  // floor((h - r) / 2)
+  delta = -2.f * n - r;
+  return (e >> 1) - (int)n;
+}
+
+struct Window {
+  float h, m;  // reach in sensor px and floor(reach / 2)
+};
+
+template <int NR, int NG>
+struct Layout {
+  static constexpr int kE = 2 * (NR + NG);       // factors: RB phase 0, RB phase 1, G phase 0, G phase 1
+  static constexpr int kWords = 4 + kE;          // four first cells, then the factors
+  static constexpr int kRow = (kWords + 3) / 4 * 4;
+};
+
+// Raw samples of group g (eight columns of a row) of the box at (x0, y0), or zeros off the frame.
+__device__ __forceinline__ uint4 load_group(const LpaSensorK &S, int x0, int y0, int g, int groups_x) {
+  const int row = g / groups_x, X = x0 + 8 * (g - row * groups_x), Y = y0 + row;
+  if (X < 0 || X >= S.width || Y < 0 || Y >= S.height) return make_uint4(0, 0, 0, 0);
+  return __ldg(reinterpret_cast<const uint4 *>(S.raw + (size_t)Y * S.raw_pitch + X));
+}
+
+__device__ __forceinline__ void store_group(const LpaSensorK &S, int x0, int y0, int g, int groups_x, uint4 q, float2 *planes) {
+  const int row = g / groups_x, col = g - row * groups_x, X = x0 + 8 * col, Y = y0 + row;
+  const int PW = S.box_w >> 1, PP = PW * (S.box_h >> 1);
+  const bool scalar = !S.bias && !S.rvar && !S.satf && !S.prnu;
+  const bool in = X >= 0 && Y >= 0 && Y < S.height;
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+  float4 *even = reinterpret_cast<float4 *>(planes + 2 * (row & 1) * PP + (row >> 1) * PW + 4 * col);
+  float4 *odd = reinterpret_cast<float4 *>(planes + (2 * (row & 1) + 1) * PP + (row >> 1) * PW + 4 * col);
+  float2 v[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    const uint32_t y = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
+    v[k] = make_float2(0.f, 0.f);
+    if (in && X + k < S.width) {
+      const float2 fv = convert_sample<false>(S, scalar, X + k, Y, (float)y);  // (f, 1 / s2)
+      v[k] = make_float2(fv.y, fv.y * fv.x);
+    }
+  }
+  even[0] = make_float4(v[0].x, v[0].y, v[2].x, v[2].y);
+  even[1] = make_float4(v[4].x, v[4].y, v[6].x, v[6].y);
+  odd[0] = make_float4(v[1].x, v[1].y, v[3].x, v[3].y);
+  odd[1] = make_float4(v[5].x, v[5].y, v[7].x, v[7].y);
+}
+
+// Box origin of a tile in sensor s: x on a multiple of 8 (16-byte loads), y even. FP32 is enough
+// (the box has a margin of a pixel), and every thread forms the same value.
+__device__ __forceinline__ int2 box_origin(const LpaSensorK &S, int u0, int v0, int bh) {
+  float x = S.Gf[0] * (float)(S.Gf[0] < 0.f ? u0 + kBW - 1 : u0) + S.Gf[1] * (float)(S.Gf[1] < 0.f ? v0 + bh - 1 : v0);
+  float y = S.Gf[2] * (float)(S.Gf[2] < 0.f ? u0 + kBW - 1 : u0) + S.Gf[3] * (float)(S.Gf[3] < 0.f ? v0 + bh - 1 : v0);
+  x = fminf(fmaxf(x + S.Gt[0] - S.ext_x, -LPA_FAR_F), LPA_FAR_F);
+  y = fminf(fmaxf(y + S.Gt[1] - S.ext_y, -LPA_FAR_F), LPA_FAR_F);
+  return make_int2((int)floorf(x) & ~7, (int)floorf(y) & ~1);
+}
+
+template <int NR, int NG, bool AXIS, int P>
+__global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ LpaLaunch L) {
+  using T = Layout<NR, NG>;
+  constexpr int BH = 8 * P;
+  if (*reinterpret_cast<volatile unsigned int *>(L.status) & LPA_ERR_TIMEOUT) return;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int tid = threadIdx.x, S = L.n_sensors;
+  const int nbx = (L.out_w + kBW - 1) / kBW;
+  const int y_first = lpa_first_row(L), y_end = lpa_end_row(L);
+  const int u0 = (int)(blockIdx.x % nbx) * kBW, v0 = y_first + (int)(blockIdx.x / nbx) * BH;
+  const float log2e = 1.4426950408889634f;
+  const float sg[2] = {L.sigma[0], L.sigma[0] * L.green_ratio};
+
+  // positions of the tile's columns and rows (AXIS) or of its 8 x 8 blocks' corners, in FP64
+  float *xt = reinterpret_cast<float *>(smem + L.mean_tab);
+  float *yt = xt + S * T::kWords * kBW;
+  int4 *anchor = reinterpret_cast<int4 *>(smem + L.mean_tab);
+  if constexpr (AXIS) {
+    for (int k = tid; k < S * (kBW + BH); k += kThreads) {
+      const int s = k / (kBW + BH), e = k - s * (kBW + BH);
+      const bool col = e < kBW;
+      const LpaSensorK &Sk = L.s[s];
+      const int2 o = box_origin(Sk, u0, v0, BH);
+      const double q = fmin(fmax(col ? Sk.G[0] * (u0 + e) + Sk.G[2] : Sk.G[4] * (v0 + e - kBW) + Sk.G[5], -LPA_FAR), LPA_FAR);
+      const double fl = floor(q);
+      const int l = (int)fl - (col ? o.x : o.y);
+      const float f = (float)(q - fl), a = col ? Sk.A[0] : Sk.A[3];
+      const int cells = (col ? Sk.box_w : Sk.box_h) >> 1, step = col ? 1 : Sk.box_w >> 1;
+      float *t = col ? xt + s * T::kWords * kBW + e : yt + (s * BH + e - kBW) * T::kRow;
+      const int stride = col ? kBW : 1;
+      bool ok = true;
+#pragma unroll
+      for (int g = 0; g < 2; g++) {
+        const int N = g ? NG : NR;
+        const float h = L.trunc_k * sg[g] * (col ? Sk.hx_unit : Sk.hy_unit) + 1e-3f, m = floorf(0.5f * h);
+        const float c = -log2e / (2.f * sg[g] * sg[g]) * a * a;
+#pragma unroll
+        for (int ph = 0; ph < 2; ph++) {
+          float d;
+          const int i = first_cell(l, f, ph, h, m, d), at = min(max(i, 0), cells - N);
+          ok = ok && i == at;
+          t[(2 * g + ph) * stride] = __int_as_float(at * step);
+          float *w = t + (4 + 2 * NR * g + N * ph) * stride;
+#pragma unroll
+          for (int j = 0; j < N; j++) {
+            const float dj = d + 2.f * (float)j;
+            w[j * stride] = ex2_approx(c * dj * dj);
+          }
+        }
+      }
+      if (!ok && (col ? u0 + e < L.out_w : v0 + e - kBW < y_end) && fabs(q) < 1e6) atomicOr(L.status, LPA_ERR_BOUNDS);
+    }
+  } else {
+    constexpr int NA = 8 * P;  // 8 x 8 blocks of the tile
+    for (int k = tid; k < S * NA; k += kThreads) {
+      const int s = k / NA, b = k - s * NA;
+      const LpaSensorK &Sk = L.s[s];
+      const int2 o = box_origin(Sk, u0, v0, BH);
+      const double uu = u0 + 8 * (b & 7), vv = v0 + 8 * (b >> 3);
+      const double qx = fmin(fmax(Sk.G[0] * uu + Sk.G[1] * vv + Sk.G[2], -LPA_FAR), LPA_FAR);
+      const double qy = fmin(fmax(Sk.G[3] * uu + Sk.G[4] * vv + Sk.G[5], -LPA_FAR), LPA_FAR);
+      const double fx = floor(qx), fy = floor(qy);
+      anchor[k] = make_int4((int)fx - o.x, (int)fy - o.y, __float_as_int((float)(qx - fx)), __float_as_int((float)(qy - fy)));
+    }
+  }
+
+  const int col = (tid & 31) + 32 * ((tid >> 5) & 1), row0 = (tid >> 6) * P;
+  const int u = u0 + col;
+  float2 acc[P][3];  // per row and channel: (sum K / s2, sum K f / s2)
+#pragma unroll
+  for (int k = 0; k < P; k++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) acc[k][c] = make_float2(0.f, 0.f);
+
+  int2 o = box_origin(L.s[0], u0, v0, BH);
+  uint4 q = make_uint4(0, 0, 0, 0);
+  if (tid < (L.s[0].box_w >> 3) * L.s[0].box_h) q = load_group(L.s[0], o.x, o.y, tid, L.s[0].box_w >> 3);
+#pragma unroll 1
+  for (int s = 0; s < S; s++) {
+    const LpaSensorK &Sk = L.s[s];
+    float2 *planes = reinterpret_cast<float2 *>(smem + (s & 1) * L.mean_plane);
+    const int gx = Sk.box_w >> 3, n = gx * Sk.box_h;
+    if (tid < n) store_group(Sk, o.x, o.y, tid, gx, q, planes);
+    for (int g = tid + kThreads; g < n; g += kThreads)
+      store_group(Sk, o.x, o.y, g, gx, load_group(Sk, o.x, o.y, g, gx), planes);
+    if (s + 1 < S) {  // the next sensor's samples, in flight during this one's sums
+      const LpaSensorK &Sn = L.s[s + 1];
+      o = box_origin(Sn, u0, v0, BH);
+      if (tid < (Sn.box_w >> 3) * Sn.box_h) q = load_group(Sn, o.x, o.y, tid, Sn.box_w >> 3);
+    }
+    __syncthreads();  // the planes are whole; the other buffer's readers have left it
+    const int PW = Sk.box_w >> 1, PP = PW * (Sk.box_h >> 1);
+    if constexpr (AXIS) {
+      const float *tx = xt + s * T::kWords * kBW + col;
+      int xi[4];
+      float ex[T::kE];
+#pragma unroll
+      for (int k = 0; k < 4; k++) xi[k] = __float_as_int(tx[k * kBW]);
+#pragma unroll
+      for (int k = 0; k < T::kE; k++) ex[k] = tx[(4 + k) * kBW];
+#pragma unroll
+      for (int k = 0; k < P; k++) {
+        float y[T::kRow];  // the row's cells and factors: the same for every lane
+        const float4 *ty = reinterpret_cast<const float4 *>(yt + (s * BH + row0 + k) * T::kRow);
+#pragma unroll
+        for (int j = 0; j < T::kRow / 4; j++) {
+          const float4 t = ty[j];
+          y[4 * j] = t.x, y[4 * j + 1] = t.y, y[4 * j + 2] = t.z, y[4 * j + 3] = t.w;
+        }
+        auto phase = [&](auto N_, float2 &a, int ox, int oy, int g) {
+          constexpr int N = decltype(N_)::value;
+          const float2 *pl = planes + (ox + 2 * oy) * PP + __float_as_int(y[2 * g + oy]) + xi[2 * g + ox];
+#pragma unroll
+          for (int j = 0; j < N; j++) {
+            const float ey = y[4 + 2 * NR * g + N * oy + j];
+#pragma unroll
+            for (int i = 0; i < N; i++) {
+              const float K = fmaxf(fmaf(ex[2 * NR * g + N * ox + i], ey, -L.taper), 0.f);
+              a = __ffma2_rn(make_float2(K, K), pl[j * PW + i], a);
+            }
+          }
+        };
+        phase(std::integral_constant<int, NR>(), acc[k][0], 0, 0, 0);
+        phase(std::integral_constant<int, NG>(), acc[k][1], 1, 0, 1);
+        phase(std::integral_constant<int, NG>(), acc[k][1], 0, 1, 1);
+        phase(std::integral_constant<int, NR>(), acc[k][2], 1, 1, 0);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < P; k++) {
+        const int row = row0 + k;
+        const int4 an = anchor[s * 8 * P + (row >> 3) * 8 + (col >> 3)];
+        const float du = (float)(col & 7), dv = (float)(row & 7);
+        const float px = __int_as_float(an.z) + du * Sk.Gf[0] + dv * Sk.Gf[1];
+        const float py = __int_as_float(an.w) + du * Sk.Gf[2] + dv * Sk.Gf[3];
+        const float flx = floorf(px), fly = floorf(py);
+        const int lx = an.x + (int)flx, ly = an.y + (int)fly;
+        const float fx = px - flx, fy = py - fly;
+        bool ok = true;
+        auto phase = [&](auto N_, float2 &a, int ox, int oy, int g) {
+          constexpr int N = decltype(N_)::value;
+          const float hx = L.trunc_k * sg[g] * Sk.hx_unit + 1e-3f, hy = L.trunc_k * sg[g] * Sk.hy_unit + 1e-3f;
+          const float unit = sqrtf(log2e * 0.5f) / sg[g];  // K = 2^-(unit |d|)^2 - taper
+          float dx, dy;
+          const int i0 = first_cell(lx, fx, ox, hx, floorf(0.5f * hx), dx), i = min(max(i0, 0), PW - N);
+          const int j0 = first_cell(ly, fy, oy, hy, floorf(0.5f * hy), dy), j = min(max(j0, 0), (Sk.box_h >> 1) - N);
+          ok = ok && i == i0 && j == j0;
+          const float2 *pl = planes + (ox + 2 * oy) * PP + j * PW + i;
+          const float2 CX = make_float2(Sk.A[0] * unit, Sk.A[2] * unit), CY = make_float2(Sk.A[1] * unit, Sk.A[3] * unit);
+          const float2 DX = make_float2(dx, dx), DY = make_float2(dy, dy);
+          const float2 D0 = __ffma2_rn(CY, DY, __fmul2_rn(CX, DX));
+          const float2 SX = make_float2(2.f * CX.x, 2.f * CX.y), SY = make_float2(2.f * CY.x, 2.f * CY.y);
+#pragma unroll
+          for (int r = 0; r < N; r++) {
+            float2 D = __ffma2_rn(make_float2((float)r, (float)r), SY, D0);
+#pragma unroll
+            for (int c = 0; c < N; c++, D = __fadd2_rn(D, SX)) {
+              const float K = fmaxf(ex2_approx(-fmaf(D.x, D.x, D.y * D.y)) - L.taper, 0.f);
+              a = __ffma2_rn(make_float2(K, K), pl[r * PW + c], a);
+            }
+          }
+        };
+        phase(std::integral_constant<int, NR>(), acc[k][0], 0, 0, 0);
+        phase(std::integral_constant<int, NG>(), acc[k][1], 1, 0, 1);
+        phase(std::integral_constant<int, NG>(), acc[k][1], 0, 1, 1);
+        phase(std::integral_constant<int, NR>(), acc[k][2], 1, 1, 0);
+        if (!ok && u < L.out_w && v0 + row < y_end && abs(lx) < (1 << 20) && abs(ly) < (1 << 20))
+          atomicOr(L.status, LPA_ERR_BOUNDS);
+      }
+    }
+  }
+  if (u >= L.out_w) return;
+  const size_t plane = (size_t)L.out_w * L.out_h;
+#pragma unroll
+  for (int k = 0; k < P; k++) {
+    const int v = v0 + row0 + k;
+    if (v >= y_end) return;
+    const size_t at = (size_t)v * L.out_w + u;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      const bool has = acc[k][c].x > 0.f;
+      const float val = has ? __fdividef(acc[k][c].y, acc[k][c].x) : __int_as_float(0x7fffffff);
+      if (L.out_half) reinterpret_cast<__half *>(L.out)[c * plane + at] = __float2half_rn(val);
+      else reinterpret_cast<float *>(L.out)[c * plane + at] = val;
+      if (L.choice) L.choice[c * plane + at] = has ? 0 : 255;
+    }
+  }
+}
+
+template <int NR, int NG, bool AXIS>
+const void *pick(int p) {
+  return p == 1   ? (const void *)lpa_mean<NR, NG, AXIS, 1>
+         : p == 2 ? (const void *)lpa_mean<NR, NG, AXIS, 2>
+                  : (const void *)lpa_mean<NR, NG, AXIS, 4>;
+}
+
+}  // namespace
+}  // namespace lpa
+
+int lpa_mean_size(double reach_rb, double reach_g) {
+  const double rb = std::floor(reach_rb) + 1, g = std::floor(reach_g) + 1;
+  return rb <= 3 && g <= 2 ? 0 : rb <= 4 && g <= 3 ? 1 : -1;
+}
+int lpa_mean_cells(int size, bool green) { return size == 0 ? (green ? 2 : 3) : (green ? 3 : 4); }
+uint32_t lpa_mean_tab_bytes(int size, bool axis, int p, int n_sensors) {
+  if (!axis) return (uint32_t)(n_sensors * 8 * p * 16);
+  const int words = size == 0 ? lpa::Layout<3, 2>::kWords : lpa::Layout<4, 3>::kWords;
+  const int row = size == 0 ? lpa::Layout<3, 2>::kRow : lpa::Layout<4, 3>::kRow;
+  return (uint32_t)(n_sensors * 4 * (words * lpa::kBW + row * 8 * p));
+}
+const void *lpa_mean_kernel(const LpaLaunch &L) {
+  if (L.mean_size == 0) return L.mean_axis ? lpa::pick<3, 2, true>(L.mean_p) : lpa::pick<3, 2, false>(L.mean_p);
+  return L.mean_axis ? lpa::pick<4, 3, true>(L.mean_p) : lpa::pick<4, 3, false>(L.mean_p);
+}
+unsigned lpa_mean_grid(const LpaLaunch &L) {
+  const long rows = lpa_end_row(L) - lpa_first_row(L), bh = 8 * L.mean_p;
+  return (unsigned)((L.out_w + lpa::kBW - 1) / lpa::kBW * ((rows + bh - 1) / bh));
+}
+cudaError_t lpa_launch_mean(const LpaLaunch &L, cudaStream_t st) {
+  const void *fn = lpa_mean_kernel(L);
+  cudaError_t e = lpa_opt_in(fn);
+  if (e != cudaSuccess) return e;
+  void *args[] = {const_cast<LpaLaunch *>(&L)};
+  return cudaLaunchKernel(fn, dim3(lpa_mean_grid(L)), dim3(LPA_MEAN_THREADS), args, L.smem_bytes, st);
+}

@@ -535,7 +535,7 @@ hdr_status hdr_submit(hdr_server *srv, const hdr_request *req, uint64_t *ticket)
   j.choice_bytes = req->choice_host ? px : 0;
   j.scratch_bytes = req->adaptive ? px / 3 * 5 * sizeof(float) : 0;  // 5 floats per output pixel
   // the frame's converted planes, where its steps copy converted footprints
-  const bool conv = lpa_conv_eligible(&req->params, req->adaptive != 0) && srv->cfg.batch.stages != 2 &&
+  const bool conv = lpa_conv_eligible(srv->ctx, req->rig_id, &req->params, req->adaptive != 0) && srv->cfg.batch.stages != 2 &&
                     srv->cfg.batch.form == 0;
   j.conv_bytes = conv ? lpa_conv_elems(srv->ctx, req->rig_id) * sizeof(float2) : 0;
   bytes += align256(j.out_bytes) + align256(j.choice_bytes) + align256(j.scratch_bytes) + align256(j.conv_bytes);

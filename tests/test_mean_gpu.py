@@ -1,0 +1,160 @@
+"""Order 0 with one window scale (lpa_mean): every pixel against the oracle, and the same bits from
+every entry point.
+
+Covered where its tiles and windows can go wrong: outputs around the 64-pixel tile width and the 8
+P rows of a tile, axis-parallel and rotated rigs, 1x, enlarged, reduced and mirrored outputs, both
+candidate-cell sizes and the windows between them, odd sensors with calibration frames, outputs past the
+sensors, one and eight sensors, and the larger tiles of big frames on sampled pixels. Tolerance: the parity
+rule of tests/parity.py, unchanged.
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_1308_4908_gb300 import synth
+from tests import parity
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1308_4908_gb300 import hdr
+    c = hdr.Context(0)
+    yield c
+    c.close()
+
+
+def _frame(w, h, rot, n=2, sigma=0.7, seed=1500, calibrated=False, **over):
+    p = synth.Params(order=0, sigmas=(sigma,), out_w=w, out_h=h)
+    fr = synth._build_frame(seed + n, n, w, h, [2.0 ** (-2 * k) for k in range(n)], 1.3, rot, 0.0, p, "mean")
+    if calibrated:
+        r = np.random.default_rng(seed)
+        s = fr.sensors[0]
+        s.bias_frame = (s.black + r.uniform(-2, 2, (h, w))).astype(np.float32)
+        s.prnu_frame = r.uniform(0.95, 1.05, (h, w)).astype(np.float32)
+        s.read_var_frame = r.uniform(6, 12, (h, w)).astype(np.float32)
+        s.sat_frame = r.integers(200, 4096, (h, w)).astype(np.uint16)
+    return dataclasses.replace(fr, params=dataclasses.replace(p, **over))
+
+
+def _run(ctx, fr, rig=0):
+    p = fr.params
+    ctx.set_rig(rig, fr.sensors)
+    raws = [torch.from_numpy(s.raw).cuda() for s in fr.sensors]
+    ch = torch.full((3, p.out_h, p.out_w), 77, dtype=torch.uint8, device="cuda")
+    dt = torch.float16 if p.out_dtype else torch.float32
+    out = torch.full((3, p.out_h, p.out_w), -7.0, dtype=dt, device="cuda")
+    ctx.reconstruct(rig, p, raws, out=out, choice=ch)
+    ctx.check()
+    return out.float().cpu().numpy(), ch.cpu().numpy(), raws
+
+
+def _against_oracle(fr, out, ch, pix, extra=0.0):
+    p = fr.params
+    o = oracle.reconstruct(fr.sensors, p, pix, levels=True)
+    parity.compare(out[:, pix[:, 1], pix[:, 0]], ch[:, pix[:, 1], pix[:, 0]], o, pix, 1, 0, p.ici_gamma, p.min_pivot,
+                   extra_rel=extra)
+
+
+def _every_pixel(p):
+    vv, uu = np.mgrid[0:p.out_h, 0:p.out_w]
+    return np.stack([uu.ravel(), vv.ravel()], axis=1)
+
+
+@pytest.mark.parametrize("rot", [0.0, 0.3, 7.0])
+@pytest.mark.parametrize("w,h", [(1, 1), (63, 7), (64, 8), (65, 9), (131, 34)])
+def test_tile_edges(ctx, w, h, rot):
+    fr = _frame(w, h, rot)
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
+@pytest.mark.parametrize("rot", [0.0, 0.4])
+@pytest.mark.parametrize("sigma,green", [(0.3, 1.0), (0.66, 0.5), (0.7, 0.70710678), (0.99, 0.7), (1.2, 0.8), (1.3, 0.6)])
+def test_window_sizes(ctx, sigma, green, rot):
+    """Windows of 1 to 4 cells a side, green as large as the others, and one just too large for the
+    kernel (1.34 x 3 px reaches five cells), with calibration frames and saturated pixels."""
+    fr = _frame(71, 45, rot, sigma=sigma, green_ratio=green, calibrated=True)
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+    fr = dataclasses.replace(fr, params=dataclasses.replace(fr.params, sigmas=(1.34,)))
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
+@pytest.mark.parametrize("rot", [0.0, 0.3])
+@pytest.mark.parametrize("ow,oh", [(142, 90), (107, 68), (50, 31), (18, 12), (9, 6)])
+def test_resampled_outputs(ctx, ow, oh, rot):
+    """Enlarged and reduced outputs; the eightfold reduction outgrows every kernel's staging and stays
+    refused."""
+    from paper_1308_4908_gb300 import hdr
+    fr = _frame(71, 45, rot, out_w=ow, out_h=oh, out_affine=synth.output_affine(71, 45, ow, oh))
+    if ow == 9:
+        with pytest.raises(hdr.HdrError) as e:
+            _run(ctx, fr)
+        assert e.value.status == hdr.HDR_E_UNSUPPORTED
+        return
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
+@pytest.mark.parametrize("affine", [[[-1.0, 0, 70.0], [0, 1.0, 0]], [[0, 1.0, 0.2], [1.0, 0, -0.3]],
+                                    [[1.0, 0, -20.0], [0, -1.0, 60.0]]])
+def test_mirrored_transposed_and_outside(ctx, affine):
+    """Output mappings that mirror, transpose, and reach past the sensors (NaN, level 255 there)."""
+    fr = _frame(71, 45, 0.0, out_affine=np.array(affine))
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+    assert np.array_equal(np.isnan(out), ch == 255)
+
+
+@pytest.mark.parametrize("n", [1, 8])
+@pytest.mark.parametrize("rot", [0.0, 2.0])
+def test_sensor_counts_and_half(ctx, n, rot):
+    fr = _frame(80, 33, rot, n=n, out_dtype=1)
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params), extra=parity.HALF_TOL)
+
+
+@pytest.mark.parametrize("w,h,rot", [(832, 760, 0.0), (832, 760, 0.2), (1250, 1010, 0.0), (1250, 1010, 0.2)])
+def test_larger_tiles_and_every_entry_point(ctx, w, h, rot):
+    """Two and four rows per thread (the frame sizes that choose them): sampled pixels and the border
+    against the oracle; batches of every launch configuration, the host-buffer bands and a server that
+    takes the frame in steps of odd tile counts return the same bits."""
+    from paper_1308_4908_gb300 import hdr
+    fr = _frame(w, h, rot)
+    out, ch, raws = _run(ctx, fr)
+    p = fr.params
+    r = np.random.default_rng(w)
+    pix = np.concatenate([np.stack([r.integers(0, w, 1500), r.integers(0, h, 1500)], 1),
+                          [[0, 0], [w - 1, 0], [0, h - 1], [w - 1, h - 1]]])
+    _against_oracle(fr, out, ch, pix)
+    for cfg in (hdr.hdr_batch_config(16, 0, 1, 0), hdr.hdr_batch_config(8, 0, 1, 0),
+                hdr.hdr_batch_config(16, 0, 1, 0, 2, 1), hdr.hdr_batch_config(16, 0, 1, 0, 1, 2)):
+        o = torch.full((3, h, w), -7.0, device="cuda")
+        c = torch.full((3, h, w), 77, dtype=torch.uint8, device="cuda")
+        keep = [raws]
+        ctx.reconstruct_batch([ctx.frame(0, p, raws, o, c, keep)], cfg)
+        ctx.check()
+        np.testing.assert_array_equal(o.cpu().numpy(), out)
+        np.testing.assert_array_equal(c.cpu().numpy(), ch)
+    host = [np.ascontiguousarray(s.raw) for s in fr.sensors]
+    o, c = np.full((3, h, w), -7.0, np.float32), np.full((3, h, w), 77, np.uint8)
+    ctx.reconstruct_host(0, p, host, o, c)
+    np.testing.assert_array_equal(o, out)
+    np.testing.assert_array_equal(c, ch)
+    own = hdr.Context(0)
+    try:
+        own.set_rig(0, fr.sensors)
+        srv = hdr.Server(own, max_frames=2, pool_bytes=256 << 20, step_tiles=777)
+        o[:], c[:] = -7.0, 77
+        assert srv.poll(srv.submit(0, p, host, o, c)).status == hdr.HDR_OK
+        srv.close()
+    finally:
+        own.close()
+    np.testing.assert_array_equal(o, out)
+    np.testing.assert_array_equal(c, ch)
