@@ -734,6 +734,14 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     return HDR_OK;
   }
   L.tx_bytes = tx;
+  // the pixel steps that span two sensor px of the first sensor (the others differ by their slight
+  // misalignment); beyond 4 (enlargements over 2.25 times) neighbours differ little: as at 1x
+  auto stride = [](double step) {
+    const double n = std::round(2.0 / step);
+    return n >= 1.0 && n <= 4.0 ? (int)n : n < 1.0 ? 1 : 2;
+  };
+  const double *G0 = L.s[0].G;
+  L.px_map = 4 * (stride(std::hypot(G0[1], G0[4])) - 1) + stride(std::hypot(G0[0], G0[3])) - 1;
   // a usable fit's equilibrated pivots lie in (min_pivot, 1]: when min_pivot * cond_fallback >= 2
   // their spread never exceeds cond_fallback and the FP64 re-solve cannot trigger
   const bool f64_possible = p->cond_fallback > 0.0 && (p->min_pivot - 1e-4) * p->cond_fallback < 2.0;

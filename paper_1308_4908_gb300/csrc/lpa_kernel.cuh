@@ -20,8 +20,8 @@
 //      ascending order, with a warp-wide early exit once every lane's
 //      intersection is empty; order fallback at the largest scale; NaN when
 //      nothing is usable.
-// Warps hold pixels of one output parity class (16x8 pixels, stride 2), so on
-// rigs close to a translation at 1x output every lane sees the same sample
+// Warps hold pixels of one phase class (PixelMap: 8x4 pixels at stride 2 at 1x
+// output), so on rigs close to a translation every lane sees the same sample
 // layout and the window loops run without divergence.
 #pragma once
 #include <cuda_fp16.h>
@@ -509,6 +509,33 @@ struct MultiScale {
   static constexpr int value = lpa_scales_per_walk(ORDER, COMP, MODE);
 };
 
+// Which pixel of its 16 x TH tile each thread takes. Output pixels whose step spans two sensor pixels
+// (one cell of a colour phase) see the samples at the same fractions: every 2nd pixel at 1x, 3rd
+// at 1.5x, 4th at 2x. The threads take the classes of pixels equal modulo (sx, sy) one after the
+// other (each class row by row; classes in serpentine order, so that a warp holding the end of one
+// class and the start of the next mixes neighbours), sx and sy in 1..4. At 1x this is 8 x 4 pixels
+// of one parity class per warp; 1920 x 1080 -> 2880 x 1620 at order 1, four scales, ran with 25.6 of
+// 32 lanes active per instruction and 64 M bank conflicts under that map: 3528 us, 2928 us under
+// its own.
+template <int TH>
+struct PixelMap {
+  uint8_t at[16][LPA_TILE * TH];  // [4 (sy - 1) + sx - 1][thread]: u | v << 4
+  constexpr PixelMap() : at{} {
+    for (int sy = 1; sy <= 4; sy++)
+      for (int sx = 1; sx <= 4; sx++) {
+        int n = 0;
+        for (int cy = 0; cy < sy; cy++)
+          for (int k = 0; k < sx; k++) {
+            const int cx = (cy & 1) ? sx - 1 - k : k;
+            for (int v = cy; v < TH; v += sy)
+              for (int u = cx; u < LPA_TILE; u += sx) at[4 * (sy - 1) + sx - 1][n++] = (uint8_t)(u | v << 4);
+          }
+      }
+  }
+};
+template <int TH>
+static __device__ const PixelMap<TH> pixel_map = PixelMap<TH>();
+
 struct Anchor {
   int ix, iy;
   float fx, fy;
@@ -906,11 +933,15 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
   // PX output pixels per thread, one after the other: slot k takes the rows k TH .. k TH + TH - 1
 #pragma unroll 1
   for (int slot = 0; slot < PX; slot++) {
-    // pixel of this thread: warp = parity class x half tile, lanes 8 x 4 at stride 2
-    const int warp = tid >> 5, lane = tid & 31;
-    const int par = warp & 3, hf = warp >> 2;
-    const int u = u0 + 2 * (lane & 7) + (par & 1);
-    const int v = v0 + 2 * ((lane >> 3) + 4 * hf) + (par >> 1) + slot * TH;
+    // this thread's pixel of the 16 x TH tile, read again where it is stored (a register through the
+    // window loops costs more)
+    auto mine = [&]() {
+      uint32_t m;
+      asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(m) : "l"(&pixel_map<TH>.at[RD(L.px_map)][tid]));
+      return (int)m;
+    };
+    const int at = mine();
+    const int u = u0 + (at & 15), v = v0 + (at >> 4) + slot * TH;
     const bool pix = (u < RD(L.out_w)) && (v < RD(L.out_h));
     const int ab = ((u - u0) >> 3) + 2 * ((v - v0) >> 3);  // < NA
     const int du = (u - u0) & 7, dv = (v - v0) & 7;
@@ -918,7 +949,10 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
     const int J = RD(L.n_scales);
     const int NL = J + ORDER;
     const size_t plane_px = (size_t)RD(L.out_w) * RD(L.out_h);
-    const size_t opix = (size_t)v * RD(L.out_w) + u;
+    auto index = [&]() {  // of the pixel in an output plane (at most 2^29 pixels)
+      const int m = mine();
+      return (uint32_t)(v0 + (m >> 4) + slot * TH) * (uint32_t)RD(L.out_w) + (uint32_t)(u0 + (m & 15));
+    };
     const float log2e = 1.4426950408889634f;
 
     constexpr bool TAB = lpa_mode_tab(MODE), STEER = lpa_mode_steered(MODE), GRAD = MODE == LPA_GRADIENTS;
@@ -939,7 +973,10 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
     }
     float4 Q = make_float4(1.f, 0.f, 1.f, 0.f);  // steering matrix of this pixel (Section 5.4)
     if constexpr (STEER)
-      if (pix) Q = make_float4(L.aux[opix * 3], L.aux[opix * 3 + 1], L.aux[opix * 3 + 2], 0.f);
+      if (pix) {
+        const float *q = L.aux + (size_t)index() * 3;
+        Q = make_float4(q[0], q[1], q[2], 0.f);
+      }
 
     using MOM = typename MomentsSel<ORDER, COMP, lpa_mode_var(MODE)>::type;
     // the fit of one (channel, scale) from its moments: factorised unless no lane of the warp has as
@@ -958,7 +995,7 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
     };
     auto put_level = [&](int c, int level, const FitOut &f) {
       if (DIAG && pix) {
-        float *o = L.levels + (((size_t)c * NL + level) * plane_px + opix) * 2;
+        float *o = L.levels + (((size_t)c * NL + level) * plane_px + index()) * 2;
         o[0] = f.valid ? f.c0 : __int_as_float(0x7fffffff);
         o[1] = f.valid ? f.var : __int_as_float(0x7fffffff);
       }
@@ -978,6 +1015,7 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
         if constexpr (ORDER >= 2) take(fallback_fit<ORDER, 1, F64>(m, RD(L.min_pivot), RD(L.cond_fallback)), 1);
       }
       if (pix) {
+        const size_t opix = index();
         if (RD(L.out_half))
           reinterpret_cast<__half *>(RD(L.out))[c * plane_px + opix] = __float2half_rn(ici.val);
         else
@@ -1064,8 +1102,9 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
         const FitOut f = fit_of(m);
         if constexpr (GRAD) {  // Section 5.4: the order-1 fit's linear coefficients; 0 if not usable
           if (pix) {
-            L.aux[opix * 2] = f.valid ? f.c1 : 0.f;
-            L.aux[opix * 2 + 1] = f.valid ? f.c2 : 0.f;
+            float *g = L.aux + (size_t)index() * 2;
+            g[0] = f.valid ? f.c1 : 0.f;
+            g[1] = f.valid ? f.c2 : 0.f;
           }
           break;
         }
