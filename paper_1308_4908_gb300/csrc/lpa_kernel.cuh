@@ -302,6 +302,83 @@ struct MomentsLean {
   __device__ __forceinline__ T Kv(int) const { return T(0); }
 };
 
+// comp_add on two sums at once: hi + lo += a b in each half, every operation rounded as there
+// (differences as products with -1; `na` is -a, so that the residual needs no negation).
+__device__ __forceinline__ void comp_add2(float2 &hi, float2 &lo, float2 a, float2 na, float2 b) {
+  const float2 M = make_float2(-1.f, -1.f);
+  const float2 p = __fmul2_rn(a, b);
+  const float2 npe = __ffma2_rn(na, b, p);  // -(a b - p)
+  const float2 s = __fadd2_rn(hi, p);
+  const float2 bb = __ffma2_rn(hi, M, s);
+  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, M, s), M, hi), __ffma2_rn(bb, M, p));
+  hi = s;
+  lo = __fadd2_rn(lo, __ffma2_rn(npe, M, e));
+}
+
+// Compensated sums of orders 1 and 2 without the variance sums, two at a time: the Gram sums in
+// pairs of monomials, (sum w, sum w f) together. The same terms, order and roundings as
+// Moments<ORDER, true>, whose one sum at a time issued 10 scalar operations a sum (87 % of issue
+// slots; order 2, 21 sums a sample).
+template <int ORDER>
+struct MomentsCompLean {
+  static constexpr bool HAS_VAR = false;
+  static constexpr int NA = n_monos(ORDER);
+  static constexpr int NB = n_unknowns(ORDER);
+  static constexpr int NP = ORDER == 2 ? 10 : 5;
+  // pairs: 0 (a_0, b_0), 1 (a_1, a_2), 2 (a_3, a_5), 3 (b_1, b_2), 4 (a_4, a_12 or nothing), then at order 2:
+  // 5 (a_6, a_9), 6 (a_7, a_8), 7 (a_10, a_14), 8 (a_11, a_13), 9 (b_3, b_5); b_4 alone
+  float2 h[NP], l[NP];
+  float b4, b4l;
+  float cnt;
+
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < NP; i++) h[i] = l[i] = make_float2(0.f, 0.f);
+    b4 = b4l = cnt = 0.f;
+  }
+  __device__ __forceinline__ float count() const { return cnt; }
+  __device__ __forceinline__ void add2(float2 D, float2 D2, float w, float wf, float) {
+    const float2 W = make_float2(w, w), NW = make_float2(-w, -w), F = make_float2(wf, wf), NF = make_float2(-wf, -wf);
+    const float m4 = D.x * D.y;
+    comp_add2(h[0], l[0], make_float2(w, wf), make_float2(-w, -wf), make_float2(1.f, 1.f));
+    comp_add2(h[1], l[1], W, NW, D);
+    comp_add2(h[2], l[2], W, NW, D2);
+    comp_add2(h[3], l[3], F, NF, D);
+    if constexpr (ORDER == 2) {
+      comp_add2(h[4], l[4], W, NW, make_float2(m4, D2.x * D2.y));
+      comp_add2(h[5], l[5], W, NW, __fmul2_rn(D2, D));
+      comp_add2(h[6], l[6], W, NW, make_float2(D2.x * D.y, m4 * D.y));
+      comp_add2(h[7], l[7], W, NW, __fmul2_rn(D2, D2));
+      comp_add2(h[8], l[8], W, NW, make_float2(D2.x * m4, m4 * D2.y));
+      comp_add2(h[9], l[9], F, NF, D2);
+      comp_add(b4, b4l, wf, m4);
+    } else {
+      comp_add(h[4].x, l[4].x, w, m4);
+    }
+    cnt += 1.f;
+  }
+  template <typename T>
+  static __device__ __forceinline__ T sum(float hi, float lo) {
+    return (T)hi + (T)lo;
+  }
+  template <typename T>
+  __device__ __forceinline__ T A(int i) const {
+    constexpr int at[15] = {0, 1, 1, 2, 4, 2, 5, 6, 6, 5, 7, 8, 4, 8, 7};
+    constexpr bool second[15] = {0, 0, 1, 0, 0, 1, 0, 0, 1, 1, 0, 0, 1, 1, 1};
+    const int k = at[i] < NP ? at[i] : 0;
+    return second[i] ? sum<T>(h[k].y, l[k].y) : sum<T>(h[k].x, l[k].x);
+  }
+  template <typename T>
+  __device__ __forceinline__ T B(int i) const {
+    if (i == 0) return sum<T>(h[0].y, l[0].y);
+    if (i == 4) return sum<T>(b4, b4l);
+    const int k = i <= 2 ? 3 : NP - 1;
+    return (i == 2 || i == 5) ? sum<T>(h[k].y, l[k].y) : sum<T>(h[k].x, l[k].x);
+  }
+  template <typename T>
+  __device__ __forceinline__ T Kv(int) const { return T(0); }
+};
+
 // The accumulator a kernel uses: paired for plain FP32 sums of order >= 1.
 template <int ORDER, bool COMP, bool VAR = true, bool PACKED = (LPA_PACKED_MOMENTS != 0) && !COMP && ORDER >= 1>
 struct MomentsSel {
@@ -314,6 +391,14 @@ struct MomentsSel<ORDER, false, true, true> {
 template <int ORDER>
 struct MomentsSel<ORDER, false, false, true> {
   using type = MomentsLean<ORDER>;
+};
+template <>
+struct MomentsSel<1, true, false, false> {
+  using type = MomentsCompLean<1>;
+};
+template <>
+struct MomentsSel<2, true, false, false> {
+  using type = MomentsCompLean<2>;
 };
 
 // ---------------------------------------------------------------- solve
