@@ -30,16 +30,17 @@ __device__ __forceinline__ float quotient(float hi, float lo, float den, float r
   return __fadd_rn(qh, ql * 1.00006f) == qh ? qh : exact();
 }
 
-// One thread: 8 consecutive pixels of one row (one 16-byte load per frame, eight frames in flight).
+// One thread: 8 consecutive pixels of one row (one 16-byte load per frame, sixteen frames in flight).
 // Exact sums S1 = sum y (< 2^28) and S2 = sum y^2 (< 2^44); mean = S1 / n and the unbiased variance
 // (n S2 - S1^2) / (n (n - 1)), each the FP64 quotient rounded to FP32, which is the correctly
 // rounded quotient (it lies further from every midpoint of two floats than an FP64 rounding, or on
 // it exactly), so it is formed in FP32 pairs instead: an FP64 instruction takes 16 cycles of an SM,
 // and the two divisions per pixel kept its FP64 pipe busy for 78 % of the kernel. Two frames' samples of a
 // pixel are summed at a time as 16 x 8-bit dot products: y (1, 1), y (low bytes), y (high bytes).
-// 64 frames of 2330 x 1752: 114 us (4.9 TB/s) against 187 us with the FP64 divisions and 64-bit
-// products per sample; bound by the reads.
-__global__ void __launch_bounds__(kThreads) calib_stats(const uint16_t *__restrict__ frames, int n, int width,
+// 64 frames of 2330 x 1752: 95 us (5.8 TB/s) against 187 us with the FP64 divisions and 64-bit
+// products per sample; bound by the reads. Sixteen loads in flight of 512 threads per SM: eight of
+// 1024 threads took 113 us (its CTAs fill 3.3 waves), half of the frames per thread 96 us.
+__global__ void __launch_bounds__(kThreads, 2) calib_stats(const uint16_t *__restrict__ frames, int n, int width,
                                                         int height, int pitch, long long stride,
                                                         float *__restrict__ mean, float *__restrict__ var) {
   const int groups = (width + 7) >> 3;
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kThreads) calib_stats(const uint16_t *__restri
       }
     };
     int f = f0;
-#pragma unroll 4
+#pragma unroll 8
     for (; f + 1 < f1; f += 2) {
       const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p + (long long)f * stride));
       const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p + (long long)(f + 1) * stride));
