@@ -65,10 +65,10 @@ inline const void *lpa_kernel(int order, bool comp, bool diag, int mode, int til
 
 // Order 0 with one window scale (LPA_MEAN). The kernel template for windows that reach reach_rb (R, B) and
 // reach_g (G) sensor px, -1 if they hold more cells than any is built for; its candidate cells per
-// axis; bytes of its position tables for p rows per thread.
+// axis; bytes of its position tables for p rows per thread (classes: periodic positions, both axes' classes).
 int lpa_mean_size(double reach_rb, double reach_g);
 int lpa_mean_cells(int size, bool green);
-uint32_t lpa_mean_tab_bytes(int size, bool axis, int p, int n_sensors);
+uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors);
 // Its kernel (LPA_MEAN_THREADS threads), grid and launch over the tile rows of L's range.
 const void *lpa_mean_kernel(const LpaLaunch &L);
 unsigned lpa_mean_grid(const LpaLaunch &L);

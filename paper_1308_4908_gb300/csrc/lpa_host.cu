@@ -311,6 +311,7 @@ namespace {
 struct MeanPlan {
   int size = -1;      // kernel template, -1: another kernel
   bool axis = true;   // every sensor's axes are parallel to the output's
+  int tx = 0, ty = 0; // output pixels to a cell of a colour phase where that is exact (2 or 4), else 0
   int p = 1;          // output rows per thread
   double rb = 0, g = 0;  // window radius of R and B, and of G (reference px)
 };
@@ -329,12 +330,20 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   m.g = m.rb * p->green_ratio;
   m.axis = p->out_affine[1] == 0.0 && p->out_affine[3] == 0.0;
   double most = 0.0;
+  auto period = [](double step) {  // of positions modulo 2 px, to the tolerance of the tabulated weights
+    return std::fabs(step - 1.0) <= 1e-12 ? 2 : std::fabs(step - 0.5) <= 1e-12 ? 4 : 0;
+  };
   for (int s = 0; s < rig.n; s++) {
-    double t[6];
+    double t[6], G[6];
     invert_affine(rig.s[s].d.affine, t);
+    compose_affine(t, p->out_affine, G);
+    const int tx = period(G[0]), ty = period(G[4]);
+    m.tx = s == 0 || m.tx == tx ? tx : 0;
+    m.ty = s == 0 || m.ty == ty ? ty : 0;
     most = std::max(most, std::max(std::hypot(t[0], t[1]), std::hypot(t[3], t[4])));
     m.axis = m.axis && t[1] == 0.0 && t[3] == 0.0;
   }
+  if (!m.axis || !m.tx || !m.ty) m.tx = m.ty = 0;
   m.size = lpa_mean_size(m.rb * most + 2e-3, m.g * most + 2e-3);
   const long long px = (long long)p->out_w * p->out_h;
   m.p = px >= 4LL * 152 * 64 * 32 ? 4 : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
@@ -370,7 +379,7 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, uint3
     mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);
     need = std::max(need, 8.0 * bw * bh);
   }
-  const double all = 2.0 * need + lpa_mean_tab_bytes(m.size, m.axis, m.p, rig.n);
+  const double all = 2.0 * need + lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n);
   if (all > 110.0 * 1024) return 0;
   *plane = (uint32_t)need;
   *tab = 2u * *plane;
@@ -730,6 +739,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     L.mean_p = mean.p;
     L.mean_size = mean.size;
     L.mean_axis = mean.axis ? 1 : 0;
+    L.mean_tx = mean.tx;
+    L.mean_ty = mean.ty;
     L.stages = 1;
     return HDR_OK;
   }
@@ -1579,7 +1590,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis : L.px,
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 128 * (L.mean_tx != 0) : L.px,
                    L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};

@@ -101,9 +101,10 @@ struct LpaLaunch {
   int mode;
   float *aux;
   // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, whether every sensor's axes are
-  // parallel to the output's, bytes of one buffer of colour-phase planes (two from offset 0) and
+  // parallel to the output's, the pixels that span one cell of a colour phase where that is exact for
+  // every sensor (2 or 4 on each axis, else both 0), bytes of one buffer of colour-phase planes (two from offset 0) and
   // the offset of the position tables
-  int mean_p, mean_size, mean_axis;
+  int mean_p, mean_size, mean_axis, mean_tx, mean_ty;
   uint32_t mean_plane, mean_tab;
 };
 

@@ -18,9 +18,12 @@
 // 4096^2 FP16 1226 -> 303 us, the four sensors (tabulated windows before) 517 -> 172 us, 64^2 14.4 -> 10.3 us a call;
 // 1024 x 900, three rotated sensors 147 -> 78 us.
 //
-// AXIS: every sensor's axes are parallel to the output's, so the Gaussian factors into a column and
+// kAxis: every sensor's axes are parallel to the output's, so the Gaussian factors into a column and
 // a row factor, tabulated per tile: a cell is one FMA, one maximum, the load and the paired FMA.
-// Otherwise each cell forms its offset and one exponential.
+// kPeriodic: besides, 2 or 4 output pixels span exactly one cell of a colour phase (translated sensors at
+// 1x or twofold output), so pixels that far apart see the same offsets: a thread takes P rows of one
+// class, forms the K of its cells once per sensor and slides the window down one cell a row, each
+// loaded cell serving up to N rows. kGeneral: each cell forms its offset and one exponential.
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -100,7 +103,42 @@ __device__ __forceinline__ int2 box_origin(const LpaSensorK &S, int u0, int v0, 
   return make_int2((int)floorf(x) & ~7, (int)floorf(y) & ~1);
 }
 
-template <int NR, int NG, bool AXIS, int P>
+enum { kGeneral = 0, kAxis = 1, kPeriodic = 2 };
+
+// The cells and factors of one position along one axis for every (window, phase): words of Layout at
+// t[0], t[stride], ... `last`: how many cells further the last position served by the entry lies. Returns
+// false if a first cell had to be moved so that all of them lie in the box.
+template <int NR, int NG>
+__device__ __forceinline__ bool axis_entry(const LpaLaunch &L, const LpaSensorK &Sk, bool col, int l, float f, int last, float *t,
+                                           int stride) {
+  const float log2e = 1.4426950408889634f;
+  const float a = col ? Sk.A[0] : Sk.A[3];
+  const int cells = (col ? Sk.box_w : Sk.box_h) >> 1, step = col ? 1 : Sk.box_w >> 1;
+  bool ok = true;
+#pragma unroll
+  for (int g = 0; g < 2; g++) {
+    const int N = g ? NG : NR;
+    const float sg = g ? L.sigma[0] * L.green_ratio : L.sigma[0];
+    const float h = L.trunc_k * sg * (col ? Sk.hx_unit : Sk.hy_unit) + 1e-3f, m = floorf(0.5f * h);
+    const float c = -log2e / (2.f * sg * sg) * a * a;
+#pragma unroll
+    for (int ph = 0; ph < 2; ph++) {
+      float d;
+      const int i = first_cell(l, f, ph, h, m, d), at = max(min(i, cells - N - last), 0);
+      ok = ok && i == at;
+      t[(2 * g + ph) * stride] = __int_as_float(at * step);
+      float *w = t + (4 + 2 * NR * g + N * ph) * stride;
+#pragma unroll
+      for (int j = 0; j < N; j++) {
+        const float dj = d + 2.f * (float)j;
+        w[j * stride] = ex2_approx(c * dj * dj);
+      }
+    }
+  }
+  return ok;
+}
+
+template <int NR, int NG, int FORM, int P>
 __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ LpaLaunch L) {
   using T = Layout<NR, NG>;
   constexpr int BH = 8 * P;
@@ -117,7 +155,24 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
   float *xt = reinterpret_cast<float *>(smem + L.mean_tab);
   float *yt = xt + S * T::kWords * kBW;
   int4 *anchor = reinterpret_cast<int4 *>(smem + L.mean_tab);
-  if constexpr (AXIS) {
+  const int tx = L.mean_tx, ty = L.mean_ty;
+  if constexpr (FORM == kPeriodic) {
+    // one entry per sensor, axis and class of positions: class c starts at G c + G_t, and the n-th
+    // pixel of a class lies exactly 2 n px further, whatever the tile
+    if (tid < S * (tx + ty)) {
+      const int s = tid / (tx + ty), e = tid - s * (tx + ty);
+      const bool col = e < tx;
+      const int c = col ? e : e - tx;
+      const LpaSensorK &Sk = L.s[s];
+      const int2 o = box_origin(Sk, u0, v0, BH);
+      const double q = fmin(fmax(col ? Sk.G[0] * c + Sk.G[2] : Sk.G[4] * c + Sk.G[5], -LPA_FAR), LPA_FAR), fl = floor(q);
+      const int l = (int)fl + (col ? 2 * (u0 / tx) - o.x : 2 * (v0 / ty) - o.y);
+      float *t = xt + tid * T::kRow;
+      const int last = col ? (kBW - 1) / tx : (BH - 1) / ty;
+      if (!axis_entry<NR, NG>(L, Sk, col, l, (float)(q - fl), last, t, 1) && (col ? u0 + c < L.out_w : v0 + c < y_end) && fabs(q) < 1e6)
+        atomicOr(L.status, LPA_ERR_BOUNDS);
+    }
+  } else if constexpr (FORM == kAxis) {
     for (int k = tid; k < S * (kBW + BH); k += kThreads) {
       const int s = k / (kBW + BH), e = k - s * (kBW + BH);
       const bool col = e < kBW;
@@ -126,31 +181,10 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
       const double q = fmin(fmax(col ? Sk.G[0] * (u0 + e) + Sk.G[2] : Sk.G[4] * (v0 + e - kBW) + Sk.G[5], -LPA_FAR), LPA_FAR);
       const double fl = floor(q);
       const int l = (int)fl - (col ? o.x : o.y);
-      const float f = (float)(q - fl), a = col ? Sk.A[0] : Sk.A[3];
-      const int cells = (col ? Sk.box_w : Sk.box_h) >> 1, step = col ? 1 : Sk.box_w >> 1;
       float *t = col ? xt + s * T::kWords * kBW + e : yt + (s * BH + e - kBW) * T::kRow;
-      const int stride = col ? kBW : 1;
-      bool ok = true;
-#pragma unroll
-      for (int g = 0; g < 2; g++) {
-        const int N = g ? NG : NR;
-        const float h = L.trunc_k * sg[g] * (col ? Sk.hx_unit : Sk.hy_unit) + 1e-3f, m = floorf(0.5f * h);
-        const float c = -log2e / (2.f * sg[g] * sg[g]) * a * a;
-#pragma unroll
-        for (int ph = 0; ph < 2; ph++) {
-          float d;
-          const int i = first_cell(l, f, ph, h, m, d), at = min(max(i, 0), cells - N);
-          ok = ok && i == at;
-          t[(2 * g + ph) * stride] = __int_as_float(at * step);
-          float *w = t + (4 + 2 * NR * g + N * ph) * stride;
-#pragma unroll
-          for (int j = 0; j < N; j++) {
-            const float dj = d + 2.f * (float)j;
-            w[j * stride] = ex2_approx(c * dj * dj);
-          }
-        }
-      }
-      if (!ok && (col ? u0 + e < L.out_w : v0 + e - kBW < y_end) && fabs(q) < 1e6) atomicOr(L.status, LPA_ERR_BOUNDS);
+      if (!axis_entry<NR, NG>(L, Sk, col, l, (float)(q - fl), 0, t, col ? kBW : 1) &&
+          (col ? u0 + e < L.out_w : v0 + e - kBW < y_end) && fabs(q) < 1e6)
+        atomicOr(L.status, LPA_ERR_BOUNDS);
     }
   } else {
     constexpr int NA = 8 * P;  // 8 x 8 blocks of the tile
@@ -166,7 +200,9 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
     }
   }
 
-  const int col = (tid & 31) + 32 * ((tid >> 5) & 1), row0 = (tid >> 6) * P;
+  // this thread's column and its P rows: row0 + k, or (kPeriodic) row0 + ty k
+  const int col = (tid & 31) + 32 * ((tid >> 5) & 1), group = tid >> 6;
+  const int row0 = FORM == kPeriodic ? group / ty * (ty * P) + group % ty : group * P;
   const int u = u0 + col;
   float2 acc[P][3];  // per row and channel: (sum K / s2, sum K f / s2)
 #pragma unroll
@@ -192,7 +228,34 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
     }
     __syncthreads();  // the planes are whole; the other buffer's readers have left it
     const int PW = Sk.box_w >> 1, PP = PW * (Sk.box_h >> 1);
-    if constexpr (AXIS) {
+    if constexpr (FORM == kPeriodic) {
+      const float *ex = xt + (s * (tx + ty) + col % tx) * T::kRow;
+      const float *ey = xt + (s * (tx + ty) + tx + group % ty) * T::kRow;
+      const int shift = col / tx + group / ty * P * PW;  // whole cells from the class's first pixel
+      auto phase = [&](auto N_, auto c_, int ox, int oy, int g) {
+        constexpr int N = decltype(N_)::value, c = decltype(c_)::value;
+        const float *fx = ex + 4 + 2 * NR * g + N * ox, *fy = ey + 4 + 2 * NR * g + N * oy;
+        float K[N][N];
+#pragma unroll
+        for (int j = 0; j < N; j++)
+#pragma unroll
+          for (int i = 0; i < N; i++) K[j][i] = fmaxf(fmaf(fx[i], fy[j], -L.taper), 0.f);
+        const float2 *pl = planes + (ox + 2 * oy) * PP + shift + __float_as_int(ex[2 * g + ox]) + __float_as_int(ey[2 * g + oy]);
+#pragma unroll
+        for (int r = 0; r < N + P - 1; r++)
+#pragma unroll
+          for (int i = 0; i < N; i++) {
+            const float2 cell = pl[r * PW + i];
+#pragma unroll
+            for (int k = 0; k < P; k++)
+              if (r - k >= 0 && r - k < N) acc[k][c] = __ffma2_rn(make_float2(K[r - k][i], K[r - k][i]), cell, acc[k][c]);
+          }
+      };
+      phase(std::integral_constant<int, NR>(), std::integral_constant<int, 0>(), 0, 0, 0);
+      phase(std::integral_constant<int, NG>(), std::integral_constant<int, 1>(), 1, 0, 1);
+      phase(std::integral_constant<int, NG>(), std::integral_constant<int, 1>(), 0, 1, 1);
+      phase(std::integral_constant<int, NR>(), std::integral_constant<int, 2>(), 1, 1, 0);
+    } else if constexpr (FORM == kAxis) {
       const float *tx = xt + s * T::kWords * kBW + col;
       int xi[4];
       float ex[T::kE];
@@ -275,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
   const size_t plane = (size_t)L.out_w * L.out_h;
 #pragma unroll
   for (int k = 0; k < P; k++) {
-    const int v = v0 + row0 + k;
+    const int v = v0 + row0 + (FORM == kPeriodic ? ty * k : k);
     if (v >= y_end) return;
     const size_t at = (size_t)v * L.out_w + u;
 #pragma unroll
@@ -289,11 +352,17 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
   }
 }
 
-template <int NR, int NG, bool AXIS>
+template <int NR, int NG, int FORM>
 const void *pick(int p) {
-  return p == 1   ? (const void *)lpa_mean<NR, NG, AXIS, 1>
-         : p == 2 ? (const void *)lpa_mean<NR, NG, AXIS, 2>
-                  : (const void *)lpa_mean<NR, NG, AXIS, 4>;
+  return p == 1   ? (const void *)lpa_mean<NR, NG, FORM, 1>
+         : p == 2 ? (const void *)lpa_mean<NR, NG, FORM, 2>
+                  : (const void *)lpa_mean<NR, NG, FORM, 4>;
+}
+template <int NR, int NG>
+const void *pick(const LpaLaunch &L) {
+  return L.mean_tx     ? pick<NR, NG, kPeriodic>(L.mean_p)
+         : L.mean_axis ? pick<NR, NG, kAxis>(L.mean_p)
+                       : pick<NR, NG, kGeneral>(L.mean_p);
 }
 
 }  // namespace
@@ -304,16 +373,14 @@ int lpa_mean_size(double reach_rb, double reach_g) {
   return rb <= 3 && g <= 2 ? 0 : rb <= 4 && g <= 3 ? 1 : -1;
 }
 int lpa_mean_cells(int size, bool green) { return size == 0 ? (green ? 2 : 3) : (green ? 3 : 4); }
-uint32_t lpa_mean_tab_bytes(int size, bool axis, int p, int n_sensors) {
+uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors) {
   if (!axis) return (uint32_t)(n_sensors * 8 * p * 16);
   const int words = size == 0 ? lpa::Layout<3, 2>::kWords : lpa::Layout<4, 3>::kWords;
   const int row = size == 0 ? lpa::Layout<3, 2>::kRow : lpa::Layout<4, 3>::kRow;
+  if (classes) return (uint32_t)(n_sensors * 4 * row * classes);
   return (uint32_t)(n_sensors * 4 * (words * lpa::kBW + row * 8 * p));
 }
-const void *lpa_mean_kernel(const LpaLaunch &L) {
-  if (L.mean_size == 0) return L.mean_axis ? lpa::pick<3, 2, true>(L.mean_p) : lpa::pick<3, 2, false>(L.mean_p);
-  return L.mean_axis ? lpa::pick<4, 3, true>(L.mean_p) : lpa::pick<4, 3, false>(L.mean_p);
-}
+const void *lpa_mean_kernel(const LpaLaunch &L) { return L.mean_size == 0 ? lpa::pick<3, 2>(L) : lpa::pick<4, 3>(L); }
 unsigned lpa_mean_grid(const LpaLaunch &L) {
   const long rows = lpa_end_row(L) - lpa_first_row(L), bh = 8 * L.mean_p;
   return (unsigned)((L.out_w + lpa::kBW - 1) / lpa::kBW * ((rows + bh - 1) / bh));
