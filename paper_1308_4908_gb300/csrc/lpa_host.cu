@@ -365,9 +365,9 @@ void mean_box(const MeanPlan &m, const double G[6], double hxu, double hyu, int 
   *bh = ((int)std::ceil(std::fabs(G[3]) * w + std::fabs(G[4]) * h + sides(hyu, ext_y)) + 2 + 1) / 2 * 2;
 }
 
-// lpa_mean's shared memory for a rig (two buffers of the largest box's planes, then the tables), or 0
-// where it would leave fewer than two CTAs on an SM.
-uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, uint32_t *plane, uint32_t *tab) {
+// lpa_mean's shared memory for a rig: planes of the largest box for *bufs sensors (all, or as many as
+// leave two CTAs on an SM), then the tables; 0 where not even one sensor's fit.
+uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *bufs, uint32_t *plane, uint32_t *tab) {
   double need = 0.0;
   for (int s = 0; s < rig.n; s++) {
     double t[6], G[6];
@@ -379,17 +379,19 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, uint3
     mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);
     need = std::max(need, 8.0 * bw * bh);
   }
-  const double all = 2.0 * need + lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n);
-  if (all > 110.0 * 1024) return 0;
+  const double tables = lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n), room = 110.0 * 1024 - tables;
+  if (need > room) return 0;
+  *bufs = std::min(rig.n, (int)(room / need));
   *plane = (uint32_t)need;
-  *tab = 2u * *plane;
-  return (uint32_t)all;
+  *tab = *bufs * *plane;
+  return *tab + (uint32_t)tables;
 }
 
 bool runs_mean(const Rig &rig, const hdr_params *p) {
   const MeanPlan m = mean_plan(rig, p);
+  int bufs;
   uint32_t plane, tab;
-  return m.size >= 0 && mean_smem(rig, p, m, &plane, &tab) > 0;
+  return m.size >= 0 && mean_smem(rig, p, m, &bufs, &plane, &tab) > 0;
 }
 
 bool conv_eligible(const Rig &rig, const hdr_params *p, bool adaptive, bool mean = true) {
@@ -614,7 +616,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   MeanPlan mean;
   if (env.mean) mean = mean_plan(rig, p);
   if (mean.size >= 0) {
-    L.smem_bytes = mean_smem(rig, p, mean, &L.mean_plane, &L.mean_tab);
+    L.smem_bytes = mean_smem(rig, p, mean, &L.mean_bufs, &L.mean_plane, &L.mean_tab);
     if (L.smem_bytes == 0) mean.size = -1;
   }
   if (mean.size >= 0) conv = nullptr;  // lpa_mean reads the raw frames
@@ -655,6 +657,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     K.raw_pitch = d.pitch_elems;
     if (mean.size >= 0) {
       mean_box(mean, K.G, hxu, hyu, &K.box_w, &K.box_h, &K.ext_x, &K.ext_y);
+      // rounded up: exact for the box's at most 14,000 groups (2^32 / 14,000 exceeds any box_w / 8)
+      K.group_magic = (uint32_t)(((1ull << 32) + K.box_w / 8 - 1) / (K.box_w / 8));
       continue;
     }
     // staging box: the tile's pixel points span |G_lin| * (TILE-1) in sensor space; add the

@@ -44,6 +44,7 @@ struct alignas(64) LpaSensorK {
   const uint16_t *raw;
   float2 *conv;
   int raw_pitch, conv_pitch, conv_h;
+  uint32_t group_magic;     // lpa_mean: g / (box_w / 8) = high word of g times this, for the box's groups
 };
 
 struct LpaLaunch {
@@ -102,9 +103,9 @@ struct LpaLaunch {
   float *aux;
   // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, whether every sensor's axes are
   // parallel to the output's, the pixels that span one cell of a colour phase where that is exact for
-  // every sensor (2 or 4 on each axis, else both 0), bytes of one buffer of colour-phase planes (two from offset 0) and
-  // the offset of the position tables
-  int mean_p, mean_size, mean_axis, mean_tx, mean_ty;
+  // every sensor (2 or 4 on each axis, else both 0), sensors staged at a time, bytes of one sensor's
+  // colour-phase planes (from offset 0) and the offset of the position tables
+  int mean_p, mean_size, mean_axis, mean_tx, mean_ty, mean_bufs;
   uint32_t mean_plane, mean_tab;
 };
 

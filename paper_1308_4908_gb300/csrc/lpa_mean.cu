@@ -8,10 +8,10 @@
 // exp(-r^2 / 2 sigma^2) - exp(-k^2 / 2) (Eq. 8) is not positive there and is cut at 0.
 //
 // A CTA of 512 threads reconstructs 64 x 8 P pixels, P rows per thread; lanes are consecutive
-// pixels of a row, so stores coalesce and neighbours read the same cells. Sensors come one after the
-// other: their raw footprint is read straight from global memory (16-byte loads, the next sensor's
-// in flight during this one's sums), converted once per sample (Eqs. 18 and 20) into colour-phase
-// planes of (1 / s2, f / s2) in shared memory, double-buffered: one barrier per sensor. Each cell is
+// pixels of a row, so stores coalesce and neighbours read the same cells. The raw footprints of all sensors
+// (of as many as two CTAs' shared memory holds) are read straight from global memory (16-byte loads,
+// two in flight per thread) and converted once per sample (Eqs. 18 and 20) into colour-phase planes of
+// (1 / s2, f / s2) in shared memory; one barrier later the sums of every sensor follow. Each cell is
 // then one shared load and one paired FMA into (sum K / s2, sum K f / s2). No conversion pass goes
 // ahead of the kernel: with 64 x 32 tiles a sample is converted about 1.5 times, and the pass cost
 // 47 us of 517 on four 2336 x 1752 sensors. Measured against the general kernel with that pass: 2 x 2048^2 ->
@@ -62,36 +62,11 @@ struct Layout {
   static constexpr int kRow = (kWords + 3) / 4 * 4;
 };
 
-// Raw samples of group g (eight columns of a row) of the box at (x0, y0), or zeros off the frame.
-__device__ __forceinline__ uint4 load_group(const LpaSensorK &S, int x0, int y0, int g, int groups_x) {
-  const int row = g / groups_x, X = x0 + 8 * (g - row * groups_x), Y = y0 + row;
-  if (X < 0 || X >= S.width || Y < 0 || Y >= S.height) return make_uint4(0, 0, 0, 0);
-  return __ldg(reinterpret_cast<const uint4 *>(S.raw + (size_t)Y * S.raw_pitch + X));
-}
-
-__device__ __forceinline__ void store_group(const LpaSensorK &S, int x0, int y0, int g, int groups_x, uint4 q, float2 *planes) {
-  const int row = g / groups_x, col = g - row * groups_x, X = x0 + 8 * col, Y = y0 + row;
-  const int PW = S.box_w >> 1, PP = PW * (S.box_h >> 1);
-  const bool scalar = !S.bias && !S.rvar && !S.satf && !S.prnu;
-  const bool in = X >= 0 && Y >= 0 && Y < S.height;
-  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-  float4 *even = reinterpret_cast<float4 *>(planes + 2 * (row & 1) * PP + (row >> 1) * PW + 4 * col);
-  float4 *odd = reinterpret_cast<float4 *>(planes + (2 * (row & 1) + 1) * PP + (row >> 1) * PW + 4 * col);
-  float2 v[8];
-#pragma unroll
-  for (int k = 0; k < 8; k++) {
-    const uint32_t y = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
-    v[k] = make_float2(0.f, 0.f);
-    if (in && X + k < S.width) {
-      const float2 fv = convert_sample<false>(S, scalar, X + k, Y, (float)y);  // (f, 1 / s2)
-      v[k] = make_float2(fv.y, fv.y * fv.x);
-    }
-  }
-  even[0] = make_float4(v[0].x, v[0].y, v[2].x, v[2].y);
-  even[1] = make_float4(v[4].x, v[4].y, v[6].x, v[6].y);
-  odd[0] = make_float4(v[1].x, v[1].y, v[3].x, v[3].y);
-  odd[1] = make_float4(v[5].x, v[5].y, v[7].x, v[7].y);
-}
+// A group of eight columns of one row of a sensor's box: where it lies and its raw samples, zeros off the frame.
+struct Group {
+  int s, row, col, X, Y;
+  uint4 q;
+};
 
 // Box origin of a tile in sensor s: x on a multiple of 8 (16-byte loads), y even. FP32 is enough
 // (the box has a margin of a pixel), and every thread forms the same value.
@@ -101,6 +76,45 @@ __device__ __forceinline__ int2 box_origin(const LpaSensorK &S, int u0, int v0, 
   x = fminf(fmaxf(x + S.Gt[0] - S.ext_x, -LPA_FAR_F), LPA_FAR_F);
   y = fminf(fmaxf(y + S.Gt[1] - S.ext_y, -LPA_FAR_F), LPA_FAR_F);
   return make_int2((int)floorf(x) & ~7, (int)floorf(y) & ~1);
+}
+
+__device__ __forceinline__ Group load_group(const LpaLaunch &L, int s, int g, int u0, int v0, int bh) {
+  const LpaSensorK &S = L.s[s];
+  const int2 o = box_origin(S, u0, v0, bh);
+  Group r;
+  r.s = s;
+  r.row = (int)__umulhi((unsigned)g, S.group_magic);
+  r.col = g - r.row * (S.box_w >> 3);
+  r.X = o.x + 8 * r.col;
+  r.Y = o.y + r.row;
+  r.q = make_uint4(0, 0, 0, 0);
+  if (r.X >= 0 && r.X < S.width && r.Y >= 0 && r.Y < S.height)
+    r.q = __ldg(reinterpret_cast<const uint4 *>(S.raw + (size_t)r.Y * S.raw_pitch + r.X));
+  return r;
+}
+
+__device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, float2 *planes) {
+  const LpaSensorK &S = L.s[r.s];
+  const int PW = S.box_w >> 1, PP = PW * (S.box_h >> 1);
+  const bool scalar = !S.bias && !S.rvar && !S.satf && !S.prnu;
+  const int n = r.X >= 0 && r.Y >= 0 && r.Y < S.height ? S.width - r.X : 0;  // columns inside the frame
+  const uint32_t w[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
+  float4 *even = reinterpret_cast<float4 *>(planes + 2 * (r.row & 1) * PP + (r.row >> 1) * PW + 4 * r.col);
+  float4 *odd = even + (PP >> 1);
+  float2 v[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    const uint32_t y = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
+    v[k] = make_float2(0.f, 0.f);
+    if (k < n) {
+      const float2 fv = convert_sample<false>(S, scalar, r.X + k, r.Y, (float)y);  // (f, 1 / s2)
+      v[k] = make_float2(fv.y, fv.y * fv.x);
+    }
+  }
+  even[0] = make_float4(v[0].x, v[0].y, v[2].x, v[2].y);
+  even[1] = make_float4(v[4].x, v[4].y, v[6].x, v[6].y);
+  odd[0] = make_float4(v[1].x, v[1].y, v[3].x, v[3].y);
+  odd[1] = make_float4(v[5].x, v[5].y, v[7].x, v[7].y);
 }
 
 enum { kGeneral = 0, kAxis = 1, kPeriodic = 2 };
@@ -210,23 +224,35 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
 #pragma unroll
     for (int c = 0; c < 3; c++) acc[k][c] = make_float2(0.f, 0.f);
 
-  int2 o = box_origin(L.s[0], u0, v0, BH);
-  uint4 q = make_uint4(0, 0, 0, 0);
-  if (tid < (L.s[0].box_w >> 3) * L.s[0].box_h) q = load_group(L.s[0], o.x, o.y, tid, L.s[0].box_w >> 3);
+  // the sensors of one filling of the plane buffers at a time (all of them, unless they are many)
 #pragma unroll 1
-  for (int s = 0; s < S; s++) {
-    const LpaSensorK &Sk = L.s[s];
-    float2 *planes = reinterpret_cast<float2 *>(smem + (s & 1) * L.mean_plane);
-    const int gx = Sk.box_w >> 3, n = gx * Sk.box_h;
-    if (tid < n) store_group(Sk, o.x, o.y, tid, gx, q, planes);
-    for (int g = tid + kThreads; g < n; g += kThreads)
-      store_group(Sk, o.x, o.y, g, gx, load_group(Sk, o.x, o.y, g, gx), planes);
-    if (s + 1 < S) {  // the next sensor's samples, in flight during this one's sums
-      const LpaSensorK &Sn = L.s[s + 1];
-      o = box_origin(Sn, u0, v0, BH);
-      if (tid < (Sn.box_w >> 3) * Sn.box_h) q = load_group(Sn, o.x, o.y, tid, Sn.box_w >> 3);
+  for (int s0 = 0; s0 < S; s0 += L.mean_bufs) {
+    const int s1 = min(S, s0 + L.mean_bufs);
+    if (s0) __syncthreads();  // the buffers' readers have left them
+    int total = 0;
+    for (int s = s0; s < s1; s++) total += (L.s[s].box_w >> 3) * L.s[s].box_h;
+    auto fetch = [&](int k) {
+      int s = s0, n = (L.s[s0].box_w >> 3) * L.s[s0].box_h;
+      while (k >= n) k -= n, s++, n = (L.s[s].box_w >> 3) * L.s[s].box_h;
+      return load_group(L, s, k, u0, v0, BH);
+    };
+    auto put = [&](const Group &r) { store_group(L, r, reinterpret_cast<float2 *>(smem + (r.s - s0) * L.mean_plane)); };
+    for (int k = tid; k < total; k += 2 * kThreads) {  // two loads in flight per thread
+      const bool two = k + kThreads < total;
+      const Group a = fetch(k);
+      if (two) {
+        const Group b = fetch(k + kThreads);
+        put(a);
+        put(b);
+      } else {
+        put(a);
+      }
     }
-    __syncthreads();  // the planes are whole; the other buffer's readers have left it
+    __syncthreads();  // the planes (and the position tables) are whole
+#pragma unroll 1
+  for (int s = s0; s < s1; s++) {
+    const LpaSensorK &Sk = L.s[s];
+    const float2 *planes = reinterpret_cast<const float2 *>(smem + (s - s0) * L.mean_plane);
     const int PW = Sk.box_w >> 1, PP = PW * (Sk.box_h >> 1);
     if constexpr (FORM == kPeriodic) {
       const float *ex = xt + (s * (tx + ty) + col % tx) * T::kRow;
@@ -334,20 +360,34 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
       }
     }
   }
+  }
   if (u >= L.out_w) return;
-  const size_t plane = (size_t)L.out_w * L.out_h;
+  // per channel: a pointer to the first row's pixel and the step to the next
+  const size_t plane = (size_t)L.out_w * L.out_h, first = (size_t)(v0 + row0) * L.out_w + u;
+  const uint32_t next = (uint32_t)L.out_w * (FORM == kPeriodic ? ty : 1);
+  const int rows = v0 + row0 < y_end ? (y_end - v0 - row0 - 1) / (FORM == kPeriodic ? ty : 1) + 1 : 0;
 #pragma unroll
-  for (int k = 0; k < P; k++) {
-    const int v = v0 + row0 + (FORM == kPeriodic ? ty * k : k);
-    if (v >= y_end) return;
-    const size_t at = (size_t)v * L.out_w + u;
+  for (int c = 0; c < 3; c++) {
+    float val[P];
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
-      const bool has = acc[k][c].x > 0.f;
-      const float val = has ? __fdividef(acc[k][c].y, acc[k][c].x) : __int_as_float(0x7fffffff);
-      if (L.out_half) reinterpret_cast<__half *>(L.out)[c * plane + at] = __float2half_rn(val);
-      else reinterpret_cast<float *>(L.out)[c * plane + at] = val;
-      if (L.choice) L.choice[c * plane + at] = has ? 0 : 255;
+    for (int k = 0; k < P; k++)
+      val[k] = acc[k][c].x > 0.f ? __fdividef(acc[k][c].y, acc[k][c].x) : __int_as_float(0x7fffffff);
+    if (L.out_half) {
+      __half *o = reinterpret_cast<__half *>(L.out) + c * plane + first;
+#pragma unroll
+      for (int k = 0; k < P; k++, o += next)
+        if (k < rows) *o = __float2half_rn(val[k]);
+    } else {
+      float *o = reinterpret_cast<float *>(L.out) + c * plane + first;
+#pragma unroll
+      for (int k = 0; k < P; k++, o += next)
+        if (k < rows) *o = val[k];
+    }
+    if (L.choice) {
+      uint8_t *o = L.choice + c * plane + first;
+#pragma unroll
+      for (int k = 0; k < P; k++, o += next)
+        if (k < rows) *o = acc[k][c].x > 0.f ? 0 : 255;
     }
   }
 }
