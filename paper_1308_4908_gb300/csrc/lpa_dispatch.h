@@ -69,9 +69,11 @@ inline const void *lpa_kernel(int order, bool comp, bool diag, int mode, int til
 int lpa_mean_size(double reach_rb, double reach_g);
 int lpa_mean_cells(int size, bool green);
 uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors);
-// Its kernel (LPA_MEAN_THREADS threads), grid and launch over the tile rows of L's range.
+// The output rows of `count` unit tiles from tile0 on (whole tile rows) into L.
+void lpa_mean_rows(LpaLaunch &L, int tile0, int count);
+// Its kernel (LPA_MEAN_THREADS threads), grid and launch over those rows.
 const void *lpa_mean_kernel(const LpaLaunch &L);
-unsigned lpa_mean_grid(const LpaLaunch &L);
+dim3 lpa_mean_grid(const LpaLaunch &L);
 cudaError_t lpa_launch_mean(const LpaLaunch &L, cudaStream_t st);
 
 // Conversion of rows R of every sensor of L into its planes (LpaSensorK::conv), for a plan with

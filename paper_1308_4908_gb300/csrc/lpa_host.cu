@@ -323,7 +323,8 @@ struct MeanPlan {
 // per pixel), fewer for smaller frames (more CTAs).
 MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   MeanPlan m;
-  if (p->order != 0 || p->n_scales != 1 || p->accum != 0 || p->weight_mode != 0 || !(p->min_pivot < 0.99) ||
+  // (its grid has a row of tiles per y index: at most 65535 of 8 rows)
+  if (p->out_h > 65535 * 8 || p->order != 0 || p->n_scales != 1 || p->accum != 0 || p->weight_mode != 0 || !(p->min_pivot < 0.99) ||
       !(p->cond_fallback <= 0.0 || p->cond_fallback >= 1.0))
     return m;
   m.rb = p->trunc_k * p->sigma[0];
@@ -743,8 +744,9 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     L.mean_p = mean.p;
     L.mean_size = mean.size;
     L.mean_axis = mean.axis ? 1 : 0;
-    L.mean_tx = mean.tx;
-    L.mean_ty = mean.ty;
+    L.mean_lx = mean.tx / 2;  // 2 or 4 pixels
+    L.mean_ly = mean.ty / 2;
+    if (L.tiles_x > 0 && L.tiles_y > 0) lpa_mean_rows(L, 0, L.tiles_x * L.tiles_y);
     L.stages = 1;
     return HDR_OK;
   }
@@ -1246,6 +1248,7 @@ hdr_status hdr_reconstruct_host(hdr_ctx *ctx, int32_t rig_id, const hdr_params *
     L.tile0 = r0 * L.tiles_x;
     L.tile_count = (r1 - r0) * L.tiles_x;
     if (L.tile_count > 0) {
+      if (L.mode == LPA_MEAN) lpa_mean_rows(L, L.tile0, L.tile_count);
       st = launch(L, params->accum, false, sb);
       if (st) return st;
     }
@@ -1548,7 +1551,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       return fail(HDR_E_INVALID, "frame %d: tile range [%d, %d) outside [0, %d)", f, ranges[f].x, ranges[f].y, nt);
     plans[f].tile0 = ranges ? ranges[f].x : 0;
     grid[f] = ranges ? ranges[f].y - ranges[f].x : nt;
-    if (plans[f].mode == LPA_MEAN) plans[f].tile_count = grid[f];
+    if (plans[f].mode == LPA_MEAN && grid[f] > 0) lpa_mean_rows(plans[f], plans[f].tile0, grid[f]);
   }
   std::vector<int> order;
   for (int f = 0; f < n; f++)
@@ -1594,12 +1597,12 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 128 * (L.mean_tx != 0) : L.px,
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 128 * (L.mean_lx != 0) : L.px,
                    L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};
     r.func = const_cast<void *>(fn);
-    r.gridDim = dim3(mean ? lpa_mean_grid(L) : (unsigned)lpa_grid_ctas(grid[f], L.stages));
+    r.gridDim = mean ? lpa_mean_grid(L) : dim3((unsigned)lpa_grid_ctas(grid[f], L.stages));
     r.blockDim = dim3(mean ? (unsigned)LPA_MEAN_THREADS : (unsigned)(LPA_TILE * L.tile_h / L.px));
     r.sharedMemBytes = L.smem_bytes;
     r.kernelParams = args.back().data();

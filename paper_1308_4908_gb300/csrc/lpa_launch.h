@@ -103,19 +103,12 @@ struct LpaLaunch {
   float *aux;
   // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, whether every sensor's axes are
   // parallel to the output's, the pixels that span one cell of a colour phase where that is exact for
-  // every sensor (2 or 4 on each axis, else both 0), sensors staged at a time, bytes of one sensor's
+  // every sensor (as powers of two, 1 or 2 on each axis, else both 0), sensors staged at a time, bytes of one sensor's
   // colour-phase planes (from offset 0) and the offset of the position tables
-  int mean_p, mean_size, mean_axis, mean_tx, mean_ty, mean_bufs;
+  int mean_p, mean_size, mean_axis, mean_lx, mean_ly, mean_bufs;
+  int mean_y0, mean_y1;          // output rows of the launch (lpa_mean_rows)
   uint32_t mean_plane, mean_tab;
 };
-
-// Output rows [first, end) of a launch's unit tiles (whole tile rows).
-__host__ __device__ inline int lpa_first_row(const LpaLaunch &L) { return L.tile0 / L.tiles_x * L.tile_h; }
-__host__ __device__ inline int lpa_end_row(const LpaLaunch &L) {
-  const int count = L.tile_count > 0 ? L.tile_count : L.tiles_x * L.tiles_y - L.tile0;
-  const int end = ((L.tile0 + count - 1) / L.tiles_x + 1) * L.tile_h;
-  return end < L.out_h ? end : L.out_h;
-}
 
 // LPA_SEARCHED_F32, LPA_STEERED_F32, LPA_TABULATED_F32: the searched, steered or tabulated window
 // with every fit solved in FP32 only, for parameters under which the FP64 re-solve can never

@@ -101,14 +101,31 @@ __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, 
   const uint32_t w[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
   float4 *even = reinterpret_cast<float4 *>(planes + 2 * (r.row & 1) * PP + (r.row >> 1) * PW + 4 * r.col);
   float4 *odd = even + (PP >> 1);
-  float2 v[8];
+  float2 v[8];  // (1 / s2, f / s2)
+  if (scalar) {  // convert_sample's arithmetic, two samples at a time
 #pragma unroll
-  for (int k = 0; k < 8; k++) {
-    const uint32_t y = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
-    v[k] = make_float2(0.f, 0.f);
-    if (k < n) {
-      const float2 fv = convert_sample<false>(S, scalar, r.X + k, r.Y, (float)y);  // (f, 1 / s2)
-      v[k] = make_float2(fv.y, fv.y * fv.x);
+    for (int k = 0; k < 4; k++) {
+      const float y0 = (float)(w[k] & 0xffffu), y1 = (float)(w[k] >> 16);
+      const float2 e = __fadd2_rn(make_float2(y0, y1), make_float2(-S.black, -S.black));
+      const float2 f = __fmul2_rn(e, make_float2(S.inv_gtn, S.inv_gtn));
+      const float2 d = __ffma2_rn(make_float2(S.gain, S.gain), make_float2(fmaxf(e.x, 0.f), fmaxf(e.y, 0.f)),
+                                  make_float2(S.read_var, S.read_var));
+      float2 iv = make_float2(__fdividef(S.gtn2, d.x), __fdividef(S.gtn2, d.y));
+      iv.x = y0 < S.sat && 2 * k < n ? iv.x : 0.f;
+      iv.y = y1 < S.sat && 2 * k + 1 < n ? iv.y : 0.f;
+      const float2 ivf = __fmul2_rn(iv, f);
+      v[2 * k] = make_float2(iv.x, ivf.x);
+      v[2 * k + 1] = make_float2(iv.y, ivf.y);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const uint32_t y = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
+      v[k] = make_float2(0.f, 0.f);
+      if (k < n) {
+        const float2 fv = convert_sample<false>(S, scalar, r.X + k, r.Y, (float)y);  // (f, 1 / s2)
+        v[k] = make_float2(fv.y, fv.y * fv.x);
+      }
     }
   }
   even[0] = make_float4(v[0].x, v[0].y, v[2].x, v[2].y);
@@ -159,9 +176,8 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
   if (*reinterpret_cast<volatile unsigned int *>(L.status) & LPA_ERR_TIMEOUT) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, S = L.n_sensors;
-  const int nbx = (L.out_w + kBW - 1) / kBW;
-  const int y_first = lpa_first_row(L), y_end = lpa_end_row(L);
-  const int u0 = (int)(blockIdx.x % nbx) * kBW, v0 = y_first + (int)(blockIdx.x / nbx) * BH;
+  const int y_end = L.mean_y1;
+  const int u0 = (int)blockIdx.x * kBW, v0 = L.mean_y0 + (int)blockIdx.y * BH;
   const float log2e = 1.4426950408889634f;
   const float sg[2] = {L.sigma[0], L.sigma[0] * L.green_ratio};
 
@@ -169,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
   float *xt = reinterpret_cast<float *>(smem + L.mean_tab);
   float *yt = xt + S * T::kWords * kBW;
   int4 *anchor = reinterpret_cast<int4 *>(smem + L.mean_tab);
-  const int tx = L.mean_tx, ty = L.mean_ty;
+  const int lx = L.mean_lx, ly = L.mean_ly, tx = 1 << lx, ty = 1 << ly;  // kPeriodic: pixels to a cell
   if constexpr (FORM == kPeriodic) {
     // one entry per sensor, axis and class of positions: class c starts at G c + G_t, and the n-th
     // pixel of a class lies exactly 2 n px further, whatever the tile
@@ -180,9 +196,9 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
       const LpaSensorK &Sk = L.s[s];
       const int2 o = box_origin(Sk, u0, v0, BH);
       const double q = fmin(fmax(col ? Sk.G[0] * c + Sk.G[2] : Sk.G[4] * c + Sk.G[5], -LPA_FAR), LPA_FAR), fl = floor(q);
-      const int l = (int)fl + (col ? 2 * (u0 / tx) - o.x : 2 * (v0 / ty) - o.y);
+      const int l = (int)fl + (col ? 2 * (u0 >> lx) - o.x : 2 * (v0 >> ly) - o.y);
       float *t = xt + tid * T::kRow;
-      const int last = col ? (kBW - 1) / tx : (BH - 1) / ty;
+      const int last = col ? (kBW - 1) >> lx : (BH - 1) >> ly;
       if (!axis_entry<NR, NG>(L, Sk, col, l, (float)(q - fl), last, t, 1) && (col ? u0 + c < L.out_w : v0 + c < y_end) && fabs(q) < 1e6)
         atomicOr(L.status, LPA_ERR_BOUNDS);
     }
@@ -216,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
 
   // this thread's column and its P rows: row0 + k, or (kPeriodic) row0 + ty k
   const int col = (tid & 31) + 32 * ((tid >> 5) & 1), group = tid >> 6;
-  const int row0 = FORM == kPeriodic ? group / ty * (ty * P) + group % ty : group * P;
+  const int row0 = FORM == kPeriodic ? (group >> ly) * (P << ly) + (group & (ty - 1)) : group * P;
   const int u = u0 + col;
   float2 acc[P][3];  // per row and channel: (sum K / s2, sum K f / s2)
 #pragma unroll
@@ -255,9 +271,9 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
     const float2 *planes = reinterpret_cast<const float2 *>(smem + (s - s0) * L.mean_plane);
     const int PW = Sk.box_w >> 1, PP = PW * (Sk.box_h >> 1);
     if constexpr (FORM == kPeriodic) {
-      const float *ex = xt + (s * (tx + ty) + col % tx) * T::kRow;
-      const float *ey = xt + (s * (tx + ty) + tx + group % ty) * T::kRow;
-      const int shift = col / tx + group / ty * P * PW;  // whole cells from the class's first pixel
+      const float *ex = xt + (s * (tx + ty) + (col & (tx - 1))) * T::kRow;
+      const float *ey = xt + (s * (tx + ty) + tx + (group & (ty - 1))) * T::kRow;
+      const int shift = (col >> lx) + (group >> ly) * P * PW;  // whole cells from the class's first pixel
       auto phase = [&](auto N_, auto c_, int ox, int oy, int g) {
         constexpr int N = decltype(N_)::value, c = decltype(c_)::value;
         const float *fx = ex + 4 + 2 * NR * g + N * ox, *fy = ey + 4 + 2 * NR * g + N * oy;
@@ -364,8 +380,9 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
   if (u >= L.out_w) return;
   // per channel: a pointer to the first row's pixel and the step to the next
   const size_t plane = (size_t)L.out_w * L.out_h, first = (size_t)(v0 + row0) * L.out_w + u;
-  const uint32_t next = (uint32_t)L.out_w * (FORM == kPeriodic ? ty : 1);
-  const int rows = v0 + row0 < y_end ? (y_end - v0 - row0 - 1) / (FORM == kPeriodic ? ty : 1) + 1 : 0;
+  const int step = FORM == kPeriodic ? ly : 0;
+  const uint32_t next = (uint32_t)L.out_w << step;
+  const int rows = v0 + row0 < y_end ? ((y_end - v0 - row0 - 1) >> step) + 1 : 0;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     float val[P];
@@ -400,7 +417,7 @@ const void *pick(int p) {
 }
 template <int NR, int NG>
 const void *pick(const LpaLaunch &L) {
-  return L.mean_tx     ? pick<NR, NG, kPeriodic>(L.mean_p)
+  return L.mean_lx     ? pick<NR, NG, kPeriodic>(L.mean_p)
          : L.mean_axis ? pick<NR, NG, kAxis>(L.mean_p)
                        : pick<NR, NG, kGeneral>(L.mean_p);
 }
@@ -421,14 +438,19 @@ uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_senso
   return (uint32_t)(n_sensors * 4 * (words * lpa::kBW + row * 8 * p));
 }
 const void *lpa_mean_kernel(const LpaLaunch &L) { return L.mean_size == 0 ? lpa::pick<3, 2>(L) : lpa::pick<4, 3>(L); }
-unsigned lpa_mean_grid(const LpaLaunch &L) {
-  const long rows = lpa_end_row(L) - lpa_first_row(L), bh = 8 * L.mean_p;
-  return (unsigned)((L.out_w + lpa::kBW - 1) / lpa::kBW * ((rows + bh - 1) / bh));
+dim3 lpa_mean_grid(const LpaLaunch &L) {
+  const int bh = 8 * L.mean_p;
+  return dim3((unsigned)((L.out_w + lpa::kBW - 1) / lpa::kBW), (unsigned)((L.mean_y1 - L.mean_y0 + bh - 1) / bh));
+}
+void lpa_mean_rows(LpaLaunch &L, int tile0, int count) {
+  L.mean_y0 = tile0 / L.tiles_x * L.tile_h;
+  L.mean_y1 = ((tile0 + count - 1) / L.tiles_x + 1) * L.tile_h;
+  if (L.mean_y1 > L.out_h) L.mean_y1 = L.out_h;
 }
 cudaError_t lpa_launch_mean(const LpaLaunch &L, cudaStream_t st) {
   const void *fn = lpa_mean_kernel(L);
   cudaError_t e = lpa_opt_in(fn);
   if (e != cudaSuccess) return e;
   void *args[] = {const_cast<LpaLaunch *>(&L)};
-  return cudaLaunchKernel(fn, dim3(lpa_mean_grid(L)), dim3(LPA_MEAN_THREADS), args, L.smem_bytes, st);
+  return cudaLaunchKernel(fn, lpa_mean_grid(L), dim3(LPA_MEAN_THREADS), args, L.smem_bytes, st);
 }
