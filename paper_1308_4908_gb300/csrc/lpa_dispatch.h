@@ -71,7 +71,7 @@ int lpa_mean_cells(int size, bool green);
 uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors);
 // The output rows of `count` unit tiles from tile0 on (whole tile rows) into L.
 void lpa_mean_rows(LpaLaunch &L, int tile0, int count);
-// Its kernel (LPA_MEAN_THREADS threads), grid and launch over those rows.
+// Its kernel (lpa_mean_threads(L.mean_p) threads), grid and launch over those rows.
 const void *lpa_mean_kernel(const LpaLaunch &L);
 dim3 lpa_mean_grid(const LpaLaunch &L);
 cudaError_t lpa_launch_mean(const LpaLaunch &L, cudaStream_t st);

@@ -319,8 +319,8 @@ struct MeanPlan {
 // windows of at most 4 x 4 (R, B) and 3 x 3 (G) cells of a colour phase. A fit of one unknown has the
 // equilibrated pivot 1, so it is usable with any sample (min_pivot below 1) and never solved again
 // in FP64 (cond_fallback at least 1, or none); other parameters keep the general kernel.
-// Rows per thread: four once 64 x 32 tiles fill the SMs' two resident CTAs twice (less halo converted
-// per pixel), fewer for smaller frames (more CTAs).
+// Rows per thread: four, or eight of half as many threads in the periodic form, once 64 x 32 tiles fill
+// the SMs' two resident CTAs twice (less halo converted per pixel), fewer for smaller frames (more CTAs).
 MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   MeanPlan m;
   // (its grid has a row of tiles per y index: at most 65535 of 8 rows)
@@ -347,7 +347,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   if (!m.axis || !m.tx || !m.ty) m.tx = m.ty = 0;
   m.size = lpa_mean_size(m.rb * most + 2e-3, m.g * most + 2e-3);
   const long long px = (long long)p->out_w * p->out_h;
-  m.p = px >= 4LL * 152 * 64 * 32 ? 4 : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
+  m.p = px >= 4LL * 152 * 64 * 32 ? (m.tx ? 8 : 4) : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
   return m;
 }
 
@@ -356,7 +356,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
 // the alignment of its origin (x to 8, y to 2).
 void mean_box(const MeanPlan &m, const double G[6], double hxu, double hyu, int *bw, int *bh, float *ext_x, float *ext_y) {
   const int nr = lpa_mean_cells(m.size, false), ng = lpa_mean_cells(m.size, true);
-  const double w = LPA_MEAN_TILE_W - 1, h = 8 * m.p - 1;
+  const double w = LPA_MEAN_TILE_W - 1, h = lpa_mean_tile_h(m.p) - 1;
   auto sides = [&](double unit, float *ext) {
     const double rb = m.rb * unit + 2e-3, g = m.g * unit + 2e-3;
     *ext = (float)(std::max(rb, g) + 1.0);
@@ -367,7 +367,7 @@ void mean_box(const MeanPlan &m, const double G[6], double hxu, double hyu, int 
 }
 
 // lpa_mean's shared memory for a rig: planes of the largest box for *bufs sensors (all, or as many as
-// leave two CTAs on an SM), then the tables; 0 where not even one sensor's fit.
+// leave two CTAs of 512 threads or three of 256 on an SM), then the tables; 0 where not even one sensor's fit.
 uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *bufs, uint32_t *plane, uint32_t *tab) {
   double need = 0.0;
   for (int s = 0; s < rig.n; s++) {
@@ -380,7 +380,7 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *
     mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);
     need = std::max(need, 8.0 * bw * bh);
   }
-  const double tables = lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n), room = 110.0 * 1024 - tables;
+  const double tables = lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n), room = (m.p == 8 ? 73.0 : 110.0) * 1024 - tables;
   if (need > room) return 0;
   *bufs = std::min(rig.n, (int)(room / need));
   *plane = (uint32_t)need;
@@ -1603,7 +1603,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
     cudaKernelNodeParams r{};
     r.func = const_cast<void *>(fn);
     r.gridDim = mean ? lpa_mean_grid(L) : dim3((unsigned)lpa_grid_ctas(grid[f], L.stages));
-    r.blockDim = dim3(mean ? (unsigned)LPA_MEAN_THREADS : (unsigned)(LPA_TILE * L.tile_h / L.px));
+    r.blockDim = dim3(mean ? (unsigned)lpa_mean_threads(L.mean_p) : (unsigned)(LPA_TILE * L.tile_h / L.px));
     r.sharedMemBytes = L.smem_bytes;
     r.kernelParams = args.back().data();
     kp.push_back(r);

@@ -9,13 +9,16 @@
 #define LPA_TILE 16         // output tile width in pixels; the height TH is 8 or 16 (one thread per pixel)
 #define LPA_ANCHOR 8        // edge of the output blocks whose sensor positions are anchored in FP64
 #define LPA_MARGIN 4        // staging margin in sensor px around every window box
-#define LPA_MEAN_THREADS 512
 #define LPA_MEAN_TILE_W 64
 #define LPA_STAGED_TILES 4  // tiles per CTA of the single-frame kernel with two staging buffers
 
 // Device status word bits (read and cleared by hdr_check).
 #define LPA_ERR_TIMEOUT 1u  // a bounded mbarrier wait ran out
 #define LPA_ERR_BOUNDS 2u   // a window row fell outside the staged footprint
+
+// lpa_mean with P output rows per thread: threads per CTA and rows of its tiles.
+__host__ __device__ constexpr int lpa_mean_threads(int p) { return p == 8 ? 256 : 512; }
+__host__ __device__ constexpr int lpa_mean_tile_h(int p) { return lpa_mean_threads(p) / LPA_MEAN_TILE_W * p; }
 
 struct alignas(64) LpaSensorK {
   CUtensorMap tmap;         // 2-D tiled map of the raw frame (uint16, dims width x height)

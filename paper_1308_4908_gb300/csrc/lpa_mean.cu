@@ -7,7 +7,9 @@
 // the window can hold), so the loops unroll, and a cell outside the window needs no test: its value
 // exp(-r^2 / 2 sigma^2) - exp(-k^2 / 2) (Eq. 8) is not positive there and is cut at 0.
 //
-// A CTA of 512 threads reconstructs 64 x 8 P pixels, P rows per thread; lanes are consecutive
+// A CTA of 512 threads reconstructs 64 x 8 P pixels, P rows per thread (kPeriodic on large frames: 256
+// threads, P = 8, so that each cell and factor serves twice the rows: 187 -> 152 us enlarging 2 x 2048^2 twofold,
+// 100 -> 93 us on the camera frame; three CTAs per SM, at two 173 and 96 us, at four 160 and 98 us); lanes are consecutive
 // pixels of a row, so stores coalesce and neighbours read the same cells. The raw footprints of all sensors
 // (of as many as two CTAs' shared memory holds) are read straight from global memory (16-byte loads,
 // two in flight per thread) and converted once per sample (Eqs. 18 and 20) into colour-phase planes of
@@ -15,7 +17,7 @@
 // then one shared load and one paired FMA into (sum K / s2, sum K f / s2). No conversion pass goes
 // ahead of the kernel: with 64 x 32 tiles a sample is converted about 1.5 times, and the pass cost
 // 47 us of 517 on four 2336 x 1752 sensors. Measured against the general kernel with that pass: 2 x 2048^2 ->
-// 4096^2 FP16 1226 -> 303 us, the four sensors (tabulated windows before) 517 -> 172 us, 64^2 14.4 -> 10.3 us a call;
+// 4096^2 FP16 1226 -> 152 us, the four sensors (tabulated windows before) 517 -> 93 us, 64^2 14.4 -> 10.3 us a call;
 // 1024 x 900, three rotated sensors 147 -> 78 us.
 //
 // kAxis: every sensor's axes are parallel to the output's, so the Gaussian factors into a column and
@@ -37,7 +39,6 @@
 namespace lpa {
 namespace {
 
-constexpr int kThreads = LPA_MEAN_THREADS;
 constexpr int kBW = LPA_MEAN_TILE_W;
 
 // First candidate cell of a window along one axis of one colour phase: the position is cell `l` (from
@@ -170,9 +171,9 @@ __device__ __forceinline__ bool axis_entry(const LpaLaunch &L, const LpaSensorK 
 }
 
 template <int NR, int NG, int FORM, int P>
-__global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ LpaLaunch L) {
+__global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(const __grid_constant__ LpaLaunch L) {
   using T = Layout<NR, NG>;
-  constexpr int BH = 8 * P;
+  constexpr int kThreads = lpa_mean_threads(P), BH = lpa_mean_tile_h(P);
   if (*reinterpret_cast<volatile unsigned int *>(L.status) & LPA_ERR_TIMEOUT) return;
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, S = L.n_sensors;
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
         atomicOr(L.status, LPA_ERR_BOUNDS);
     }
   } else {
-    constexpr int NA = 8 * P;  // 8 x 8 blocks of the tile
+    constexpr int NA = BH;  // 8 x 8 blocks of the tile
     for (int k = tid; k < S * NA; k += kThreads) {
       const int s = k / NA, b = k - s * NA;
       const LpaSensorK &Sk = L.s[s];
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_mean(const __grid_constant__ 
 #pragma unroll
       for (int k = 0; k < P; k++) {
         const int row = row0 + k;
-        const int4 an = anchor[s * 8 * P + (row >> 3) * 8 + (col >> 3)];
+        const int4 an = anchor[s * BH + (row >> 3) * 8 + (col >> 3)];
         const float du = (float)(col & 7), dv = (float)(row & 7);
         const float px = __int_as_float(an.z) + du * Sk.Gf[0] + dv * Sk.Gf[1];
         const float py = __int_as_float(an.w) + du * Sk.Gf[2] + dv * Sk.Gf[3];
@@ -413,6 +414,7 @@ template <int NR, int NG, int FORM>
 const void *pick(int p) {
   return p == 1   ? (const void *)lpa_mean<NR, NG, FORM, 1>
          : p == 2 ? (const void *)lpa_mean<NR, NG, FORM, 2>
+         : p == 8 && FORM == kPeriodic ? (const void *)lpa_mean<NR, NG, kPeriodic, 8>
                   : (const void *)lpa_mean<NR, NG, FORM, 4>;
 }
 template <int NR, int NG>
@@ -431,15 +433,15 @@ int lpa_mean_size(double reach_rb, double reach_g) {
 }
 int lpa_mean_cells(int size, bool green) { return size == 0 ? (green ? 2 : 3) : (green ? 3 : 4); }
 uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors) {
-  if (!axis) return (uint32_t)(n_sensors * 8 * p * 16);
+  if (!axis) return (uint32_t)(n_sensors * lpa_mean_tile_h(p) * 16);
   const int words = size == 0 ? lpa::Layout<3, 2>::kWords : lpa::Layout<4, 3>::kWords;
   const int row = size == 0 ? lpa::Layout<3, 2>::kRow : lpa::Layout<4, 3>::kRow;
   if (classes) return (uint32_t)(n_sensors * 4 * row * classes);
-  return (uint32_t)(n_sensors * 4 * (words * lpa::kBW + row * 8 * p));
+  return (uint32_t)(n_sensors * 4 * (words * lpa::kBW + row * lpa_mean_tile_h(p)));
 }
 const void *lpa_mean_kernel(const LpaLaunch &L) { return L.mean_size == 0 ? lpa::pick<3, 2>(L) : lpa::pick<4, 3>(L); }
 dim3 lpa_mean_grid(const LpaLaunch &L) {
-  const int bh = 8 * L.mean_p;
+  const int bh = lpa_mean_tile_h(L.mean_p);
   return dim3((unsigned)((L.out_w + lpa::kBW - 1) / lpa::kBW), (unsigned)((L.mean_y1 - L.mean_y0 + bh - 1) / bh));
 }
 void lpa_mean_rows(LpaLaunch &L, int tile0, int count) {
@@ -452,5 +454,5 @@ cudaError_t lpa_launch_mean(const LpaLaunch &L, cudaStream_t st) {
   cudaError_t e = lpa_opt_in(fn);
   if (e != cudaSuccess) return e;
   void *args[] = {const_cast<LpaLaunch *>(&L)};
-  return cudaLaunchKernel(fn, lpa_mean_grid(L), dim3(LPA_MEAN_THREADS), args, L.smem_bytes, st);
+  return cudaLaunchKernel(fn, lpa_mean_grid(L), dim3((unsigned)lpa_mean_threads(L.mean_p)), args, L.smem_bytes, st);
 }
