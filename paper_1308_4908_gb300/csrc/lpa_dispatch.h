@@ -66,6 +66,7 @@ inline const void *lpa_kernel(int order, bool comp, bool diag, int mode, int til
 // Order 0 with one window scale (LPA_MEAN). The kernel template for windows that reach reach_rb (R, B) and
 // reach_g (G) sensor px, -1 if they hold more cells than any is built for; its candidate cells per
 // axis; bytes of its position tables for p rows per thread (classes: periodic positions, both axes' classes).
+// (sizes 2 and 3 are lpa_grad's: 3 and 4 cells)
 int lpa_mean_size(double reach_rb, double reach_g);
 int lpa_mean_cells(int size, bool green);
 uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors);
@@ -75,6 +76,10 @@ void lpa_mean_rows(LpaLaunch &L, int tile0, int count);
 const void *lpa_mean_kernel(const LpaLaunch &L);
 dim3 lpa_mean_grid(const LpaLaunch &L);
 cudaError_t lpa_launch_mean(const LpaLaunch &L, cudaStream_t st);
+
+// The gradient pass of small windows (lpa_grad.cu), for a plan with mean_size 2 or 3; f64: with the FP64
+// re-solve.
+cudaError_t lpa_launch_grad(const LpaLaunch &L, bool f64, cudaStream_t st);
 
 // Conversion of rows R of every sensor of L into its planes (LpaSensorK::conv), for a plan with
 // conv = 1; lit: the printed noise weight (square root of the inverse variance).

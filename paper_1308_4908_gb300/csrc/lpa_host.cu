@@ -286,6 +286,7 @@ struct PlanEnv {
   bool single = true;  // frames with one scale may leave the variance sums out (LPA_ONE)
   bool mean = true;    // small windows of order 0 may run lpa_mean (not the level maps, whose kernel also
                        // writes Var C_0, nor the persistent batch kernels)
+  bool grad = false;   // the gradient pass: lpa_grad where its windows are small enough
 };
 
 bool is_identity_linear(const double *a) {
@@ -351,6 +352,25 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   return m;
 }
 
+// Whether the gradient pass of these parameters (order 1, one scale) runs lpa_grad: plain sums and green
+// windows of at most 4 x 4 cells. Two rows per thread once 64 x 16 tiles fill the SMs twice.
+MeanPlan grad_plan(const Rig &rig, const hdr_params *p) {
+  MeanPlan m;
+  m.axis = false;
+  m.rb = m.g = p->trunc_k * p->sigma[0] * p->green_ratio;
+  if (p->accum != 0 || p->out_h > 65535 * 8) return m;
+  double most = 0.0;
+  for (int s = 0; s < rig.n; s++) {
+    double t[6];
+    invert_affine(rig.s[s].d.affine, t);
+    most = std::max(most, std::max(std::hypot(t[0], t[1]), std::hypot(t[3], t[4])));
+  }
+  const double cells = std::floor(m.g * most + 2e-3) + 1;
+  m.size = cells <= 3 ? 2 : cells <= 4 ? 3 : -1;
+  m.p = (long long)p->out_w * p->out_h >= 4LL * 152 * 64 * 16 ? 2 : 1;
+  return m;
+}
+
 // Staging box of lpa_mean for sensor transform G: the tile's points, `left` px before the first one (the
 // window's reach) and up to the last candidate cell after the last, one px of margin on each side, and
 // the alignment of its origin (x to 8, y to 2).
@@ -378,7 +398,7 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *
     int bw, bh;
     float ex, ey;
     mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);
-    need = std::max(need, 8.0 * bw * bh);
+    need = std::max(need, (m.size >= 2 ? 4.0 : 8.0) * bw * bh);  // lpa_grad keeps the green half
   }
   const double tables = lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n), room = (m.p == 8 ? 73.0 : 110.0) * 1024 - tables;
   if (need > room) return 0;
@@ -616,11 +636,13 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   size_t conv_off = 0;
   MeanPlan mean;
   if (env.mean) mean = mean_plan(rig, p);
+  if (env.grad) mean = grad_plan(rig, p);
   if (mean.size >= 0) {
     L.smem_bytes = mean_smem(rig, p, mean, &L.mean_bufs, &L.mean_plane, &L.mean_tab);
-    if (L.smem_bytes == 0) mean.size = -1;
+    // (lpa_grad stages every sensor at once)
+    if (L.smem_bytes == 0 || (env.grad && L.mean_bufs < rig.n)) mean.size = -1;
   }
-  if (mean.size >= 0) conv = nullptr;  // lpa_mean reads the raw frames
+  if (mean.size >= 0) conv = nullptr;  // lpa_mean and lpa_grad read the raw frames
   L.conv = conv ? 1 : 0;
   for (int s = 0; s < rig.n; s++) {
     const hdr_sensor_desc &d = rig.s[s].d;
@@ -739,8 +761,16 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
       }
     }
   }
+  // the pixel steps that span two sensor px of the first sensor (the others differ by their slight
+  // misalignment); beyond 4 (enlargements over 2.25 times) neighbours differ little: as at 1x
+  auto stride = [](double step) {
+    const double n = std::round(2.0 / step);
+    return n >= 1.0 && n <= 4.0 ? (int)n : n < 1.0 ? 1 : 2;
+  };
+  const double *G0 = L.s[0].G;
+  L.px_map = 4 * (stride(std::hypot(G0[1], G0[4])) - 1) + stride(std::hypot(G0[0], G0[3])) - 1;
   if (mean.size >= 0) {
-    L.mode = LPA_MEAN;
+    L.mode = env.grad ? LPA_GRADIENTS : LPA_MEAN;
     L.mean_p = mean.p;
     L.mean_size = mean.size;
     L.mean_axis = mean.axis ? 1 : 0;
@@ -751,14 +781,6 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     return HDR_OK;
   }
   L.tx_bytes = tx;
-  // the pixel steps that span two sensor px of the first sensor (the others differ by their slight
-  // misalignment); beyond 4 (enlargements over 2.25 times) neighbours differ little: as at 1x
-  auto stride = [](double step) {
-    const double n = std::round(2.0 / step);
-    return n >= 1.0 && n <= 4.0 ? (int)n : n < 1.0 ? 1 : 2;
-  };
-  const double *G0 = L.s[0].G;
-  L.px_map = 4 * (stride(std::hypot(G0[1], G0[4])) - 1) + stride(std::hypot(G0[0], G0[3])) - 1;
   // a usable fit's equilibrated pivots lie in (min_pivot, 1]: when min_pivot * cond_fallback >= 2
   // their spread never exceeds cond_fallback and the FP64 re-solve cannot trigger
   const bool f64_possible = p->cond_fallback > 0.0 && (p->min_pivot - 1e-4) * p->cond_fallback < 2.0;
@@ -801,8 +823,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
 }
 
 hdr_status plan(hdr_ctx *ctx, const Rig &rig, const hdr_params *p, const uint16_t *const *raw, LpaLaunch &L,
-                double reach = 1.0, bool levels = false, int stages = 1, float2 *conv = nullptr) {
-  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels, !levels}, rig, p, raw, L,
+                double reach = 1.0, bool levels = false, int stages = 1, float2 *conv = nullptr, bool grad = false) {
+  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels, !levels, grad}, rig, p, raw, L,
                   LPA_FRAME_TILE_H, reach, stages, conv);
 }
 
@@ -1812,14 +1834,30 @@ hdr_status lpa_launch_mode(hdr_ctx *ctx, int32_t rig_id, const hdr_params *param
     return fail(HDR_E_UNSUPPORTED, "the adaptive passes use the inverse-variance weight (weight_mode 0)");
   hdr_params p = *params;
   p.tab_weights = 0;  // the window is searched: offsets or weights differ per pixel
+  LpaLaunch L;
+  const Rig &rig = ctx->rigs[rig_id];
+  if (mode == LPA_GRADIENTS) {
+    uint32_t plane, tab;
+    int bufs = 0;
+    const MeanPlan m = grad_plan(rig, &p);
+    if (m.size >= 0 && mean_smem(rig, &p, m, &bufs, &plane, &tab) > 0 && bufs == rig.n) {
+      s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, nullptr, true);
+      if (s) return s;
+      if (L.out_w == 0 || L.out_h == 0) return HDR_OK;
+      L.aux = aux;
+      const bool f64 = p.cond_fallback > 0.0 && (p.min_pivot - 1e-4) * p.cond_fallback < 2.0;
+      cudaError_t e = lpa_launch_grad(L, f64, st);
+      if (e != cudaSuccess) return fail(HDR_E_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+      return HDR_OK;
+    }
+  }
   float2 *conv = nullptr;
   if (ahead) {
-    s = conv_buffer(ctx, ctx->rigs[rig_id], &p, true, &conv);
+    s = conv_buffer(ctx, rig, &p, true, &conv);
     if (s) return s;
   }
-  LpaLaunch L;
   // (planned as for the level maps: the kernel of `mode` is the general one, with its variance sums)
-  s = plan(ctx, ctx->rigs[rig_id], &p, raw_dev, L, reach, true, 1, conv);
+  s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, conv);
   if (s) return s;
   if (L.conv) {  // the frame converted once, then the pass
     s = convert_rows(ctx, L, all_rows(L), true, st);

@@ -33,28 +33,11 @@
 
 #include "lpa_dispatch.h"
 #include "lpa_launch.h"
-#include "lpa_convert.cuh"
 #include "lpa_ptx.cuh"
+#include "lpa_tile.cuh"
 
 namespace lpa {
 namespace {
-
-constexpr int kBW = LPA_MEAN_TILE_W;
-
-// First candidate cell of a window along one axis of one colour phase: the position is cell `l` (from
-// the box origin, even) plus fraction f; the window reaches h (m = floor(h / 2)). Returns the
-// lattice index (cell o + 2 i) and its offset from the position.
-__device__ __forceinline__ int first_cell(int l, float f, int o, float h, float m, float &delta) {
-  const int e = l - o;
-  const float r = (e & 1) ? f + 1.f : f;             // position from the even lattice cell below, in [0, 2)
-  const float n = (h - r) * 0.5f < m ? m - 1.f : m;  // floor((h - r) / 2)
-  delta = -2.f * n - r;
-  return (e >> 1) - (int)n;
-}
-
-struct Window {
-  float h, m;  // reach in sensor px and floor(reach / 2)
-};
 
 template <int NR, int NG>
 struct Layout {
@@ -62,37 +45,6 @@ struct Layout {
   static constexpr int kWords = 4 + kE;          // four first cells, then the factors
   static constexpr int kRow = (kWords + 3) / 4 * 4;
 };
-
-// A group of eight columns of one row of a sensor's box: where it lies and its raw samples, zeros off the frame.
-struct Group {
-  int s, row, col, X, Y;
-  uint4 q;
-};
-
-// Box origin of a tile in sensor s: x on a multiple of 8 (16-byte loads), y even. FP32 is enough
-// (the box has a margin of a pixel), and every thread forms the same value.
-__device__ __forceinline__ int2 box_origin(const LpaSensorK &S, int u0, int v0, int bh) {
-  float x = S.Gf[0] * (float)(S.Gf[0] < 0.f ? u0 + kBW - 1 : u0) + S.Gf[1] * (float)(S.Gf[1] < 0.f ? v0 + bh - 1 : v0);
-  float y = S.Gf[2] * (float)(S.Gf[2] < 0.f ? u0 + kBW - 1 : u0) + S.Gf[3] * (float)(S.Gf[3] < 0.f ? v0 + bh - 1 : v0);
-  x = fminf(fmaxf(x + S.Gt[0] - S.ext_x, -LPA_FAR_F), LPA_FAR_F);
-  y = fminf(fmaxf(y + S.Gt[1] - S.ext_y, -LPA_FAR_F), LPA_FAR_F);
-  return make_int2((int)floorf(x) & ~7, (int)floorf(y) & ~1);
-}
-
-__device__ __forceinline__ Group load_group(const LpaLaunch &L, int s, int g, int u0, int v0, int bh) {
-  const LpaSensorK &S = L.s[s];
-  const int2 o = box_origin(S, u0, v0, bh);
-  Group r;
-  r.s = s;
-  r.row = (int)__umulhi((unsigned)g, S.group_magic);
-  r.col = g - r.row * (S.box_w >> 3);
-  r.X = o.x + 8 * r.col;
-  r.Y = o.y + r.row;
-  r.q = make_uint4(0, 0, 0, 0);
-  if (r.X >= 0 && r.X < S.width && r.Y >= 0 && r.Y < S.height)
-    r.q = __ldg(reinterpret_cast<const uint4 *>(S.raw + (size_t)r.Y * S.raw_pitch + r.X));
-  return r;
-}
 
 __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, float2 *planes) {
   const LpaSensorK &S = L.s[r.s];
@@ -103,17 +55,11 @@ __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, 
   float4 *even = reinterpret_cast<float4 *>(planes + 2 * (r.row & 1) * PP + (r.row >> 1) * PW + 4 * r.col);
   float4 *odd = even + (PP >> 1);
   float2 v[8];  // (1 / s2, f / s2)
-  if (scalar) {  // convert_sample's arithmetic, two samples at a time
+  if (scalar) {
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-      const float y0 = (float)(w[k] & 0xffffu), y1 = (float)(w[k] >> 16);
-      const float2 e = __fadd2_rn(make_float2(y0, y1), make_float2(-S.black, -S.black));
-      const float2 f = __fmul2_rn(e, make_float2(S.inv_gtn, S.inv_gtn));
-      const float2 d = __ffma2_rn(make_float2(S.gain, S.gain), make_float2(fmaxf(e.x, 0.f), fmaxf(e.y, 0.f)),
-                                  make_float2(S.read_var, S.read_var));
-      float2 iv = make_float2(__fdividef(S.gtn2, d.x), __fdividef(S.gtn2, d.y));
-      iv.x = y0 < S.sat && 2 * k < n ? iv.x : 0.f;
-      iv.y = y1 < S.sat && 2 * k + 1 < n ? iv.y : 0.f;
+      float2 f, iv;
+      convert_two(S, (float)(w[k] & 0xffffu), (float)(w[k] >> 16), 2 * k < n, 2 * k + 1 < n, f, iv);
       const float2 ivf = __fmul2_rn(iv, f);
       v[2 * k] = make_float2(iv.x, ivf.x);
       v[2 * k + 1] = make_float2(iv.y, ivf.y);
@@ -246,25 +192,9 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
   for (int s0 = 0; s0 < S; s0 += L.mean_bufs) {
     const int s1 = min(S, s0 + L.mean_bufs);
     if (s0) __syncthreads();  // the buffers' readers have left them
-    int total = 0;
-    for (int s = s0; s < s1; s++) total += (L.s[s].box_w >> 3) * L.s[s].box_h;
-    auto fetch = [&](int k) {
-      int s = s0, n = (L.s[s0].box_w >> 3) * L.s[s0].box_h;
-      while (k >= n) k -= n, s++, n = (L.s[s].box_w >> 3) * L.s[s].box_h;
-      return load_group(L, s, k, u0, v0, BH);
-    };
-    auto put = [&](const Group &r) { store_group(L, r, reinterpret_cast<float2 *>(smem + (r.s - s0) * L.mean_plane)); };
-    for (int k = tid; k < total; k += 2 * kThreads) {  // two loads in flight per thread
-      const bool two = k + kThreads < total;
-      const Group a = fetch(k);
-      if (two) {
-        const Group b = fetch(k + kThreads);
-        put(a);
-        put(b);
-      } else {
-        put(a);
-      }
-    }
+    stage_boxes<kThreads>(L, s0, s1, u0, v0, BH, [&](const Group &r) {
+      store_group(L, r, reinterpret_cast<float2 *>(smem + (r.s - s0) * L.mean_plane));
+    });
     __syncthreads();  // the planes (and the position tables) are whole
 #pragma unroll 1
   for (int s = s0; s < s1; s++) {
@@ -431,7 +361,9 @@ int lpa_mean_size(double reach_rb, double reach_g) {
   const double rb = std::floor(reach_rb) + 1, g = std::floor(reach_g) + 1;
   return rb <= 3 && g <= 2 ? 0 : rb <= 4 && g <= 3 ? 1 : -1;
 }
-int lpa_mean_cells(int size, bool green) { return size == 0 ? (green ? 2 : 3) : (green ? 3 : 4); }
+int lpa_mean_cells(int size, bool green) {
+  return size >= 2 ? size + 1 : size == 0 ? (green ? 2 : 3) : (green ? 3 : 4);
+}
 uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors) {
   if (!axis) return (uint32_t)(n_sensors * lpa_mean_tile_h(p) * 16);
   const int words = size == 0 ? lpa::Layout<3, 2>::kWords : lpa::Layout<4, 3>::kWords;

@@ -315,3 +315,35 @@ def test_metric_windows_and_near_rank_one(ctx, window_sigma, grad_scale):
     q = ctx.calpa_metric(c, torch.from_numpy(g).cuda()).cpu().numpy()
     check_metric(q, oracle.steering_metric(g.astype(np.float64), c.window_sigma, c.alpha, c.lambda1, c.lambda2,
                                            c.min_eig, c.max_eig, c.grad_scale))
+
+
+@pytest.mark.parametrize("w,h,scale,grad_sigma", [(1, 1, 1.0, 1.2), (63, 15, 1.0, 0.6), (65, 17, 1.0, 1.2),
+                                                   (130, 33, 1.5, 1.8), (96, 48, 2.0, 1.2), (40, 30, 0.6, 1.0),
+                                                   (65, 17, 1.0, 2.0)])
+def test_gradient_tiles_and_windows(ctx, w, h, scale, grad_sigma):
+    """The gradient pass's own kernel around its 64 x 8 tiles, at every pixel stride, with green windows of
+    2, 3 and 4 cells (and one of 5, which the general kernel takes), an odd sensor with calibration
+    frames and a rotated one: pass 1's tolerance of the module docstring at every pixel."""
+    import dataclasses
+    sw, sh = max(24, round(w / scale) + 3), max(24, round(h / scale) + 2)
+    p = synth.Params(order=2, sigmas=(0.8, 1.2), out_w=w, out_h=h,
+                     out_affine=np.array([[1 / scale, 0, 0.7], [0, 1 / scale, 0.4]]))
+    fr = synth._build_frame(1700 + w, 3, sw, sh, (1.0, 1 / 8, 1 / 64), 1.2, 0.4, 1e-3, p, "grad")
+    r = np.random.default_rng(w)
+    s = fr.sensors[1]
+    s.bias_frame = (s.black + r.uniform(-2, 2, (sh, sw))).astype(np.float32)
+    s.prnu_frame = r.uniform(0.95, 1.05, (sh, sw)).astype(np.float32)
+    s.read_var_frame = r.uniform(6, 12, (sh, sw)).astype(np.float32)
+    s.sat_frame = np.full((sh, sw), 3000, np.uint16)
+    c = _calpa(grad_sigma=grad_sigma)
+    ctx.set_rig(0, fr.sensors)
+    g = ctx.calpa_gradients(0, p, c, _raws(fr))
+    ctx.check()
+    check_gradients(fr, p, c, g.cpu().numpy())
+    # the buffer may start at any float
+    flat = torch.full((w * h * 2 + 1,), 7.0, device="cuda")
+    from paper_1308_4908_gb300 import hdr
+    hdr.hdr_calpa_gradients(ctx.handle, 0, hdr.params_struct(p), c, [int(x.data_ptr()) for x in _raws(fr)],
+                            flat.data_ptr() + 4, torch.cuda.current_stream().cuda_stream)
+    ctx.check()
+    np.testing.assert_array_equal(flat[1:].cpu().numpy(), g.cpu().numpy().ravel())
