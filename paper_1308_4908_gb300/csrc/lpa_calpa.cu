@@ -67,10 +67,16 @@ __device__ __forceinline__ float2 pair_sqrt(float2 a) {  // a >= 0
 // Bound by the FP32 pipe: 36 pipe cycles per warp and disc cell (12 operations on each of three
 // sums, gx^2 and gy^2 side by side in paired instructions). The same sums in FP64 kept the FP64
 // pipe 84 % busy: gradients and matrices of 1920 x 1080 with 29 cells took 751 us, with this kernel
-// 324 us.
+// and looped discs 324 us.
+//
+// UNIT: the disc of window_sigma 1 (radius 3: half widths 0, 2, 2, 3, 2, 2, 0), unrolled, so that a
+// cell is its two loads and its arithmetic (the loops over any disc issued 65 instructions a cell: 130 us
+// for 1920 x 1080, unrolled 101 us).
+__host__ __device__ constexpr int unit_row(int dj) { return dj == 0 ? 3 : dj == 3 || dj == -3 ? 0 : 2; }
+template <bool UNIT>
 __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__ MetricArgs A) {
   extern __shared__ __align__(16) float4 sm[];
-  const int r = A.r, TW = kBX + 2 * r, TH = kBY + 2 * r;
+  const int r = UNIT ? 3 : A.r, TW = kBX + 2 * r, TH = kBY + 2 * r;
   float4 *sd = sm;                                        // (gx^2, gy^2, their residuals)
   float2 *sx = reinterpret_cast<float2 *>(sm + TW * TH);  // (gx gy, its residual)
   // one-dimensional grid over the 32 x 8 blocks (any output height)
@@ -94,33 +100,43 @@ __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__
   const float2 minus = make_float2(-1.f, -1.f);
   float2 S = make_float2(0.f, 0.f), E = S;  // (sum w gx^2, sum w gy^2) and what rounding dropped
   float s = 0.f, e = 0.f;                   // the same of sum w gx gy
-  for (int dj = -r; dj <= r; dj++) {
-    const int rw = A.rw[dj + r];
-    const int at = (threadIdx.y + r + dj) * TW + threadIdx.x + r;
+  auto add = [&](float2 w, int at) {
+    const float4 d = sd[at];
+    const float2 x = sx[at];
+    {
+      const float2 X = make_float2(d.x, d.y), W = make_float2(w.x, w.x);
+      const float2 P = __fmul2_rn(W, X);
+      float2 q = __ffma2_rn(W, X, make_float2(-P.x, -P.y));
+      q = __ffma2_rn(W, make_float2(d.z, d.w), q);
+      q = __ffma2_rn(make_float2(w.y, w.y), X, q);
+      const float2 t = __fadd2_rn(S, P), z = __ffma2_rn(S, minus, t);
+      const float2 k = __ffma2_rn(__ffma2_rn(z, minus, t), minus, S);  // S - (t - z)
+      E = __fadd2_rn(E, __fadd2_rn(__fadd2_rn(k, __ffma2_rn(z, minus, P)), q));
+      S = t;
+    }
+    {
+      const float p = __fmul_rn(w.x, x.x);
+      const float q = fmaf(w.y, x.x, fmaf(w.x, x.y, __fmaf_rn(w.x, x.x, -p)));
+      const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+      const float k = __fsub_rn(s, __fsub_rn(t, z));
+      e = __fadd_rn(e, __fadd_rn(__fadd_rn(k, __fsub_rn(p, z)), q));
+      s = t;
+    }
+  };
+  const int mid = (threadIdx.y + r) * TW + threadIdx.x + r;
+  if constexpr (UNIT) {
+    float2 w[10];
+#pragma unroll
+    for (int k = 0; k < 10; k++) w[k] = A.w[k];
+#pragma unroll
+    for (int dj = -3; dj <= 3; dj++)
+#pragma unroll
+      for (int di = -unit_row(dj); di <= unit_row(dj); di++) add(w[di * di + dj * dj], mid + dj * TW + di);
+  } else {
+    for (int dj = -r; dj <= r; dj++) {
+      const int rw = A.rw[dj + r];
 #pragma unroll 2
-    for (int di = -rw; di <= rw; di++) {
-      const float2 w = A.w[di * di + dj * dj];
-      const float4 d = sd[at + di];
-      const float2 x = sx[at + di];
-      {
-        const float2 X = make_float2(d.x, d.y), W = make_float2(w.x, w.x);
-        const float2 P = __fmul2_rn(W, X);
-        float2 q = __ffma2_rn(W, X, make_float2(-P.x, -P.y));
-        q = __ffma2_rn(W, make_float2(d.z, d.w), q);
-        q = __ffma2_rn(make_float2(w.y, w.y), X, q);
-        const float2 t = __fadd2_rn(S, P), z = __ffma2_rn(S, minus, t);
-        const float2 k = __ffma2_rn(__ffma2_rn(z, minus, t), minus, S);  // S - (t - z)
-        E = __fadd2_rn(E, __fadd2_rn(__fadd2_rn(k, __ffma2_rn(z, minus, P)), q));
-        S = t;
-      }
-      {
-        const float p = __fmul_rn(w.x, x.x);
-        const float q = fmaf(w.y, x.x, fmaf(w.x, x.y, __fmaf_rn(w.x, x.x, -p)));
-        const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-        const float k = __fsub_rn(s, __fsub_rn(t, z));
-        e = __fadd_rn(e, __fadd_rn(__fadd_rn(k, __fsub_rn(p, z)), q));
-        s = t;
-      }
+      for (int di = -rw; di <= rw; di++) add(A.w[di * di + dj * dj], mid + dj * TW + di);
     }
   }
   int M = A.cells;
@@ -152,7 +168,7 @@ __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__
   if (l2.x < 0x1p-18f * l1.x) {
     double da = 0.0, db = 0.0, dc = 0.0;
     for (int dj = -r; dj <= r; dj++) {
-      const int rw = A.rw[dj + r], at = (threadIdx.y + r + dj) * TW + threadIdx.x + r;
+      const int rw = A.rw[dj + r], at = mid + dj * TW;
       for (int di = -rw; di <= rw; di++) {
         const float2 wp = A.w[di * di + dj * dj], x = sx[at + di];
         const float4 q = sd[at + di];
@@ -302,7 +318,10 @@ hdr_status hdr_calpa_metric(hdr_ctx *ctx, int32_t out_w, int32_t out_h, const hd
   A.max_eig = (float)calpa->max_eig;
   const unsigned blocks = (unsigned)(((long long)out_w + kBX - 1) / kBX * (((long long)out_h + kBY - 1) / kBY));
   const size_t smem = (size_t)(kBX + 2 * A.r) * (kBY + 2 * A.r) * (sizeof(float4) + sizeof(float2));  // at most 35 KB
-  calpa_metric<<<blocks, dim3(kBX, kBY), smem, (cudaStream_t)cuda_stream>>>(A);
+  bool unit = A.r == 3;
+  for (int dj = -3; dj <= 3 && unit; dj++) unit = A.rw[dj + 3] == unit_row(dj);
+  if (unit) calpa_metric<true><<<blocks, dim3(kBX, kBY), smem, (cudaStream_t)cuda_stream>>>(A);
+  else calpa_metric<false><<<blocks, dim3(kBX, kBY), smem, (cudaStream_t)cuda_stream>>>(A);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return lpa_fail(HDR_E_CUDA, cudaGetErrorString(e));
   return HDR_OK;
