@@ -404,6 +404,23 @@ def params_struct(p) -> hdr_params:
     return h
 
 
+def _current_stream() -> int:
+    """The current stream's handle. torch.cuda.current_stream() builds a Stream object for it (2.9 us of a
+    10 us call); the accessor below returns the handle alone in 0.1 us where torch has it."""
+    global _raw_stream
+    import torch
+    if _raw_stream is None:
+        get = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        dev = getattr(torch._C, "_cuda_getDevice", None)
+        stream = torch.cuda.current_stream().cuda_stream  # initialises CUDA
+        usable = get is not None and dev is not None and get(dev()) == stream
+        _raw_stream = (lambda: get(dev())) if usable else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
+
+
+_raw_stream = None
+
+
 class Context:
     """One library context on one CUDA device; rigs are uploaded once and stay resident."""
 
@@ -433,9 +450,9 @@ class Context:
 
     @staticmethod
     def _stream(stream):
-        import torch
-        s = stream if stream is not None else torch.cuda.current_stream()
-        return s.cuda_stream
+        if stream is not None:
+            return stream.cuda_stream
+        return _current_stream()
 
     def reconstruct(self, rig_id: int, params, raws, out=None, choice=None, levels=None, stream=None):
         """Reconstruct one frame from device tensors `raws` (uint16 [H, pitch] each); returns `out`."""
