@@ -421,7 +421,10 @@ __host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j
 // Jacobi-equilibrated matrix D A D (D = diag(A)^{-1/2}), which are d_j / A_jj: equilibration
 // changes L but scales each pivot by 1 / A_jj. l = A^{-1} e_0, C_0 = l^T b,
 // Var C_0 = l^T (Phi^T W S W Phi) l with S the sample variances.
-template <typename T, int P, class MOM, bool COEF = false>
+// ANY: dmin and the values are wanted whatever the pivots (the FP64 re-solve looks at fits just below
+// min_pivot); without it a pivot or diagonal that is not positive only has to leave valid false (dmin
+// keeps its value, which is not above min_pivot >= 0; what follows may be NaN), and no reciprocal is guarded.
+template <typename T, int P, class MOM, bool COEF = false, bool ANY = true>
 __device__ __forceinline__ FitOut solve(const MOM &m, float min_pivot) {
   FitOut r;
   T a[P * (P + 1) / 2];  // lower triangle, overwritten by L (below the diagonal) and D
@@ -434,7 +437,7 @@ __device__ __forceinline__ FitOut solve(const MOM &m, float min_pivot) {
 #pragma unroll
   for (int i = 0; i < P; i++) {
     pos = pos && (a[tri(i, i)] > T(0));
-    rdiag[i] = a[tri(i, i)] > T(0) ? rcp_t(a[tri(i, i)]) : T(0);
+    rdiag[i] = !ANY || a[tri(i, i)] > T(0) ? rcp_t(a[tri(i, i)]) : T(0);
   }
   // triangular loops are written with fixed trip counts and guards so that they unroll fully;
   // u holds L_iq d_q (the column before its division by the pivot), so that each update term
@@ -451,7 +454,7 @@ __device__ __forceinline__ FitOut solve(const MOM &m, float min_pivot) {
     const T de = dj * rdiag[j];  // pivot of the equilibrated matrix
     dmin = de < dmin ? de : dmin;
     dmax = de > dmax ? de : dmax;
-    dinv[j] = dj > T(0) ? rcp_t(dj) : T(0);
+    dinv[j] = !ANY || dj > T(0) ? rcp_t(dj) : T(0);
 #pragma unroll
     for (int i = 0; i < P; i++) {
       if (i > j) {
@@ -540,7 +543,7 @@ __device__ __forceinline__ FitOut solve(const MOM &m, float min_pivot) {
 // cond_fallback and the fit could still pass min_pivot in exact arithmetic.
 template <int P, class MOM, bool COEF = false, bool F64 = true>
 __device__ __forceinline__ FitOut solve_with_fallback(const MOM &m, float min_pivot, float cond_fallback) {
-  FitOut r = solve<float, P, MOM, COEF>(m, min_pivot);
+  FitOut r = solve<float, P, MOM, COEF, F64>(m, min_pivot);
   if constexpr (!F64) return r;
   bool redo = cond_fallback > 0.f && m.count() >= (float)P && !(r.dmin * cond_fallback >= r.dmax) &&
               r.dmin > min_pivot - LPA_PIVOT_FP32_ERR;
