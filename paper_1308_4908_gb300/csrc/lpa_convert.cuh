@@ -42,4 +42,17 @@ __device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool scal
   return stage_pair(f, iv);
 }
 
+// convert_sample<false> of two samples of a sensor without calibration frames, in paired arithmetic with
+// its roundings: f and 1 / s2, which is 0 (f is not, unlike there) where ok is false or the sample is
+// saturated.
+__device__ __forceinline__ void convert_two(const LpaSensorK &S, float y0, float y1, bool ok0, bool ok1, float2 &f, float2 &iv) {
+  const float2 e = __fadd2_rn(make_float2(y0, y1), make_float2(-S.black, -S.black));
+  f = __fmul2_rn(e, make_float2(S.inv_gtn, S.inv_gtn));
+  const float2 d = __ffma2_rn(make_float2(S.gain, S.gain), make_float2(fmaxf(e.x, 0.f), fmaxf(e.y, 0.f)),
+                              make_float2(S.read_var, S.read_var));
+  iv = make_float2(__fdividef(S.gtn2, d.x), __fdividef(S.gtn2, d.y));
+  iv.x = y0 < S.sat && ok0 ? iv.x : 0.f;
+  iv.y = y1 < S.sat && ok1 ? iv.y : 0.f;
+}
+
 }  // namespace lpa

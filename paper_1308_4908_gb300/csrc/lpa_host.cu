@@ -1604,7 +1604,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
       cudaKernelNodeParams c{};
       c.func = const_cast<void *>(lpa_convert_kernel(L.mode == LPA_LITERAL));
       c.gridDim = lpa_convert_grid(L, rows[f]);
-      c.blockDim = dim3(256);
+      c.blockDim = lpa_convert_block();
       c.sharedMemBytes = 0;
       c.kernelParams = args.back().data();
       key.push_back({-1, L.mode == LPA_LITERAL ? 1 : 0, 0, 0, 0});

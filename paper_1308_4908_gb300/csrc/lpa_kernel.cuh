@@ -1280,40 +1280,45 @@ __global__ void __launch_bounds__(LPA_TILE *TH, (FrameOccupancy<ORDER, COMP, TH,
 // blockIdx.y into its colour-phase planes (r1 may be the height + 1 of an odd height: that row is
 // outside the frame and writes zeros), with the arithmetic the reconstruction kernels use when
 // they convert staged footprints themselves (convert_sample), so the staged values are the same.
-// Each thread takes eight samples of a row per step (one 16-byte load; the rows of the raw frame
+// A thread takes eight samples of a row per step (one 16-byte load; the rows of the raw frame
 // are 16-byte aligned and padded to a multiple of 8 samples) and writes the four of each phase
-// column as two 16-byte stores, so that a warp's loads and stores are contiguous.
+// column as two 16-byte stores, so that a warp's loads and stores are contiguous. CTAs of 64 groups x 4
+// rows over a three-dimensional grid (groups, rows, sensors) and paired arithmetic: one flat 64-bit index
+// and a sample at a time took 390 instructions a group, 37 us for 3 x 2048^2.
+constexpr int kConvertX = 64, kConvertY = 4;
 template <bool LIT>
-__global__ void __launch_bounds__(256) lpa_convert(const __grid_constant__ LpaLaunch L, const LpaRows R) {
-  const int s = blockIdx.y;
+__global__ void __launch_bounds__(kConvertX *kConvertY) lpa_convert(const __grid_constant__ LpaLaunch L, const LpaRows R) {
+  const int s = blockIdx.z;
   const LpaSensorK &Sk = L.s[s];
-  const int r0 = R.r0[s], r1 = R.r1[s];
-  if (r1 <= r0) return;
   const int CP = Sk.conv_pitch, W = Sk.width;
-  const int G = (CP + 3) >> 2;  // groups of four phase columns (eight samples) per row
+  const int c0 = 4 * (int)(blockIdx.x * kConvertX + threadIdx.x), X0 = 2 * c0;  // four phase columns, eight samples
+  if (c0 >= CP) return;
   const bool scalar = !Sk.bias && !Sk.rvar && !Sk.satf && !Sk.prnu;
-  const long n = (long)(r1 - r0) * G;
   const size_t plane = (size_t)Sk.conv_h * CP;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const int Y = r0 + (int)(i / G), c0 = 4 * (int)(i % G);
-    const int X0 = 2 * c0;
-    const bool in_row = Y < Sk.height;  // the padding row of an odd height converts to zeros
-    uint16_t v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (in_row && X0 < W) {
-      const uint4 q = *reinterpret_cast<const uint4 *>(Sk.raw + (size_t)Y * Sk.raw_pitch + X0);
-      const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
+  const int last = R.r1[s];
+  for (int Y = R.r0[s] + (int)(blockIdx.y * kConvertY + threadIdx.y); Y < last; Y += (int)gridDim.y * kConvertY) {
+    const int n = Y < Sk.height ? W - X0 : 0;  // samples inside the frame (the padding row of an odd height: none)
+    uint4 q = make_uint4(0, 0, 0, 0);
+    if (n > 0) q = *reinterpret_cast<const uint4 *>(Sk.raw + (size_t)Y * Sk.raw_pitch + X0);
+    const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
+    float2 e[4], o[4];  // columns c0 .. c0 + 3 of the even-x and the odd-x phase
+    if (!LIT && scalar) {
 #pragma unroll
       for (int k = 0; k < 4; k++) {
-        v[2 * k] = (uint16_t)(w4[k] & 0xffffu);
-        v[2 * k + 1] = (uint16_t)(w4[k] >> 16);
+        float2 f, iv;
+        const float y0 = (float)(w4[k] & 0xffffu), y1 = (float)(w4[k] >> 16);
+        const bool in0 = 2 * k < n && y0 < Sk.sat, in1 = 2 * k + 1 < n && y1 < Sk.sat;
+        convert_two(Sk, y0, y1, in0, in1, f, iv);
+        e[k] = stage_pair(in0 ? f.x : 0.f, iv.x);
+        o[k] = stage_pair(in1 ? f.y : 0.f, iv.y);
       }
-    }
-    float2 e[4], o[4];  // columns c0 .. c0 + 3 of the even-x and the odd-x phase
+    } else {
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const int X = X0 + 2 * k;
-      e[k] = in_row && X < W ? convert_sample<LIT>(Sk, scalar, X, Y, (float)v[2 * k]) : stage_pair(0.f, 0.f);
-      o[k] = in_row && X + 1 < W ? convert_sample<LIT>(Sk, scalar, X + 1, Y, (float)v[2 * k + 1]) : stage_pair(0.f, 0.f);
+      for (int k = 0; k < 4; k++) {
+        const int X = X0 + 2 * k;
+        e[k] = 2 * k < n ? convert_sample<LIT>(Sk, scalar, X, Y, (float)(w4[k] & 0xffffu)) : stage_pair(0.f, 0.f);
+        o[k] = 2 * k + 1 < n ? convert_sample<LIT>(Sk, scalar, X + 1, Y, (float)(w4[k] >> 16)) : stage_pair(0.f, 0.f);
+      }
     }
     float2 *de = Sk.conv + (size_t)(2 * (Y & 1)) * plane + (size_t)(Y >> 1) * CP + c0;  // colour phase (0, Y & 1)
     float2 *dodd = de + plane;                                                         // colour phase (1, Y & 1)
