@@ -3,6 +3,7 @@
 #include <stdint.h>
 
 #include "lpa_launch.h"
+#include "lpa_ptx.cuh"
 
 // sensor-space positions are clamped to +-LPA_FAR px (far outside any sensor) before integer conversion
 #define LPA_FAR 1.0e7
@@ -23,7 +24,7 @@ __device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool scal
     if (y < Sk.sat) {
       const float e0 = y - Sk.black;
       f = e0 * Sk.inv_gtn;
-      iv = __fdividef(Sk.gtn2, fmaf(Sk.gain, fmaxf(e0, 0.f), Sk.read_var));
+      iv = div_approx(Sk.gtn2, fmaf(Sk.gain, fmaxf(e0, 0.f), Sk.read_var));
       if (LIT) iv = sqrtf(iv);
     }
   } else {
@@ -34,8 +35,8 @@ __device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool scal
     if (y < sat) {
       const float a = Sk.prnu ? Sk.prnu[px] : 1.f;
       const float e0 = y - b;
-      f = __fdividef(e0 * Sk.inv_gtn, a);
-      iv = __fdividef(Sk.gtn2 * a * a, fmaf(Sk.gain, fmaxf(e0, 0.f), rv));
+      f = div_approx(e0 * Sk.inv_gtn, a);
+      iv = div_approx(Sk.gtn2 * a * a, fmaf(Sk.gain, fmaxf(e0, 0.f), rv));
       if (LIT) iv = sqrtf(iv);
     }
   }
@@ -50,7 +51,7 @@ __device__ __forceinline__ void convert_two(const LpaSensorK &S, float y0, float
   f = __fmul2_rn(e, make_float2(S.inv_gtn, S.inv_gtn));
   const float2 d = __ffma2_rn(make_float2(S.gain, S.gain), make_float2(fmaxf(e.x, 0.f), fmaxf(e.y, 0.f)),
                               make_float2(S.read_var, S.read_var));
-  iv = make_float2(__fdividef(S.gtn2, d.x), __fdividef(S.gtn2, d.y));
+  iv = make_float2(div_approx(S.gtn2, d.x), div_approx(S.gtn2, d.y));
   iv.x = y0 < S.sat && ok0 ? iv.x : 0.f;
   iv.y = y1 < S.sat && ok1 ? iv.y : 0.f;
 }

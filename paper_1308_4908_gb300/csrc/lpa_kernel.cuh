@@ -410,7 +410,7 @@ struct FitOut {
   float c1, c2;      // first-order coefficients c = A^{-1} b (only when asked for)
 };
 
-__device__ __forceinline__ float rcp_t(float x) { return __fdividef(1.f, x); }
+__device__ __forceinline__ float rcp_t(float x) { return rcp_approx(x); }
 __device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
 
 // packed lower-triangle index (i >= j)

@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
     float val[P];
 #pragma unroll
     for (int k = 0; k < P; k++)
-      val[k] = acc[k][c].x > 0.f ? __fdividef(acc[k][c].y, acc[k][c].x) : __int_as_float(0x7fffffff);
+      val[k] = acc[k][c].x > 0.f ? div_approx(acc[k][c].y, acc[k][c].x) : __int_as_float(0x7fffffff);
     if (L.out_half) {
       __half *o = reinterpret_cast<__half *>(L.out) + c * plane + first;
 #pragma unroll

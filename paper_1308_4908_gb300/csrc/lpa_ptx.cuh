@@ -15,6 +15,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// 1 / x as the FP32 reciprocal unit gives it: __fdividef(1, x) for every normal x. That function also
+// scales denormal x (four instructions for one), of which it can return only the reciprocals of [2^-128,
+// 2^-126) as finite numbers; here these are infinite too.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// a / b as __fdividef rounds it (the product with the approximate reciprocal).
+__device__ __forceinline__ float div_approx(float a, float b) { return __fmul_rn(a, rcp_approx(b)); }
+
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
