@@ -312,6 +312,7 @@ namespace {
 struct MeanPlan {
   int size = -1;      // kernel template, -1: another kernel
   bool axis = true;   // every sensor's axes are parallel to the output's
+  bool even = true;   // every sensor's map is a rotation (or reflection) and an even scale
   int tx = 0, ty = 0; // output pixels to a cell of a colour phase where that is exact (2 or 4), else 0
   int p = 1;          // output rows per thread
   double rb = 0, g = 0;  // window radius of R and B, and of G (reference px)
@@ -344,6 +345,8 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
     m.ty = s == 0 || m.ty == ty ? ty : 0;
     most = std::max(most, std::max(std::hypot(t[0], t[1]), std::hypot(t[3], t[4])));
     m.axis = m.axis && t[1] == 0.0 && t[3] == 0.0;
+    const double *a = rig.s[s].d.affine;
+    m.even = m.even && std::fabs(a[0] * a[1] + a[3] * a[4]) <= 1e-9 * std::min(a[0] * a[0] + a[3] * a[3], a[1] * a[1] + a[4] * a[4]);
   }
   if (!m.axis || !m.tx || !m.ty) m.tx = m.ty = 0;
   m.size = lpa_mean_size(m.rb * most + 2e-3, m.g * most + 2e-3);
@@ -773,7 +776,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     L.mode = env.grad ? LPA_GRADIENTS : LPA_MEAN;
     L.mean_p = mean.p;
     L.mean_size = mean.size;
-    L.mean_axis = mean.axis ? 1 : 0;
+    L.mean_axis = mean.axis ? 1 : mean.even ? 2 : 0;
     L.mean_lx = mean.tx / 2;  // 2 or 4 pixels
     L.mean_ly = mean.ty / 2;
     if (L.tiles_x > 0 && L.tiles_y > 0) lpa_mean_rows(L, 0, L.tiles_x * L.tiles_y);
@@ -1619,7 +1622,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 128 * (L.mean_lx != 0) : L.px,
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 256 * (L.mean_lx != 0) : L.px,
                    L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};

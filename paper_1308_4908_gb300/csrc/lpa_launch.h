@@ -104,8 +104,8 @@ struct LpaLaunch {
   // LPA_LITERAL: the searched window with the noise weight printed in Eq. 6 (K / s, not K / s2).
   int mode;
   float *aux;
-  // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, whether every sensor's axes are
-  // parallel to the output's, the pixels that span one cell of a colour phase where that is exact for
+  // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, its form (1: every
+  // sensor's axes parallel to the output's, 2: every sensor's map a rotation and an even scale, 0: any), the pixels that span one cell of a colour phase where that is exact for
   // every sensor (as powers of two, 1 or 2 on each axis, else both 0), sensors staged at a time, bytes of one sensor's
   // colour-phase planes (from offset 0) and the offset of the position tables
   int mean_p, mean_size, mean_axis, mean_lx, mean_ly, mean_bufs;

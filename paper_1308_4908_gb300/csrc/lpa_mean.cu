@@ -25,7 +25,9 @@
 // kPeriodic: besides, 2 or 4 output pixels span exactly one cell of a colour phase (translated sensors at
 // 1x or twofold output), so pixels that far apart see the same offsets: a thread takes P rows of one
 // class, forms the K of its cells once per sensor and slides the window down one cell a row, each
-// loaded cell serving up to N rows. kGeneral: each cell forms its offset and one exponential.
+// loaded cell serving up to N rows. kFactored: the output is rotated against a sensor whose map is a
+// rotation and an even scale, so |d|^2 still separates in the sensor's axes; the 2 N factors of a window are
+// formed per pixel. kGeneral: each cell forms its offset and one exponential.
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -81,7 +83,7 @@ __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, 
   odd[1] = make_float4(v[5].x, v[5].y, v[7].x, v[7].y);
 }
 
-enum { kGeneral = 0, kAxis = 1, kPeriodic = 2 };
+enum { kGeneral = 0, kAxis = 1, kFactored = 2, kPeriodic = 3 };
 
 // The cells and factors of one position along one axis for every (window, phase): words of Layout at
 // t[0], t[stride], ... `last`: how many cells further the last position served by the entry lies. Returns
@@ -120,7 +122,8 @@ template <int NR, int NG, int FORM, int P>
 __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(const __grid_constant__ LpaLaunch L) {
   using T = Layout<NR, NG>;
   constexpr int kThreads = lpa_mean_threads(P), BH = lpa_mean_tile_h(P);
-  if (*reinterpret_cast<volatile unsigned int *>(L.status) & LPA_ERR_TIMEOUT) return;
+  // read now, looked at before the stores: once a bounded wait has run out, nothing is written
+  const unsigned int status = *reinterpret_cast<volatile unsigned int *>(L.status);
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, S = L.n_sensors;
   const int y_end = L.mean_y1;
@@ -136,15 +139,16 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
   if constexpr (FORM == kPeriodic) {
     // one entry per sensor, axis and class of positions: class c starts at G c + G_t, and the n-th
     // pixel of a class lies exactly 2 n px further, whatever the tile
-    if (tid < S * (tx + ty)) {
-      const int s = tid / (tx + ty), e = tid - s * (tx + ty);
+    const int entry = kThreads - 1 - tid;  // by the last threads: the first ones fetch samples
+    if (entry < S * (tx + ty)) {
+      const int s = entry / (tx + ty), e = entry - s * (tx + ty);
       const bool col = e < tx;
       const int c = col ? e : e - tx;
       const LpaSensorK &Sk = L.s[s];
       const int2 o = box_origin(Sk, u0, v0, BH);
       const double q = fmin(fmax(col ? Sk.G[0] * c + Sk.G[2] : Sk.G[4] * c + Sk.G[5], -LPA_FAR), LPA_FAR), fl = floor(q);
       const int l = (int)fl + (col ? 2 * (u0 >> lx) - o.x : 2 * (v0 >> ly) - o.y);
-      float *t = xt + tid * T::kRow;
+      float *t = xt + entry * T::kRow;
       const int last = col ? (kBW - 1) >> lx : (BH - 1) >> ly;
       if (!axis_entry<NR, NG>(L, Sk, col, l, (float)(q - fl), last, t, 1) && (col ? u0 + c < L.out_w : v0 + c < y_end) && fabs(q) < 1e6)
         atomicOr(L.status, LPA_ERR_BOUNDS);
@@ -284,6 +288,25 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
           const int j0 = first_cell(ly, fy, oy, hy, floorf(0.5f * hy), dy), j = min(max(j0, 0), (Sk.box_h >> 1) - N);
           ok = ok && i == i0 && j == j0;
           const float2 *pl = planes + (ox + 2 * oy) * PP + j * PW + i;
+          if constexpr (FORM == kFactored) {
+            const float cx = -unit * unit * fmaf(Sk.A[0], Sk.A[0], Sk.A[2] * Sk.A[2]);
+            const float cy = -unit * unit * fmaf(Sk.A[1], Sk.A[1], Sk.A[3] * Sk.A[3]);
+            float ex[N], ey[N];
+#pragma unroll
+            for (int c = 0; c < N; c++) {
+              const float x = dx + 2.f * (float)c, y = dy + 2.f * (float)c;
+              ex[c] = ex2_approx(cx * x * x);
+              ey[c] = ex2_approx(cy * y * y);
+            }
+#pragma unroll
+            for (int r = 0; r < N; r++)
+#pragma unroll
+              for (int c = 0; c < N; c++) {
+                const float K = fmaxf(fmaf(ex[c], ey[r], -L.taper), 0.f);
+                a = __ffma2_rn(make_float2(K, K), pl[r * PW + c], a);
+              }
+            return;
+          }
           const float2 CX = make_float2(Sk.A[0] * unit, Sk.A[2] * unit), CY = make_float2(Sk.A[1] * unit, Sk.A[3] * unit);
           const float2 DX = make_float2(dx, dx), DY = make_float2(dy, dy);
           const float2 D0 = __ffma2_rn(CY, DY, __fmul2_rn(CX, DX));
@@ -308,7 +331,7 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
     }
   }
   }
-  if (u >= L.out_w) return;
+  if (u >= L.out_w || (status & LPA_ERR_TIMEOUT)) return;
   // per channel: a pointer to the first row's pixel and the step to the next
   const size_t plane = (size_t)L.out_w * L.out_h, first = (size_t)(v0 + row0) * L.out_w + u;
   const int step = FORM == kPeriodic ? ly : 0;
@@ -350,8 +373,9 @@ const void *pick(int p) {
 template <int NR, int NG>
 const void *pick(const LpaLaunch &L) {
   return L.mean_lx     ? pick<NR, NG, kPeriodic>(L.mean_p)
-         : L.mean_axis ? pick<NR, NG, kAxis>(L.mean_p)
-                       : pick<NR, NG, kGeneral>(L.mean_p);
+         : L.mean_axis == 1 ? pick<NR, NG, kAxis>(L.mean_p)
+         : L.mean_axis == 2 ? pick<NR, NG, kFactored>(L.mean_p)
+                            : pick<NR, NG, kGeneral>(L.mean_p);
 }
 
 }  // namespace

@@ -112,6 +112,18 @@ def test_mirrored_transposed_and_outside(ctx, affine):
     assert np.array_equal(np.isnan(out), ch == 255)
 
 
+@pytest.mark.parametrize("w,h,scale", [(131, 34, 1.0), (97, 66, 1.4)])
+def test_sheared_sensors(ctx, w, h, scale):
+    """Sensors whose axes are neither orthogonal nor evenly scaled: the windows are ellipses in the
+    sensor and the Gaussian does not factor."""
+    fr = _frame(w, h, 1.0, n=3, out_affine=np.array([[1 / scale, 0.01, 0.3], [-0.02, 1 / scale, 0.6]]))
+    for k, s in enumerate(fr.sensors):
+        s.affine = s.affine @ np.array([[1.0, 0.03 * (k + 1), 0.0], [0.0, 1.0 + 0.04 * k, 0.0], [0.0, 0.0, 1.0]])
+        s.raw = synth.simulate_raw(fr.scene, s, 1500, k)
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
 @pytest.mark.parametrize("n", [1, 8])
 @pytest.mark.parametrize("rot", [0.0, 2.0])
 def test_sensor_counts_and_half(ctx, n, rot):
