@@ -317,16 +317,17 @@ struct MeanPlan {
   int p = 1;          // output rows per thread
   double rb = 0, g = 0;  // window radius of R and B, and of G (reference px)
 };
-// Whether a frame runs lpa_mean: order 0, one scale, plain sums, the inverse-variance weight, and
+// Whether a frame runs lpa_mean: order 0, one scale, the inverse-variance weight, and
 // windows of at most 4 x 4 (R, B) and 3 x 3 (G) cells of a colour phase. A fit of one unknown has the
 // equilibrated pivot 1, so it is usable with any sample (min_pivot below 1) and never solved again
 // in FP64 (cond_fallback at least 1, or none); other parameters keep the general kernel.
 // Rows per thread: four, or eight of half as many threads in the periodic form, once 64 x 32 tiles fill
-// the SMs' two resident CTAs twice (less halo converted per pixel), fewer for smaller frames (more CTAs).
+// the SMs' two resident CTAs twice (less halo converted per pixel), fewer for smaller frames (more CTAs);
+// two of compensated sums (24 registers of sums a row).
 MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   MeanPlan m;
   // (its grid has a row of tiles per y index: at most 65535 of 8 rows)
-  if (p->out_h > 65535 * 8 || p->order != 0 || p->n_scales != 1 || p->accum != 0 || p->weight_mode != 0 || !(p->min_pivot < 0.99) ||
+  if (p->out_h > 65535 * 8 || p->order != 0 || p->n_scales != 1 || p->weight_mode != 0 || !(p->min_pivot < 0.99) ||
       !(p->cond_fallback <= 0.0 || p->cond_fallback >= 1.0))
     return m;
   m.rb = p->trunc_k * p->sigma[0];
@@ -351,7 +352,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   if (!m.axis || !m.tx || !m.ty) m.tx = m.ty = 0;
   m.size = lpa_mean_size(m.rb * most + 2e-3, m.g * most + 2e-3);
   const long long px = (long long)p->out_w * p->out_h;
-  m.p = px >= 4LL * 152 * 64 * 32 ? (m.tx ? 8 : 4) : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
+  m.p = p->accum ? 2 : px >= 4LL * 152 * 64 * 32 ? (m.tx ? 8 : 4) : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
   return m;
 }
 
@@ -775,6 +776,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   if (mean.size >= 0) {
     L.mode = env.grad ? LPA_GRADIENTS : LPA_MEAN;
     L.mean_p = mean.p;
+    L.mean_comp = p->accum != 0;
     L.mean_size = mean.size;
     L.mean_axis = mean.axis ? 1 : mean.even ? 2 : 0;
     L.mean_lx = mean.tx / 2;  // 2 or 4 pixels
@@ -1622,7 +1624,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 256 * (L.mean_lx != 0) : L.px,
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 256 * (L.mean_lx != 0) + 512 * L.mean_comp : L.px,
                    L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};

@@ -30,6 +30,7 @@
 #include "lpa_convert.cuh"
 #include "lpa_launch.h"
 #include "lpa_ptx.cuh"
+#include "lpa_sums.cuh"
 
 namespace lpa {
 
@@ -43,17 +44,6 @@ __host__ __device__ constexpr int ex(int m) { return (m == 1 || m == 4) ? 1 : (m
 __host__ __device__ constexpr int ey(int m) { return (m == 2 || m == 4) ? 1 : (m == 5 ? 2 : 0); }
 
 // ---------------------------------------------------------------- moments
-
-// Error-free sum of two floats (Knuth's two-sum) and product (FMA residual).
-__device__ __forceinline__ void comp_add(float &hi, float &lo, float a, float b) {
-  float p = __fmul_rn(a, b);
-  float pe = __fmaf_rn(a, b, -p);
-  float s = __fadd_rn(hi, p);
-  float bb = __fsub_rn(s, hi);
-  float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  hi = s;
-  lo = __fadd_rn(lo, __fadd_rn(e, pe));
-}
 
 // VAR: the variance sums are kept (they are not where no interval is formed: one window scale, the
 // gradient pass).
@@ -302,19 +292,6 @@ struct MomentsLean {
   __device__ __forceinline__ T Kv(int) const { return T(0); }
 };
 
-// comp_add on two sums at once: hi + lo += a b in each half, every operation rounded as there
-// (differences as products with -1; `na` is -a, so that the residual needs no negation).
-__device__ __forceinline__ void comp_add2(float2 &hi, float2 &lo, float2 a, float2 na, float2 b) {
-  const float2 M = make_float2(-1.f, -1.f);
-  const float2 p = __fmul2_rn(a, b);
-  const float2 npe = __ffma2_rn(na, b, p);  // -(a b - p)
-  const float2 s = __fadd2_rn(hi, p);
-  const float2 bb = __ffma2_rn(hi, M, s);
-  const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, M, s), M, hi), __ffma2_rn(bb, M, p));
-  hi = s;
-  lo = __fadd2_rn(lo, __ffma2_rn(npe, M, e));
-}
-
 // Compensated sums of orders 1 and 2 without the variance sums, two at a time: the Gram sums in
 // pairs of monomials, (sum w, sum w f) together. The same terms, order and roundings as
 // Moments<ORDER, true>, whose one sum at a time issued 10 scalar operations a sum (87 % of issue
@@ -340,7 +317,7 @@ struct MomentsCompLean {
   __device__ __forceinline__ void add2(float2 D, float2 D2, float w, float wf, float) {
     const float2 W = make_float2(w, w), NW = make_float2(-w, -w), F = make_float2(wf, wf), NF = make_float2(-wf, -wf);
     const float m4 = D.x * D.y;
-    comp_add2(h[0], l[0], make_float2(w, wf), make_float2(-w, -wf), make_float2(1.f, 1.f));
+    comp_sum2(h[0], l[0], make_float2(w, wf));
     comp_add2(h[1], l[1], W, NW, D);
     comp_add2(h[2], l[2], W, NW, D2);
     comp_add2(h[3], l[3], F, NF, D);

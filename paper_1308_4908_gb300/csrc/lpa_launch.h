@@ -109,6 +109,7 @@ struct LpaLaunch {
   // every sensor (as powers of two, 1 or 2 on each axis, else both 0), sensors staged at a time, bytes of one sensor's
   // colour-phase planes (from offset 0) and the offset of the position tables
   int mean_p, mean_size, mean_axis, mean_lx, mean_ly, mean_bufs;
+  int mean_comp;                 // compensated sums
   int mean_y0, mean_y1;          // output rows of the launch (lpa_mean_rows)
   uint32_t mean_plane, mean_tab;
 };

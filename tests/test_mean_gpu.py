@@ -170,3 +170,19 @@ def test_larger_tiles_and_every_entry_point(ctx, w, h, rot):
         own.close()
     np.testing.assert_array_equal(o, out)
     np.testing.assert_array_equal(c, ch)
+
+
+@pytest.mark.parametrize("rot", [0.0, 0.3])
+@pytest.mark.parametrize("scale,shear", [(1.0, 0.0), (1.5, 0.0), (1.5, 0.05)])
+@pytest.mark.parametrize("sigma", [0.7, 1.2])
+def test_compensated_sums(ctx, sigma, scale, shear, rot):
+    """accum 1 in every form and window size, around the 64 x 16 tiles of its two rows per thread."""
+    w, h = round(90 * scale) + 1, round(33 * scale)
+    fr = _frame(90, 33, rot, n=3, sigma=sigma, accum=1, out_w=w, out_h=h,
+                out_affine=np.array([[1 / scale, 0.0, 0.2], [0.0, 1 / scale, -0.1]]))
+    if shear:
+        for k, s in enumerate(fr.sensors):
+            s.affine = s.affine @ np.array([[1.0, shear, 0.0], [0.0, 1.0, 0.0], [0.0, 0.0, 1.0]])
+            s.raw = synth.simulate_raw(fr.scene, s, 1500, k)
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
