@@ -753,6 +753,46 @@ __device__ __forceinline__ void walk_sensor(const LpaSensorK &S, int4 pos, int c
   }
 }
 
+// walk_sensor for isotropic windows that reach less than N sensor px along both axes (at most N cells a row):
+// every lane takes the N x N block from its window's first cell (cells past its box lie outside its disc), so
+// that nothing is searched, converted or reduced over the warp. Offsets are formed as walk_sensor
+// forms them.
+template <int N, class Body>
+__device__ __forceinline__ void walk_small(const LpaSensorK &S, int4 pos, int c, float hx, float hy, int x0, int y0,
+                                           const unsigned char *smem, bool active, unsigned *status, Body &&body) {
+  const float fx = __int_as_float(pos.z), fy = __int_as_float(pos.w);
+  const int PW = S.box_w >> 1, PH = S.box_h >> 1;
+  const float2 *planes = reinterpret_cast<const float2 *>(smem + S.off_planes);
+  const float a00 = S.A[0], a01 = S.A[1], a10 = S.A[2], a11 = S.A[3];
+  const float2 T2 = make_float2(2.f * a01, 2.f * a11), S2 = make_float2(2.f * a00, 2.f * a10);
+  const float fmx = floorf(0.5f * hx), fmy = floorf(0.5f * hy);
+  const int nsub = (c == 1) ? 2 : 1;
+#pragma unroll 1
+  for (int sub = 0; sub < nsub; sub++) {
+    const int ox = (c == 0) ? 0 : (c == 2 ? 1 : 1 - sub);
+    const int oy = (c == 0) ? 0 : (c == 2 ? 1 : sub);
+    const int lx = pos.x - x0 - ox, ly = pos.y - y0 - oy;
+    const float rx = (lx & 1) ? 1.f + fx : fx, ry = (ly & 1) ? 1.f + fy : fy;  // x0 and y0 are even
+    const float nx = (hx - rx) * 0.5f < fmx ? fmx - 1.f : fmx, ny = (hy - ry) * 0.5f < fmy ? fmy - 1.f : fmy;
+    const int pc = (lx >> 1) - (int)nx, pr = (ly >> 1) - (int)ny;
+    if (!active) continue;
+    if (!(pc >= 0 && pc + N <= PW && pr >= 0 && pr + N <= PH)) {  // the footprint is planned to hold every window
+      atomicOr(status, LPA_ERR_BOUNDS);
+      continue;
+    }
+    const float Dx0 = -2.f * nx - rx, Dy0 = -2.f * ny - ry;
+    const float2 DR0 = make_float2(fmaf(a00, Dx0, a01 * Dy0), fmaf(a10, Dx0, a11 * Dy0));
+    const float2 *rowp = planes + (ox + 2 * oy) * (PH * PW) + pr * PW + pc;
+    float rf = 0.f;
+#pragma unroll 1
+    for (int r = 0; r < N; r++, rowp += PW, rf += 1.f) {
+      float2 Dq = __ffma2_rn(make_float2(rf, rf), T2, DR0);
+#pragma unroll
+      for (int q = 0; q < N; q++, Dq = __fadd2_rn(Dq, S2)) body(Dq, rowp[q]);
+    }
+  }
+}
+
 template <int ORDER, int MODE, class MOM>
 __device__ __forceinline__ void accumulate_sensor(MOM &m, const LpaSensorK &S,
                                                   int4 pos, int c, float R, float R2,
@@ -762,6 +802,16 @@ __device__ __forceinline__ void accumulate_sensor(MOM &m, const LpaSensorK &S,
   // two samples in flight pay off only for the long order-2 bodies (fully unrolled rows
   // dispatched on their length were measured slower)
   constexpr int kUnroll = ORDER == 2 ? 2 : 1;
+  if constexpr (lpa_mode_one(MODE)) {
+    auto cell = [&](float2 D, float2 fv) { window_cell<ORDER, MODE>(m, D, fv, R2, cexp, taper, Q); };
+    // small windows (at most N cells a row: reach below N px; the last candidate column lies less than 2 N -
+    // reach px past the point, inside the footprint's margin of LPA_MARGIN from a reach of N - 2 on).
+    // 1024 x 900, three sensors, sigma 1.2: order 1 172 -> 154 us, order 2 239 -> 228 us; the kernels of
+    // several scales, short of registers, ran slower with it
+    const float hx = R * S.hx_unit + 1e-3f, hy = R * S.hy_unit + 1e-3f, most = fmaxf(hx, hy), least = fminf(hx, hy);
+    if (most < 3.f && least >= 1.f) return walk_small<3>(S, pos, c, hx, hy, x0, y0, smem, active, status, cell);
+    if (most < 4.f && least >= 2.f) return walk_small<4>(S, pos, c, hx, hy, x0, y0, smem, active, status, cell);
+  }
   walk_sensor<MODE, kUnroll>(S, pos, c, R, x0, y0, smem, active, status, Q, [&](float2 D, float2 fv) {
     window_cell<ORDER, MODE>(m, D, fv, R2, cexp, taper, Q);
   });

@@ -58,3 +58,33 @@ def test_values_do_not_depend_on_the_variance_sums(ctx, order, translational, ac
         ctx.check()
         np.testing.assert_array_equal(c.cpu().numpy(), ch.cpu().numpy())
         np.testing.assert_array_equal(o.cpu().numpy(), out.cpu().numpy())
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("sigma,green,zoom", [(0.34, 1.0, 1.0), (0.67, 0.5, 1.0), (0.99, 0.7, 1.0), (1.0, 1.0, 1.0),
+                                              (1.33, 0.5, 1.0), (1.34, 0.76, 1.0), (0.7, 0.9, 0.55)])
+def test_window_sizes_of_the_fixed_walk(ctx, order, sigma, green, zoom):
+    """Windows on both sides of the reaches (1, 2, 3 and 4 px, also unequal on a stretched sensor) between which
+    single-scale kernels take a fixed block of cells: the same bits as the kernels that search every
+    window (two pixels per thread)."""
+    from paper_1308_4908_gb300 import hdr
+    fr = _frame(False, order)
+    if zoom != 1.0:
+        for s in fr.sensors:
+            s.affine = s.affine @ np.array([[zoom, 0.0, 0.0], [0.0, 1.0, 0.0], [0.0, 0.0, 1.0]])
+    p = dataclasses.replace(fr.params, order=order, sigmas=(sigma,), green_ratio=green, out_w=50, out_h=47)
+    ctx.set_rig(0, fr.sensors)
+    raws = [torch.from_numpy(s.raw).cuda() for s in fr.sensors]
+    got = []
+    for batch in (False, True):
+        out = torch.full((3, 47, 50), -7.0, device="cuda")
+        ch = torch.empty((3, 47, 50), dtype=torch.uint8, device="cuda")
+        if batch:
+            keep = [raws]
+            ctx.reconstruct_batch([ctx.frame(0, p, raws, out, ch, keep)], hdr.hdr_batch_config(16, 0, 1, 0, 2, 1))
+        else:
+            ctx.reconstruct(0, p, raws, out=out, choice=ch)
+        ctx.check()
+        got.append((out.cpu().numpy(), ch.cpu().numpy()))
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    np.testing.assert_array_equal(got[0][1], got[1][1])
