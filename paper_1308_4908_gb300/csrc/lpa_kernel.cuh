@@ -195,13 +195,15 @@ struct MomentsPacked {
     }
   }
   // one sample with its monomials s, weight w = K / s2, w f and w K
-  __device__ __forceinline__ void adds(const float (&s)[15], float2 D, float2 D2, float w, float wf, float wk) {
+  // (`one` is 1, or 0 for a sample that is not counted, whose weight is 0)
+  __device__ __forceinline__ void adds(const float (&s)[15], float2 D, float2 D2, float w, float wf, float wk,
+                                       float one = 1.f) {
     const float2 W = make_float2(w, wk);
     ak[0] = __fadd2_rn(ak[0], W);
 #pragma unroll
     for (int i = 1; i < NA; i++) ak[i] = __ffma2_rn(W, make_float2(s[i], s[i]), ak[i]);
     const float2 F = make_float2(wf, wf);
-    b0n = __fadd2_rn(b0n, make_float2(wf, 1.f));
+    b0n = __fadd2_rn(b0n, make_float2(wf, one));
     b12 = __ffma2_rn(F, D, b12);
     if (NB > 3) {
       b35 = __ffma2_rn(F, D2, b35);
@@ -649,28 +651,38 @@ __device__ __forceinline__ void window_cell_ms(MOM (&m)[NSP], float2 D, float2 f
   constexpr bool LIT = MODE == LPA_LITERAL;
   const float2 D2 = __fmul2_rn(D, D);
   const float r2 = STEER ? fmaf(Q.x, D2.x, fmaf(Q.z, D2.y, 2.f * Q.y * (D.x * D.y))) : D2.x + D2.y;
-  if (!(r2 < R2[NSP - 1] && sample_ok(fv))) return;
+  // Orders 0 and 1: excluded samples (weight 0: they add exact zeros) are only left out of the count, so that
+  // the branch does not wait for the staged value (1.5x order-1 frame 2839 -> 2800 us; at order 2, whose
+  // monomials would be formed for them too, +0.7 %)
+  constexpr bool LATE = ORDER <= 1;
+  if (!(r2 < R2[NSP - 1] && (LATE || sample_ok(fv)))) return;
+  const float one = !LATE || sample_ok(fv) ? 1.f : 0.f;
   float sm[15];
   if constexpr (ORDER > 0) MOM::monomials(D, D2, sm);
-  // two scales per walk (order 2): both window values first, in one paired multiply and add (the
-  // same roundings as one at a time), so that their ex2 latencies overlap (-1 %; with four scales
-  // per walk the values of scales that miss the sample cost more than that)
+  // Window values of two scales at a time, in one paired multiply and add (the same roundings as one at a
+  // time), so that their ex2 latencies overlap: both of a two-scale walk (order 2, -1 %), and the pairs of a
+  // four-scale walk at order 0 (mixed batch 21.70 -> 21.56 ms; at order 1 the values of scales that miss
+  // the sample cost more, +0.7 %)
+  constexpr bool PAIRS = NSP == 2 || (NSP == 4 && ORDER == 0);
   float Kq[NSP];
-  if constexpr (NSP == 2) {
-    const float2 A = __fmul2_rn(make_float2(r2, r2), make_float2(cexp[0], cexp[1]));
+  auto two = [&](int q) {
+    const float2 A = __fmul2_rn(make_float2(r2, r2), make_float2(cexp[q - 1], cexp[q]));
     const float2 E = __fadd2_rn(make_float2(ex2_approx(A.x), ex2_approx(A.y)), make_float2(-taper, -taper));
-    Kq[0] = E.x;
-    Kq[1] = E.y;
-  }
+    Kq[q - 1] = E.x;
+    Kq[q] = E.y;
+  };
+  if constexpr (PAIRS) two(NSP - 1);
   // largest scale first; the windows are nested, so the first one that misses ends the loop
   // (a loop with an exit, not a chain of tests: no reconvergence point per scale)
 #pragma unroll
   for (int q = NSP - 1; q >= 0; q--) {
     if (!(r2 < R2[q])) break;
-    const float K = NSP == 2 ? Kq[q] : ex2_approx(r2 * cexp[q]) - taper;
+    if constexpr (PAIRS && NSP == 4)
+      if (q == 1) two(1);
+    const float K = PAIRS ? Kq[q] : ex2_approx(r2 * cexp[q]) - taper;
     const float2 W = weights(K, fv);
-    if constexpr (ORDER == 0) m[q].add0(W.x, W.y, (LIT ? K : W.x) * K, 1.f);
-    else m[q].adds(sm, D, D2, W.x, W.y, (LIT ? K : W.x) * K);
+    if constexpr (ORDER == 0) m[q].add0(W.x, W.y, (LIT ? K : W.x) * K, one);
+    else m[q].adds(sm, D, D2, W.x, W.y, (LIT ? K : W.x) * K, one);
   }
 }
 
