@@ -399,6 +399,11 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *
     invert_affine(rig.s[s].d.affine, t);
     compose_affine(t, p->out_affine, G);
     if (!(std::fabs(G[0]) + std::fabs(G[1]) + std::fabs(G[3]) + std::fabs(G[4]) < 16.0)) return 0;
+    // box_origin forms a tile's origin in FP32: off by less than half a px (the box's margin is one) while
+    // no term exceeds 2^20 px; outputs or offsets beyond keep the general kernel's FP64 origin
+    const double W = p->out_w, H = p->out_h;
+    if (!(std::fabs(G[0]) * W + std::fabs(G[1]) * H + std::fabs(G[2]) < 1048576.0 &&
+          std::fabs(G[3]) * W + std::fabs(G[4]) * H + std::fabs(G[5]) < 1048576.0)) return 0;
     int bw, bh;
     float ex, ey;
     mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);

@@ -186,3 +186,15 @@ def test_compensated_sums(ctx, sigma, scale, shear, rot):
             s.raw = synth.simulate_raw(fr.scene, s, 1500, k)
     out, ch, _ = _run(ctx, fr)
     _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
+@pytest.mark.parametrize("shift,w", [(-9.0e6, 9_000_064), (-5.0e5, 500_064)])
+def test_far_coordinates(ctx, shift, w):
+    """Sensors that only the last pixels of a very wide output reach: the terms of a position are
+    large there and cancel, on both sides of the line up to which FP32 box origins serve."""
+    fr = _frame(64, 8, 0.3)
+    fr = dataclasses.replace(fr, params=dataclasses.replace(fr.params, out_w=w, out_h=2, out_affine=(0.9999, 0, 0.9999 * shift, 0, 0.9999, 0)))
+    out, ch, _ = _run(ctx, fr)
+    pix = _every_pixel(dataclasses.replace(fr.params, out_w=96)) + [w - 96, 0]
+    assert np.isfinite(out[:, pix[:, 1], pix[:, 0]]).mean() > 0.5
+    _against_oracle(fr, out, ch, pix)
