@@ -164,18 +164,19 @@ __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__
   float L1 = l1.x * up, L2 = fmaxf(l2.x, 0.f) * up;
   // Nearly rank one: the pairs hold l2 to about 2^-45 l1, less than an FP32 value needs below this
   // ratio (noise keeps it above in camera frames; a lone gradient or a clean ramp is below), so T and
-  // its eigenvalues are formed again in FP64.
-  if (l2.x < 0x1p-18f * l1.x) {
+  // its eigenvalues are formed again in FP64, from the gradients: sums that left FP32's range (not a
+  // number here) come this way too.
+  if (!(l2.x >= 0x1p-18f * l1.x)) {
     double da = 0.0, db = 0.0, dc = 0.0;
-    for (int dj = -r; dj <= r; dj++) {
-      const int rw = A.rw[dj + r], at = mid + dj * TW;
-      for (int di = -rw; di <= rw; di++) {
-        const float2 wp = A.w[di * di + dj * dj], x = sx[at + di];
-        const float4 q = sd[at + di];
-        const double w = (double)wp.x + (double)wp.y;
-        da = fma(w, (double)q.x + (double)q.z, da);
-        db = fma(w, (double)x.x + (double)x.y, db);
-        dc = fma(w, (double)q.y + (double)q.w, dc);
+    for (int dj = max(-r, -v); dj <= min(r, A.H - 1 - v); dj++) {
+      const int rw = A.rw[dj + r];
+      const float2 *row = A.grad + (size_t)(v + dj) * A.W + u;
+      for (int di = max(-rw, -u); di <= min(rw, A.W - 1 - u); di++) {
+        const float2 wp = A.w[di * di + dj * dj], g = row[di];
+        const double w = (double)wp.x + (double)wp.y, gx = (double)(g.x * A.unit), gy = (double)(g.y * A.unit);
+        da = fma(w, gx * gx, da);
+        db = fma(w, gx * gy, db);
+        dc = fma(w, gy * gy, dc);
       }
     }
     const double m2 = ((double)A.m2.x + (double)A.m2.y) * (double)down;

@@ -317,6 +317,19 @@ def test_metric_windows_and_near_rank_one(ctx, window_sigma, grad_scale):
                                            c.min_eig, c.max_eig, c.grad_scale))
 
 
+@pytest.mark.parametrize("window_sigma,size", [(1.0, 3e19), (1.06, 1e25), (1.0, 1e15)])
+def test_metric_of_huge_gradients(ctx, window_sigma, size):
+    """Gradients whose squares, or their sums, leave FP32's range give matrices inside the clamp, as
+    smaller ones do, and no NaN."""
+    r = np.random.default_rng(11)
+    g = (size * r.standard_normal((37, 45, 2))).astype(np.float32)
+    g[20:, 20:] = 0.0
+    c = _calpa(window_sigma=window_sigma, grad_scale=1.0)
+    q = ctx.calpa_metric(c, torch.from_numpy(g).cuda()).cpu().numpy().astype(np.float64)
+    eig = np.linalg.eigvalsh(np.stack([q[..., [0, 1]], q[..., [1, 2]]], axis=-2))
+    assert eig.min() >= c.min_eig * (1 - 1e-5) and eig.max() <= c.max_eig * (1 + 1e-5)
+
+
 @pytest.mark.parametrize("w,h,scale,grad_sigma", [(1, 1, 1.0, 1.2), (63, 15, 1.0, 0.6), (65, 17, 1.0, 1.2),
                                                    (130, 33, 1.5, 1.8), (96, 48, 2.0, 1.2), (40, 30, 0.6, 1.0),
                                                    (65, 17, 1.0, 2.0)])
