@@ -287,6 +287,7 @@ struct PlanEnv {
   bool mean = true;    // small windows of order 0 may run lpa_mean (not the level maps, whose kernel also
                        // writes Var C_0, nor the persistent batch kernels)
   bool grad = false;   // the gradient pass: lpa_grad where its windows are small enough
+  bool ahead = true;   // the general kernel would read frames of a wave of tiles or more converted ahead
 };
 
 bool is_identity_linear(const double *a) {
@@ -608,6 +609,41 @@ hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p,
   return HDR_OK;
 }
 
+// Staging box of the general kernels for sensor transform G: the tile's pixel points span |G_lin| *
+// (TILE-1) in sensor space; add the largest window's half extent plus margin on both sides, the floor of
+// the origin and the alignment of the origin (x to 8 elements = 16 bytes, y to 2).
+void general_box(const double G[6], double hxu, double hyu, double rmax, int tile_h, float *ext_x, float *ext_y, int *bw, int *bh) {
+  *ext_x = (float)(rmax * hxu + LPA_MARGIN);
+  *ext_y = (float)(rmax * hyu + LPA_MARGIN);
+  const double span_x = std::fabs(G[0]) * (LPA_TILE - 1) + std::fabs(G[1]) * (tile_h - 1);
+  const double span_y = std::fabs(G[3]) * (LPA_TILE - 1) + std::fabs(G[4]) * (tile_h - 1);
+  *bw = ((int)std::ceil(span_x + 2.0 * *ext_x) + 9 + 7) / 8 * 8;
+  *bh = ((int)std::ceil(span_y + 2.0 * *ext_y) + 3 + 1) / 2 * 2;
+}
+
+// Whether the general kernel's staging takes a frame of these parameters (what lpa_mean and lpa_grad could
+// stage beyond that stays refused): its boxes within 256 and its shared memory, with one staging buffer.
+bool general_fits(const PlanEnv &env, const Rig &rig, const hdr_params *p, double rmax, int tile_h, int stages, int max_smem) {
+  const bool conv = env.tabs && env.ahead && stages != 2 && LPA_FRAME_CONV && (long long)p->out_w * p->out_h >= 152LL * 256;
+  bool tab = env.tabs && env.tabulate && p->tab_weights == 1 && is_identity_linear(p->out_affine);
+  long long off = 0;
+  for (int s = 0; s < rig.n; s++) {
+    double t[6], G[6];
+    invert_affine(rig.s[s].d.affine, t);
+    compose_affine(t, p->out_affine, G);
+    float ex, ey;
+    int bw, bh;
+    general_box(G, std::sqrt(t[0] * t[0] + t[1] * t[1]), std::sqrt(t[3] * t[3] + t[4] * t[4]), rmax, tile_h, &ex, &ey, &bw, &bh);
+    if (bw > 256 || bh > 256) return false;
+    off = (off + 127) / 128 * 128;
+    if (!conv) off = (off + (long long)bw * bh * 2 + 127) / 128 * 128;
+    off += (long long)bw * bh * 8;
+    tab = tab && is_identity_linear(rig.s[s].d.affine);
+  }
+  if (!tab) off = (off + 15) / 16 * 16 + (long long)rig.n * 16 * LPA_TILE * tile_h;
+  return off <= max_smem - 1024;
+}
+
 #ifndef LPA_FRAME_TILE_H
 #define LPA_FRAME_TILE_H 16  // tile height of single-frame launches
 #endif
@@ -643,13 +679,16 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   const double rmax = reach * p->trunc_k * p->sigma[p->n_scales - 1] * std::fmax(1.0, p->green_ratio);
   uint32_t off = 0, tx = 0;
   size_t conv_off = 0;
+  int max_smem = 0;
+  CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, env.device));
   MeanPlan mean;
   if (env.mean) mean = mean_plan(rig, p);
   if (env.grad) mean = grad_plan(rig, p);
   if (mean.size >= 0) {
     L.smem_bytes = mean_smem(rig, p, mean, &L.mean_bufs, &L.mean_plane, &L.mean_tab);
     // (lpa_grad stages every sensor at once)
-    if (L.smem_bytes == 0 || (env.grad && L.mean_bufs < rig.n)) mean.size = -1;
+    if (L.smem_bytes == 0 || (env.grad && L.mean_bufs < rig.n) || !general_fits(env, rig, p, rmax, tile_h, stages, max_smem))
+      mean.size = -1;
   }
   if (mean.size >= 0) conv = nullptr;  // lpa_mean and lpa_grad read the raw frames
   L.conv = conv ? 1 : 0;
@@ -693,17 +732,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
       K.group_magic = (uint32_t)(((1ull << 32) + K.box_w / 8 - 1) / (K.box_w / 8));
       continue;
     }
-    // staging box: the tile's pixel points span |G_lin| * (TILE-1) in sensor space; add the
-    // largest window's half extent plus margin on both sides, the floor of the origin and
-    // the alignment of the origin (x to 8 elements = 16 bytes, y to 2)
-    K.ext_x = (float)(rmax * hxu + LPA_MARGIN);
-    K.ext_y = (float)(rmax * hyu + LPA_MARGIN);
-    const double span_x = std::fabs(K.G[0]) * (LPA_TILE - 1) + std::fabs(K.G[1]) * (tile_h - 1);
-    const double span_y = std::fabs(K.G[3]) * (LPA_TILE - 1) + std::fabs(K.G[4]) * (tile_h - 1);
-    int bw = (int)std::ceil(span_x + 2.0 * K.ext_x) + 9;
-    int bh = (int)std::ceil(span_y + 2.0 * K.ext_y) + 3;
-    bw = (bw + 7) / 8 * 8;
-    bh = (bh + 1) / 2 * 2;
+    int bw, bh;
+    general_box(K.G, hxu, hyu, rmax, tile_h, &K.ext_x, &K.ext_y, &bw, &bh);
     if (bw > 256 || bh > 256)
       return fail(HDR_E_UNSUPPORTED, "sensor %d staging box %dx%d exceeds 256 (window or output scale too large)", s, bw, bh);
     K.box_w = bw;
@@ -808,8 +838,6 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     L.off_pos = off;
     off += (uint32_t)(rig.n * 16 * LPA_TILE * tile_h);
   }
-  int max_smem = 0;
-  CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, env.device));
   L.stages = 1;
   for (int s = 0; s < rig.n; s++) L.s[s].off_raw2 = L.s[s].off_raw;
   if (stages == 2 && !conv && lpa_stages2_built(L.mode, p->accum != 0)) {
@@ -833,8 +861,9 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
 }
 
 hdr_status plan(hdr_ctx *ctx, const Rig &rig, const hdr_params *p, const uint16_t *const *raw, LpaLaunch &L,
-                double reach = 1.0, bool levels = false, int stages = 1, float2 *conv = nullptr, bool grad = false) {
-  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels, !levels, grad}, rig, p, raw, L,
+                double reach = 1.0, bool levels = false, int stages = 1, float2 *conv = nullptr, bool grad = false,
+                bool ahead = true) {
+  return plan_env(PlanEnv{ctx->encode, ctx->status, ctx->device, &ctx->tabs, !levels, !levels, !levels, grad, ahead}, rig, p, raw, L,
                   LPA_FRAME_TILE_H, reach, stages, conv);
 }
 
@@ -1851,8 +1880,8 @@ hdr_status lpa_launch_mode(hdr_ctx *ctx, int32_t rig_id, const hdr_params *param
     int bufs = 0;
     const MeanPlan m = grad_plan(rig, &p);
     if (m.size >= 0 && mean_smem(rig, &p, m, &bufs, &plane, &tab) > 0 && bufs == rig.n) {
-      s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, nullptr, true);
-      if (s) return s;
+      s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, nullptr, true, ahead);
+      if (s) return s;  // (refused where the general kernel refuses)
       if (L.out_w == 0 || L.out_h == 0) return HDR_OK;
       L.aux = aux;
       const bool f64 = p.cond_fallback > 0.0 && (p.min_pivot - 1e-4) * p.cond_fallback < 2.0;

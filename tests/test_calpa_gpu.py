@@ -360,3 +360,19 @@ def test_gradient_tiles_and_windows(ctx, w, h, scale, grad_sigma):
                             flat.data_ptr() + 4, torch.cuda.current_stream().cuda_stream)
     ctx.check()
     np.testing.assert_array_equal(flat[1:].cpu().numpy(), g.cpu().numpy().ravel())
+
+
+def test_gradients_refused_as_by_the_general_kernel(ctx):
+    """Red and blue windows far wider than green's outgrow the general kernel's staging: refused, although
+    the gradient pass's own kernel reads green alone."""
+    import dataclasses
+    from paper_1308_4908_gb300 import hdr
+    p = synth.Params(order=2, sigmas=(0.8, 1.2), out_w=40, out_h=30, green_ratio=0.15)
+    fr = synth._build_frame(1801, 8, 48, 40, [1.0] * 8, 1.2, 0.4, 0.0, p, "grad")
+    ctx.set_rig(0, fr.sensors)
+    for grad_sigma, ok in ((1.2, True), (7.0, False)):
+        try:
+            ctx.calpa_gradients(0, p, _calpa(grad_sigma=grad_sigma), _raws(fr))
+            assert ok
+        except hdr.HdrError as e:
+            assert not ok and e.status == hdr.HDR_E_UNSUPPORTED

@@ -198,3 +198,21 @@ def test_far_coordinates(ctx, shift, w):
     pix = _every_pixel(dataclasses.replace(fr.params, out_w=96)) + [w - 96, 0]
     assert np.isfinite(out[:, pix[:, 1], pix[:, 0]]).mean() > 0.5
     _against_oracle(fr, out, ch, pix)
+
+
+@pytest.mark.parametrize("n,reduce,rot", [(8, 1.0, 0.3), (8, 2.0, 0.3), (8, 2.6, 0.0), (8, 3.2, 0.3), (4, 4.0, 0.3), (2, 6.0, 0.3), (1, 7.0, 0.0)])
+def test_refused_as_by_the_general_kernel(ctx, n, reduce, rot):
+    """Outputs that outgrow the general kernel's staging (order 1 has the same) are refused at order 0
+    too, although its own kernel could stage the sensors in turn."""
+    from paper_1308_4908_gb300 import hdr
+    fr = _frame(96, 64, rot, n=n, out_w=40, out_h=30, out_affine=np.array([[reduce, 0, 1.0], [0, reduce, 0.5]]))
+    refused = []
+    for order in (0, 1):
+        try:
+            _run(ctx, dataclasses.replace(fr, params=dataclasses.replace(fr.params, order=order)))
+            refused.append(0)
+        except hdr.HdrError as e:
+            refused.append(e.status)
+    assert refused[0] == refused[1] and refused[0] in (0, hdr.HDR_E_UNSUPPORTED)
+    if (n, reduce) in ((8, 1.0), (8, 3.2)):
+        assert (refused[0] == 0) == (reduce == 1.0)
