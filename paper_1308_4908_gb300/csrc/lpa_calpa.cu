@@ -64,45 +64,26 @@ __device__ __forceinline__ float2 pair_sqrt(float2 a) {  // a >= 0
 // pairs too; what follows them (square roots, the direction's normalisation, elongation, the power
 // and the matrix) has no cancellation and runs in FP32.
 //
-// Bound by the FP32 pipe: 36 pipe cycles per warp and disc cell (12 operations on each of three
+// Bound by the FP32 pipe: 36 pipe cycles per warp and weighted term (12 operations on each of three
 // sums, gx^2 and gy^2 side by side in paired instructions). The same sums in FP64 kept the FP64
 // pipe 84 % busy: gradients and matrices of 1920 x 1080 with 29 cells took 751 us, with this kernel
 // and looped discs 324 us.
 //
-// UNIT: the disc of window_sigma 1 (radius 3: half widths 0, 2, 2, 3, 2, 2, 0), unrolled, so that a
-// cell is its two loads and its arithmetic (the loops over any disc issued 65 instructions a cell: 130 us
-// for 1920 x 1080, unrolled 101 us).
+// UNIT: the disc of window_sigma 1 (radius 3: half widths 0, 2, 2, 3, 2, 2, 0). The Gaussian factors, so the
+// rows of a 32 x 16 block are summed along x first (over half widths 2 and 3, into shared memory) and
+// those sums along y: 14 weighted terms a pixel instead of 28 (gradients and matrices of 1920 x 1080: 212 us
+// with the 29 cells unrolled, 183 us so). Four CTAs per SM at 47 KB and 64 registers.
+constexpr int kUnitBY = 16, kUnitR = 3;
 __host__ __device__ constexpr int unit_row(int dj) { return dj == 0 ? 3 : dj == 3 || dj == -3 ? 0 : 2; }
-template <bool UNIT>
-__global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__ MetricArgs A) {
-  extern __shared__ __align__(16) float4 sm[];
-  const int r = UNIT ? 3 : A.r, TW = kBX + 2 * r, TH = kBY + 2 * r;
-  float4 *sd = sm;                                        // (gx^2, gy^2, their residuals)
-  float2 *sx = reinterpret_cast<float2 *>(sm + TW * TH);  // (gx gy, its residual)
-  // one-dimensional grid over the 32 x 8 blocks (any output height)
-  const int nbx = (A.W + kBX - 1) / kBX;
-  const int bx0 = (int)(blockIdx.x % nbx) * kBX, by0 = (int)(blockIdx.x / nbx) * kBY;
-  for (int ty = threadIdx.y; ty < TH; ty += kBY) {
-    const int Y = by0 - r + ty;
-    const float2 *row = A.grad + (size_t)max(Y, 0) * A.W;
-    for (int tx = threadIdx.x; tx < TW; tx += kBX) {
-      const int X = bx0 - r + tx;
-      float2 g = (X >= 0 && X < A.W && Y >= 0 && Y < A.H) ? row[X] : make_float2(0.f, 0.f);
-      g = make_float2(g.x * A.unit, g.y * A.unit);
-      const float xx = __fmul_rn(g.x, g.x), yy = __fmul_rn(g.y, g.y), xy = __fmul_rn(g.x, g.y);
-      sd[ty * TW + tx] = make_float4(xx, yy, __fmaf_rn(g.x, g.x, -xx), __fmaf_rn(g.y, g.y, -yy));
-      sx[ty * TW + tx] = make_float2(xy, __fmaf_rn(g.x, g.y, -xy));
-    }
-  }
-  __syncthreads();
-  const int u = bx0 + threadIdx.x, v = by0 + threadIdx.y;
-  if (u >= A.W || v >= A.H) return;
-  const float2 minus = make_float2(-1.f, -1.f);
-  float2 S = make_float2(0.f, 0.f), E = S;  // (sum w gx^2, sum w gy^2) and what rounding dropped
-  float s = 0.f, e = 0.f;                   // the same of sum w gx gy
-  auto add = [&](float2 w, int at) {
-    const float4 d = sd[at];
-    const float2 x = sx[at];
+
+// T's sums in pairs: (sum w gx^2, sum w gy^2) and sum w gx gy, with what rounding dropped.
+struct DiscSum {
+  float2 S, E;
+  float s, e;
+  __device__ __forceinline__ DiscSum() : S(make_float2(0.f, 0.f)), E(make_float2(0.f, 0.f)), s(0.f), e(0.f) {}
+  __device__ __forceinline__ DiscSum(float4 d, float2 x) : S(make_float2(d.x, d.y)), E(make_float2(d.z, d.w)), s(x.x), e(x.y) {}
+  __device__ __forceinline__ void add(float2 w, float4 d, float2 x) {
+    const float2 minus = make_float2(-1.f, -1.f);
     {
       const float2 X = make_float2(d.x, d.y), W = make_float2(w.x, w.x);
       const float2 P = __fmul2_rn(W, X);
@@ -122,23 +103,15 @@ __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__
       e = __fadd_rn(e, __fadd_rn(__fadd_rn(k, __fsub_rn(p, z)), q));
       s = t;
     }
-  };
-  const int mid = (threadIdx.y + r) * TW + threadIdx.x + r;
-  if constexpr (UNIT) {
-    float2 w[10];
-#pragma unroll
-    for (int k = 0; k < 10; k++) w[k] = A.w[k];
-#pragma unroll
-    for (int dj = -3; dj <= 3; dj++)
-#pragma unroll
-      for (int di = -unit_row(dj); di <= unit_row(dj); di++) add(w[di * di + dj * dj], mid + dj * TW + di);
-  } else {
-    for (int dj = -r; dj <= r; dj++) {
-      const int rw = A.rw[dj + r];
-#pragma unroll 2
-      for (int di = -rw; di <= rw; di++) add(A.w[di * di + dj * dj], mid + dj * TW + di);
-    }
   }
+  __device__ __forceinline__ float4 d() const { return make_float4(S.x, S.y, E.x, E.y); }
+  __device__ __forceinline__ float2 x() const { return make_float2(s, e); }
+};
+
+// The eigenvalues of T and the steering matrix of pixel (u, v).
+__device__ __forceinline__ void store_matrix(const MetricArgs &A, int r, const DiscSum &D, int u, int v) {
+  const float2 S = D.S, E = D.E;
+  const float s = D.s, e = D.e;
   int M = A.cells;
   if (u < r || v < r || u + r >= A.W || v + r >= A.H) {  // disc cells inside the image
     M = 0;
@@ -211,6 +184,77 @@ __global__ void __launch_bounds__(kBX *kBY) calpa_metric(const __grid_constant__
   o[0] = ea * ux * ux + eb * uy * uy;
   o[1] = (ea - eb) * ux * uy;
   o[2] = ea * uy * uy + eb * ux * ux;
+}
+
+template <bool UNIT>
+__global__ void __launch_bounds__(kBX *kBY, UNIT ? 4 : 1) calpa_metric(const __grid_constant__ MetricArgs A) {
+  extern __shared__ __align__(16) float4 sm[];
+  constexpr int BY = UNIT ? kUnitBY : kBY;
+  const int r = UNIT ? kUnitR : A.r, TW = kBX + 2 * r, TH = BY + 2 * r;
+  float4 *sd = sm;                                        // (gx^2, gy^2, their residuals)
+  float2 *sx = reinterpret_cast<float2 *>(sm + TW * TH);  // (gx gy, its residual)
+  // one-dimensional grid over the blocks (any output height)
+  const int nbx = (A.W + kBX - 1) / kBX;
+  const int bx0 = (int)(blockIdx.x % nbx) * kBX, by0 = (int)(blockIdx.x / nbx) * BY;
+  for (int ty = threadIdx.y; ty < TH; ty += kBY) {
+    const int Y = by0 - r + ty;
+    const float2 *row = A.grad + (size_t)max(Y, 0) * A.W;
+    for (int tx = threadIdx.x; tx < TW; tx += kBX) {
+      const int X = bx0 - r + tx;
+      float2 g = (X >= 0 && X < A.W && Y >= 0 && Y < A.H) ? row[X] : make_float2(0.f, 0.f);
+      g = make_float2(g.x * A.unit, g.y * A.unit);
+      const float xx = __fmul_rn(g.x, g.x), yy = __fmul_rn(g.y, g.y), xy = __fmul_rn(g.x, g.y);
+      sd[ty * TW + tx] = make_float4(xx, yy, __fmaf_rn(g.x, g.x, -xx), __fmaf_rn(g.y, g.y, -yy));
+      sx[ty * TW + tx] = make_float2(xy, __fmaf_rn(g.x, g.y, -xy));
+    }
+  }
+  __syncthreads();
+  const int u = bx0 + threadIdx.x, mid = threadIdx.x + r;
+  if constexpr (UNIT) {
+    constexpr int H = kUnitBY + 2 * kUnitR - 2;  // rows from the second staged one to the last but one
+    float4 *d2 = reinterpret_cast<float4 *>(sx + TW * TH), *d3 = d2 + H * kBX;  // row sums over |di| <= 2, <= 3
+    float2 *x2 = reinterpret_cast<float2 *>(d3 + kUnitBY * kBX), *x3 = x2 + H * kBX;
+    const float2 w1 = A.w[1], w4 = A.w[4], w9 = A.w[9];
+#pragma unroll 1
+    for (int y = threadIdx.y; y < H; y += kBY) {
+      const int at = (y + 1) * TW + mid, to = y * kBX + threadIdx.x;
+      DiscSum a(sd[at], sx[at]);
+      a.add(w1, sd[at - 1], sx[at - 1]);
+      a.add(w1, sd[at + 1], sx[at + 1]);
+      a.add(w4, sd[at - 2], sx[at - 2]);
+      a.add(w4, sd[at + 2], sx[at + 2]);
+      d2[to] = a.d();
+      x2[to] = a.x();
+      if (y < kUnitR - 1 || y > H - kUnitR) continue;
+      a.add(w9, sd[at - 3], sx[at - 3]);
+      a.add(w9, sd[at + 3], sx[at + 3]);
+      d3[to - (kUnitR - 1) * kBX] = a.d();
+      x3[to - (kUnitR - 1) * kBX] = a.x();
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int y = threadIdx.y; y < kUnitBY; y += kBY) {
+      const int at = (y + kUnitR - 1) * kBX + threadIdx.x, up = y * TW + mid, dn = up + 2 * kUnitR * TW;
+      DiscSum a(d3[y * kBX + threadIdx.x], x3[y * kBX + threadIdx.x]);
+      a.add(w1, d2[at - kBX], x2[at - kBX]);
+      a.add(w1, d2[at + kBX], x2[at + kBX]);
+      a.add(w4, d2[at - 2 * kBX], x2[at - 2 * kBX]);
+      a.add(w4, d2[at + 2 * kBX], x2[at + 2 * kBX]);
+      a.add(w9, sd[up], sx[up]);
+      a.add(w9, sd[dn], sx[dn]);
+      if (u < A.W && by0 + y < A.H) store_matrix(A, kUnitR, a, u, by0 + y);
+    }
+  } else {
+    const int v = by0 + threadIdx.y;
+    if (u >= A.W || v >= A.H) return;
+    DiscSum a;
+    for (int dj = -r; dj <= r; dj++) {
+      const int rw = A.rw[dj + r], at = (threadIdx.y + r + dj) * TW + mid;
+#pragma unroll 2
+      for (int di = -rw; di <= rw; di++) a.add(A.w[di * di + dj * dj], sd[at + di], sx[at + di]);
+    }
+    store_matrix(A, r, a, u, v);
+  }
 }
 
 hdr_status check_calpa(const hdr_calpa_params *c) {
@@ -317,10 +361,13 @@ hdr_status hdr_calpa_metric(hdr_ctx *ctx, int32_t out_w, int32_t out_h, const hd
   A.lambda2 = (float)calpa->lambda2;
   A.min_eig = (float)calpa->min_eig;
   A.max_eig = (float)calpa->max_eig;
-  const unsigned blocks = (unsigned)(((long long)out_w + kBX - 1) / kBX * (((long long)out_h + kBY - 1) / kBY));
-  const size_t smem = (size_t)(kBX + 2 * A.r) * (kBY + 2 * A.r) * (sizeof(float4) + sizeof(float2));  // at most 35 KB
-  bool unit = A.r == 3;
-  for (int dj = -3; dj <= 3 && unit; dj++) unit = A.rw[dj + 3] == unit_row(dj);
+  bool unit = A.r == kUnitR;
+  for (int dj = -kUnitR; dj <= kUnitR && unit; dj++) unit = A.rw[dj + kUnitR] == unit_row(dj);
+  const int by = unit ? kUnitBY : kBY;
+  const unsigned blocks = (unsigned)(((long long)out_w + kBX - 1) / kBX * (((long long)out_h + by - 1) / by));
+  size_t px = (size_t)(kBX + 2 * A.r) * (by + 2 * A.r);          // at most 35 KB
+  if (unit) px += (size_t)kBX * (2 * kUnitBY + 2 * kUnitR - 2);  // and the row sums: 46.6 KB
+  const size_t smem = px * (sizeof(float4) + sizeof(float2));
   if (unit) calpa_metric<true><<<blocks, dim3(kBX, kBY), smem, (cudaStream_t)cuda_stream>>>(A);
   else calpa_metric<false><<<blocks, dim3(kBX, kBY), smem, (cudaStream_t)cuda_stream>>>(A);
   cudaError_t e = cudaGetLastError();

@@ -317,6 +317,17 @@ def test_metric_windows_and_near_rank_one(ctx, window_sigma, grad_scale):
                                            c.min_eig, c.max_eig, c.grad_scale))
 
 
+@pytest.mark.parametrize("w,h", [(3, 3), (31, 15), (32, 16), (33, 17), (3, 40), (70, 5)])
+def test_metric_tile_edges(ctx, w, h):
+    """The default disc, summed along x and then y, around its 32 x 16 blocks."""
+    r = np.random.default_rng(100 * w + h)
+    g = (10.0 ** r.uniform(0.0, 2.0, (h, w, 1)) * r.standard_normal((h, w, 2))).astype(np.float32)
+    c = _calpa()
+    q = ctx.calpa_metric(c, torch.from_numpy(g).cuda()).cpu().numpy()
+    check_metric(q, oracle.steering_metric(g.astype(np.float64), c.window_sigma, c.alpha, c.lambda1, c.lambda2,
+                                           c.min_eig, c.max_eig, c.grad_scale))
+
+
 @pytest.mark.parametrize("window_sigma,size", [(1.0, 3e19), (1.06, 1e25), (1.0, 1e15)])
 def test_metric_of_huge_gradients(ctx, window_sigma, size):
     """Gradients whose squares, or their sums, leave FP32's range give matrices inside the clamp, as
