@@ -71,8 +71,8 @@ __device__ __forceinline__ float2 pair_sqrt(float2 a) {  // a >= 0
 //
 // UNIT: the disc of window_sigma 1 (radius 3: half widths 0, 2, 2, 3, 2, 2, 0). The Gaussian factors, so the
 // rows of a 32 x 16 block are summed along x first (over half widths 2 and 3, into shared memory) and
-// those sums along y: 14 weighted terms a pixel instead of 28 (gradients and matrices of 1920 x 1080: 212 us
-// with the 29 cells unrolled, 183 us so). Four CTAs per SM at 47 KB and 64 registers.
+// those sums along y: 7 weighted terms a pixel instead of 28 (gradients and matrices of 1920 x 1080: 212 us
+// with the 29 cells unrolled, 183 us so, 179 with cells of equal weight added first). Four CTAs per SM at 47 KB and 64 registers.
 constexpr int kUnitBY = 16, kUnitR = 3;
 __host__ __device__ constexpr int unit_row(int dj) { return dj == 0 ? 3 : dj == 3 || dj == -3 ? 0 : 2; }
 
@@ -103,6 +103,16 @@ struct DiscSum {
       e = __fadd_rn(e, __fadd_rn(__fadd_rn(k, __fsub_rn(p, z)), q));
       s = t;
     }
+  }
+  // Two terms of one weight: added first (an error-free sum and what it dropped), then weighted once.
+  __device__ __forceinline__ void add(float2 w, float4 da, float2 xa, float4 db, float2 xb) {
+    const float2 minus = make_float2(-1.f, -1.f), A = make_float2(da.x, da.y), B = make_float2(db.x, db.y);
+    const float2 t = __fadd2_rn(A, B), z = __ffma2_rn(A, minus, t);
+    const float2 k = __fadd2_rn(__ffma2_rn(__ffma2_rn(z, minus, t), minus, A), __ffma2_rn(z, minus, B));
+    const float2 l = __fadd2_rn(__fadd2_rn(make_float2(da.z, da.w), make_float2(db.z, db.w)), k);
+    const float x = __fadd_rn(xa.x, xb.x), y = __fsub_rn(x, xa.x);
+    const float m = __fadd_rn(__fsub_rn(xa.x, __fsub_rn(x, y)), __fsub_rn(xb.x, y));
+    add(w, make_float4(t.x, t.y, l.x, l.y), make_float2(x, __fadd_rn(__fadd_rn(xa.y, xb.y), m)));
   }
   __device__ __forceinline__ float4 d() const { return make_float4(S.x, S.y, E.x, E.y); }
   __device__ __forceinline__ float2 x() const { return make_float2(s, e); }
@@ -219,15 +229,12 @@ __global__ void __launch_bounds__(kBX *kBY, UNIT ? 4 : 1) calpa_metric(const __g
     for (int y = threadIdx.y; y < H; y += kBY) {
       const int at = (y + 1) * TW + mid, to = y * kBX + threadIdx.x;
       DiscSum a(sd[at], sx[at]);
-      a.add(w1, sd[at - 1], sx[at - 1]);
-      a.add(w1, sd[at + 1], sx[at + 1]);
-      a.add(w4, sd[at - 2], sx[at - 2]);
-      a.add(w4, sd[at + 2], sx[at + 2]);
+      a.add(w1, sd[at - 1], sx[at - 1], sd[at + 1], sx[at + 1]);
+      a.add(w4, sd[at - 2], sx[at - 2], sd[at + 2], sx[at + 2]);
       d2[to] = a.d();
       x2[to] = a.x();
       if (y < kUnitR - 1 || y > H - kUnitR) continue;
-      a.add(w9, sd[at - 3], sx[at - 3]);
-      a.add(w9, sd[at + 3], sx[at + 3]);
+      a.add(w9, sd[at - 3], sx[at - 3], sd[at + 3], sx[at + 3]);
       d3[to - (kUnitR - 1) * kBX] = a.d();
       x3[to - (kUnitR - 1) * kBX] = a.x();
     }
@@ -236,12 +243,9 @@ __global__ void __launch_bounds__(kBX *kBY, UNIT ? 4 : 1) calpa_metric(const __g
     for (int y = threadIdx.y; y < kUnitBY; y += kBY) {
       const int at = (y + kUnitR - 1) * kBX + threadIdx.x, up = y * TW + mid, dn = up + 2 * kUnitR * TW;
       DiscSum a(d3[y * kBX + threadIdx.x], x3[y * kBX + threadIdx.x]);
-      a.add(w1, d2[at - kBX], x2[at - kBX]);
-      a.add(w1, d2[at + kBX], x2[at + kBX]);
-      a.add(w4, d2[at - 2 * kBX], x2[at - 2 * kBX]);
-      a.add(w4, d2[at + 2 * kBX], x2[at + 2 * kBX]);
-      a.add(w9, sd[up], sx[up]);
-      a.add(w9, sd[dn], sx[dn]);
+      a.add(w1, d2[at - kBX], x2[at - kBX], d2[at + kBX], x2[at + kBX]);
+      a.add(w4, d2[at - 2 * kBX], x2[at - 2 * kBX], d2[at + 2 * kBX], x2[at + 2 * kBX]);
+      a.add(w9, sd[up], sx[up], sd[dn], sx[dn]);
       if (u < A.W && by0 + y < A.H) store_matrix(A, kUnitR, a, u, by0 + y);
     }
   } else {
