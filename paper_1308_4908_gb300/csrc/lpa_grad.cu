@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_grad(const __grid_constant__ 
     const int row = (tid >> 6) * P + k, v = v0 + row;
     MomentsLean<1> m;
     m.zero();
-    bool ok = true;
+    int moved = 0;
 #pragma unroll 1
     for (int s = 0; s < S; s++) {
       const LpaSensorK &Sk = L.s[s];
@@ -114,8 +114,8 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_grad(const __grid_constant__ 
         const int ox = 1 - sub, oy = sub;
         float Dx0, Dy0;
         const int i0 = first_cell(lx, fx, ox, hx, mx, Dx0), j0 = first_cell(ly, fy, oy, hy, my, Dy0);
-        const int i = min(max(i0, 0), PW - N), j = min(max(j0, 0), PH - N);
-        ok = ok && i == i0 && j == j0;
+        const int i = cell_in(i0, PW - N), j = cell_in(j0, PH - N);
+        moved |= (i ^ i0) | (j ^ j0);
         const float2 *pl = reinterpret_cast<const float2 *>(smem + s * L.mean_plane) + sub * (PW * PH) + j * PW + i;
         const float2 DR0 = make_float2(fmaf(a00, Dx0, a01 * Dy0), fmaf(a10, Dx0, a11 * Dy0));
 #pragma unroll
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 2) lpa_grad(const __grid_constant__ 
             window_cell<1, LPA_GRADIENTS>(m, D, pl[r * PW + c], R2, cexp, L.taper, make_float4(1.f, 0.f, 1.f, 0.f));
         }
       }
-      if (!ok && u < L.out_w && v < L.out_h && abs(lx) < (1 << 20) && abs(ly) < (1 << 20)) atomicOr(L.status, LPA_ERR_BOUNDS);
+      if (moved && u < L.out_w && v < L.out_h && abs(lx) < (1 << 20) && abs(ly) < (1 << 20)) atomicOr(L.status, LPA_ERR_BOUNDS);
     }
     const FitOut f = solve_with_fallback<3, MomentsLean<1>, true, F64>(m, L.min_pivot, L.cond_fallback);
     if (u < L.out_w && v < L.out_h) {

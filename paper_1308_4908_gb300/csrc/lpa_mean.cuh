@@ -289,15 +289,15 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
         const float flx = floorf(px), fly = floorf(py);
         const int lx = an.x + (int)flx, ly = an.y + (int)fly;
         const float fx = px - flx, fy = py - fly;
-        bool ok = true;
+        int moved = 0;
         auto phase = [&](auto N_, Sums<COMP> &a, int ox, int oy, int g) {
           constexpr int N = decltype(N_)::value;
           const float hx = L.trunc_k * sg[g] * Sk.hx_unit + 1e-3f, hy = L.trunc_k * sg[g] * Sk.hy_unit + 1e-3f;
           const float unit = sqrtf(log2e * 0.5f) / sg[g];  // K = 2^-(unit |d|)^2 - taper
           float dx, dy;
-          const int i0 = first_cell(lx, fx, ox, hx, floorf(0.5f * hx), dx), i = min(max(i0, 0), PW - N);
-          const int j0 = first_cell(ly, fy, oy, hy, floorf(0.5f * hy), dy), j = min(max(j0, 0), (Sk.box_h >> 1) - N);
-          ok = ok && i == i0 && j == j0;
+          const int i0 = first_cell(lx, fx, ox, hx, floorf(0.5f * hx), dx), i = cell_in(i0, PW - N);
+          const int j0 = first_cell(ly, fy, oy, hy, floorf(0.5f * hy), dy), j = cell_in(j0, (Sk.box_h >> 1) - N);
+          moved |= (i ^ i0) | (j ^ j0);
           const float2 *pl = planes + (ox + 2 * oy) * PP + j * PW + i;
           if constexpr (FORM == kFactored) {
             const float cx = -unit * unit * fmaf(Sk.A[0], Sk.A[0], Sk.A[2] * Sk.A[2]);
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
         phase(std::integral_constant<int, NG>(), acc[k][1], 1, 0, 1);
         phase(std::integral_constant<int, NG>(), acc[k][1], 0, 1, 1);
         phase(std::integral_constant<int, NR>(), acc[k][2], 1, 1, 0);
-        if (!ok && u < L.out_w && v0 + row < y_end && abs(lx) < (1 << 20) && abs(ly) < (1 << 20))
+        if (moved && u < L.out_w && v0 + row < y_end && abs(lx) < (1 << 20) && abs(ly) < (1 << 20))
           atomicOr(L.status, LPA_ERR_BOUNDS);
       }
     }

@@ -19,6 +19,10 @@ __device__ __forceinline__ int first_cell(int l, float f, int o, float h, float 
   return (e >> 1) - (int)n;
 }
 
+// A first cell as it is where the window's cells lie in the box, else (negative ones included) the last
+// that does: one unsigned minimum; the caller compares to record the move.
+__device__ __forceinline__ int cell_in(int i, int last) { return (int)min((unsigned)i, (unsigned)last); }
+
 // A group of eight columns of one row of a sensor's box: where it lies and its raw samples, zeros off the frame.
 struct Group {
   int s, row, col, X, Y;
