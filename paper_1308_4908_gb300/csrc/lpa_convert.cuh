@@ -15,12 +15,14 @@ namespace lpa {
 __device__ __forceinline__ float2 stage_pair(float f, float iv) { return make_float2(f, iv); }
 __device__ __forceinline__ bool sample_ok(float2 fv) { return fv.y > 0.f; }
 // The staged value of raw sample y at sensor pixel (X, Y), inside the frame: Eq. 18 and the inverse
-// of Eq. 20 (its square root for the printed weight K / s); (0, 0) when saturated. `scalar`: the
-// sensor has no per-pixel calibration frames.
+// of Eq. 20 (its square root for the printed weight K / s). An excluded sample is (0, 0), so that a window value of
+// any size times it adds nothing: a saturated one, and one whose weight is 0 or whose value, weight or
+// product FP32 cannot hold (a sensitivity or read variance decades beyond any sensor's, a bias that is
+// no number). Sensors marked plain (`plain` = LpaSensorK::plain) have no such samples besides the saturated ones.
 template <bool LIT>
-__device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool scalar, int X, int Y, float y) {
+__device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool plain, int X, int Y, float y) {
   float f = 0.f, iv = 0.f;
-  if (scalar) {
+  if (plain) {
     if (y < Sk.sat) {
       const float e0 = y - Sk.black;
       f = e0 * Sk.inv_gtn;
@@ -38,12 +40,13 @@ __device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool scal
       f = div_approx(e0 * Sk.inv_gtn, a);
       iv = div_approx(Sk.gtn2 * a * a, fmaf(Sk.gain, fmaxf(e0, 0.f), rv));
       if (LIT) iv = sqrtf(iv);
+      if (!(iv > 0.f && fabsf(iv * f) <= 3.402823466e38f)) f = iv = 0.f;
     }
   }
   return stage_pair(f, iv);
 }
 
-// convert_sample<false> of two samples of a sensor without calibration frames, in paired arithmetic with
+// convert_sample<false> of two samples of a plain sensor, in paired arithmetic with
 // its roundings: f and 1 / s2, which is 0 (f is not, unlike there) where ok is false or the sample is
 // saturated.
 __device__ __forceinline__ void convert_two(const LpaSensorK &S, float y0, float y1, bool ok0, bool ok1, float2 &f, float2 &iv) {

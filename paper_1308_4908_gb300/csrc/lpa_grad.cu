@@ -35,7 +35,6 @@ __device__ __forceinline__ int class_column(int t, int sx) {
 __device__ __forceinline__ void store_green(const LpaLaunch &L, const Group &r, float2 *planes) {
   const LpaSensorK &S = L.s[r.s];
   const int PW = S.box_w >> 1, PP = PW * (S.box_h >> 1);
-  const bool scalar = !S.bias && !S.rvar && !S.satf && !S.prnu;
   const int n = r.X >= 0 && r.Y >= 0 && r.Y < S.height ? S.width - r.X : 0;  // columns inside the frame
   const int odd = (r.row & 1) ? 0 : 1;  // the green columns of this row
   const uint32_t w[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
@@ -43,7 +42,7 @@ __device__ __forceinline__ void store_green(const LpaLaunch &L, const Group &r, 
   float y[4];
 #pragma unroll
   for (int k = 0; k < 4; k++) y[k] = (float)(odd ? w[k] >> 16 : w[k] & 0xffffu);
-  if (scalar) {
+  if (S.plain) {
 #pragma unroll
     for (int k = 0; k < 4; k += 2) {
       float2 f, iv;
@@ -54,7 +53,7 @@ __device__ __forceinline__ void store_green(const LpaLaunch &L, const Group &r, 
   } else {
 #pragma unroll
     for (int k = 0; k < 4; k++)
-      v[k] = 2 * k + odd < n ? convert_sample<false>(S, scalar, r.X + 2 * k + odd, r.Y, y[k]) : make_float2(0.f, 0.f);
+      v[k] = 2 * k + odd < n ? convert_sample<false>(S, false, r.X + 2 * k + odd, r.Y, y[k]) : make_float2(0.f, 0.f);
   }
   float4 *o = reinterpret_cast<float4 *>(planes + (r.row & 1) * PP + (r.row >> 1) * PW + 4 * r.col);
   o[0] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);

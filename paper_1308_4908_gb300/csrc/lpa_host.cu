@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
+#include <limits>
 #include <algorithm>
 #include <array>
 #include <cstring>
@@ -609,6 +610,16 @@ hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p,
   return HDR_OK;
 }
 
+// Whether every unsaturated sample of a sensor without per-pixel frames has a finite value, weight and product
+// of the two in FP32, with normal divisors (LpaSensorK::plain).
+int plain_sensor(const RigSensor &r, const LpaSensorK &K) {
+  if (r.bias || r.prnu || r.rvar || r.satf) return 0;
+  const double most = std::max(std::fabs((double)K.black), std::fabs(65535.0 - K.black));
+  const double f = most * K.inv_gtn, iv = (double)K.gtn2 / K.read_var;
+  return K.read_var >= std::numeric_limits<float>::min() && K.gain * most + K.read_var < 0x1p126 && f < 0x1p126 &&
+         iv < 0x1p126 && f * iv < 0x1p126;
+}
+
 // Staging box of the general kernels for sensor transform G: the tile's pixel points span |G_lin| *
 // (TILE-1) in sensor space; add the largest window's half extent plus margin on both sides, the floor of
 // the origin and the alignment of the origin (x to 8 elements = 16 bytes, y to 2).
@@ -724,6 +735,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     K.prnu = rig.s[s].prnu;
     K.rvar = rig.s[s].rvar;
     K.satf = rig.s[s].satf;
+    K.plain = plain_sensor(rig.s[s], K);
     K.raw = raw[s];
     K.raw_pitch = d.pitch_elems;
     if (mean.size >= 0) {

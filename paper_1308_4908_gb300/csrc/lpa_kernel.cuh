@@ -1025,13 +1025,13 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
     float2 *planes = reinterpret_cast<float2 *>(smem + Sk.off_planes);
     const int bw = Sk.box_w, n = bw * Sk.box_h, PW = bw >> 1, PP = (bw >> 1) * (Sk.box_h >> 1);
     const int x0 = fp_x0[s], y0 = fp_y0[s];
-    const bool scalar = !Sk.bias && !Sk.rvar && !Sk.satf && !Sk.prnu;
+    const bool plain = Sk.plain;
     const int W = Sk.width, H = Sk.height;
     const int step_y = NT / bw, step_x = NT - step_y * bw;
     int lx = tid % bw, ly = tid / bw;
     for (int e = tid; e < n; e += NT) {
       const int X = x0 + lx, Y = y0 + ly;
-      const float2 v = (X >= 0 && X < W && Y >= 0 && Y < H) ? convert_sample<LIT>(Sk, scalar, X, Y, (float)raw[e])
+      const float2 v = (X >= 0 && X < W && Y >= 0 && Y < H) ? convert_sample<LIT>(Sk, plain, X, Y, (float)raw[e])
                                                           : stage_pair(0.f, 0.f);
       planes[((lx & 1) + 2 * (ly & 1)) * PP + (ly >> 1) * PW + (lx >> 1)] = v;
       lx += step_x;
@@ -1332,7 +1332,7 @@ __global__ void __launch_bounds__(kConvertX *kConvertY) lpa_convert(const __grid
   const int CP = Sk.conv_pitch, W = Sk.width;
   const int c0 = 4 * (int)(blockIdx.x * kConvertX + threadIdx.x), X0 = 2 * c0;  // four phase columns, eight samples
   if (c0 >= CP) return;
-  const bool scalar = !Sk.bias && !Sk.rvar && !Sk.satf && !Sk.prnu;
+  const bool plain = Sk.plain;
   const size_t plane = (size_t)Sk.conv_h * CP;
   const int last = R.r1[s];
   for (int Y = R.r0[s] + (int)(blockIdx.y * kConvertY + threadIdx.y); Y < last; Y += (int)gridDim.y * kConvertY) {
@@ -1341,7 +1341,7 @@ __global__ void __launch_bounds__(kConvertX *kConvertY) lpa_convert(const __grid
     if (n > 0) q = *reinterpret_cast<const uint4 *>(Sk.raw + (size_t)Y * Sk.raw_pitch + X0);
     const uint32_t w4[4] = {q.x, q.y, q.z, q.w};
     float2 e[4], o[4];  // columns c0 .. c0 + 3 of the even-x and the odd-x phase
-    if (!LIT && scalar) {
+    if (!LIT && plain) {
 #pragma unroll
       for (int k = 0; k < 4; k++) {
         float2 f, iv;
@@ -1355,8 +1355,8 @@ __global__ void __launch_bounds__(kConvertX *kConvertY) lpa_convert(const __grid
 #pragma unroll
       for (int k = 0; k < 4; k++) {
         const int X = X0 + 2 * k;
-        e[k] = 2 * k < n ? convert_sample<LIT>(Sk, scalar, X, Y, (float)(w4[k] & 0xffffu)) : stage_pair(0.f, 0.f);
-        o[k] = 2 * k + 1 < n ? convert_sample<LIT>(Sk, scalar, X + 1, Y, (float)(w4[k] >> 16)) : stage_pair(0.f, 0.f);
+        e[k] = 2 * k < n ? convert_sample<LIT>(Sk, plain, X, Y, (float)(w4[k] & 0xffffu)) : stage_pair(0.f, 0.f);
+        o[k] = 2 * k + 1 < n ? convert_sample<LIT>(Sk, plain, X + 1, Y, (float)(w4[k] >> 16)) : stage_pair(0.f, 0.f);
       }
     }
     float2 *de = Sk.conv + (size_t)(2 * (Y & 1)) * plane + (size_t)(Y >> 1) * CP + c0;  // colour phase (0, Y & 1)

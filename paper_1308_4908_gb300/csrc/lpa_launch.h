@@ -30,6 +30,9 @@ struct alignas(64) LpaSensorK {
   float inv_gtn;            // 1 / (g t n)
   float gtn2;               // (g t n)^2
   float gain, read_var, black, sat;
+  // 1: no per-pixel frames, and every unsaturated sample has a finite value and weight (others are
+  // converted with a test for what FP32 cannot hold, convert_sample)
+  int plain;
   int width, height;
   int box_w, box_h;         // staged footprint in elements; box_w % 8 == 0, box_h even
   float ext_x, ext_y;       // half extent of the window box in sensor px incl. margin (max scale)

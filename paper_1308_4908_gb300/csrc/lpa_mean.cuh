@@ -51,13 +51,12 @@ struct Layout {
 __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, float2 *planes) {
   const LpaSensorK &S = L.s[r.s];
   const int PW = S.box_w >> 1, PP = PW * (S.box_h >> 1);
-  const bool scalar = !S.bias && !S.rvar && !S.satf && !S.prnu;
   const int n = r.X >= 0 && r.Y >= 0 && r.Y < S.height ? S.width - r.X : 0;  // columns inside the frame
   const uint32_t w[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
   float4 *even = reinterpret_cast<float4 *>(planes + 2 * (r.row & 1) * PP + (r.row >> 1) * PW + 4 * r.col);
   float4 *odd = even + (PP >> 1);
   float2 v[8];  // (1 / s2, f / s2)
-  if (scalar) {
+  if (S.plain) {
 #pragma unroll
     for (int k = 0; k < 4; k++) {
       float2 f, iv;
@@ -72,7 +71,7 @@ __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, 
       const uint32_t y = (k & 1) ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu;
       v[k] = make_float2(0.f, 0.f);
       if (k < n) {
-        const float2 fv = convert_sample<false>(S, scalar, r.X + k, r.Y, (float)y);  // (f, 1 / s2)
+        const float2 fv = convert_sample<false>(S, false, r.X + k, r.Y, (float)y);  // (f, 1 / s2)
         v[k] = make_float2(fv.y, fv.y * fv.x);
       }
     }
