@@ -30,9 +30,6 @@ struct alignas(64) LpaSensorK {
   float inv_gtn;            // 1 / (g t n)
   float gtn2;               // (g t n)^2
   float gain, read_var, black, sat;
-  // 1: no per-pixel frames, and every unsaturated sample has a finite value and weight (others are
-  // converted with a test for what FP32 cannot hold, convert_sample)
-  int plain;
   int width, height;
   int box_w, box_h;         // staged footprint in elements; box_w % 8 == 0, box_h even
   float ext_x, ext_y;       // half extent of the window box in sensor px incl. margin (max scale)
@@ -40,6 +37,10 @@ struct alignas(64) LpaSensorK {
   uint32_t off_raw2;        // the second staging buffer's raw box (= off_raw with one buffer)
   uint32_t off_planes;      // byte offset of the four colour-phase planes (float2 each)
   int ix_shift, iy_shift;   // tabulated weights: floor of the translation of G (sensor px)
+  // 1: no per-pixel frames, and every unsaturated sample has a finite value and weight (others are
+  // converted with a test for what FP32 cannot hold, convert_sample). Here it fills the padding before
+  // the pointers: four bytes further up every later field moved, and order-0 frames of four scales took 2 % more.
+  int plain;
   const float *bias;        // optional per-pixel frames [height][width] (device)
   const float *prnu;
   const float *rvar;
