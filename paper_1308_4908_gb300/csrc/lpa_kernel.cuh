@@ -576,30 +576,53 @@ struct MultiScale {
   static constexpr int value = lpa_scales_per_walk(ORDER, COMP, MODE);
 };
 
-// Which pixel of its 16 x TH tile each thread takes. Output pixels whose step spans two sensor pixels
-// (one cell of a colour phase) see the samples at the same fractions: every 2nd pixel at 1x, 3rd
+// Which pixel of its 16 x TH tile each thread takes. Output pixels whose step spans a whole number of colour-phase
+// cells (two sensor pixels each) see the samples at the same fractions: every 2nd pixel at 1x, 3rd
 // at 1.5x, 4th at 2x. The threads take the classes of pixels equal modulo (sx, sy) one after the
 // other (each class row by row; classes in serpentine order, so that a warp holding the end of one
 // class and the start of the next mixes neighbours), sx and sy in 1..4. At 1x this is 8 x 4 pixels
 // of one parity class per warp; 1920 x 1080 -> 2880 x 1620 at order 1, four scales, ran with 25.6 of
 // 32 lanes active per instruction and 64 M bank conflicts under that map: 3528 us, 2928 us under
 // its own.
+// Where a class fills a warp in each half of a 16-row tile, the halves come one after the other, so that a
+// frame's last half row of tiles keeps one warp in each of an SM's four schedulers (warp modulo 4)
+// busy; the second half starts from the middle class, so that no scheduler gets one class alone. Classes over the
+// whole tile put such a tile on two schedulers: 640 x 360, order 1, compensated, four scales 635 us,
+// 572 us so.
 template <int TH>
 struct PixelMap {
   uint8_t at[16][LPA_TILE * TH];  // [4 (sy - 1) + sx - 1][thread]: u | v << 4
+  static constexpr int parts(int sx, int sy) { return TH == 16 && sx != 3 && sy != 3 && sx * sy <= 4 ? 2 : 1; }
   constexpr PixelMap() : at{} {
     for (int sy = 1; sy <= 4; sy++)
       for (int sx = 1; sx <= 4; sx++) {
         int n = 0;
-        for (int cy = 0; cy < sy; cy++)
-          for (int k = 0; k < sx; k++) {
+        const int np = parts(sx, sy), rows = TH / np, classes = sx * sy;
+        for (int part = 0; part < np; part++)
+          for (int i = 0; i < classes; i++) {
+            const int c = (i + part * (classes / 2)) % classes, cy = c / sx, k = c % sx;
             const int cx = (cy & 1) ? sx - 1 - k : k;
-            for (int v = cy; v < TH; v += sy)
+            for (int v = part * rows + cy; v < (part + 1) * rows; v += sy)
               for (int u = cx; u < LPA_TILE; u += sx) at[4 * (sy - 1) + sx - 1][n++] = (uint8_t)(u | v << 4);
           }
       }
   }
+  // every pixel once in every map, and in a map of two parts the first half of the threads on the first half
+  // of the rows
+  constexpr bool sound() const {
+    for (int sy = 1; sy <= 4; sy++)
+      for (int sx = 1; sx <= 4; sx++) {
+        bool seen[LPA_TILE * TH] = {};
+        for (int t = 0; t < LPA_TILE * TH; t++) {
+          const int m = at[4 * (sy - 1) + sx - 1][t];
+          if (seen[m] || (parts(sx, sy) == 2 && (t < LPA_TILE * TH / 2) != ((m >> 4) < TH / 2))) return false;
+          seen[m] = true;
+        }
+      }
+    return true;
+  }
 };
+static_assert(PixelMap<8>().sound() && PixelMap<16>().sound(), "a tile's pixels over its threads");
 template <int TH>
 static __device__ const PixelMap<TH> pixel_map = PixelMap<TH>();
 
