@@ -812,9 +812,17 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
       }
     }
   }
-  // the pixel steps that span two sensor px of the first sensor (the others differ by their slight
-  // misalignment); beyond 4 (enlargements over 2.25 times) neighbours differ little: as at 1x
+  // the pixel steps (1 to 4) after which the samples repeat at the first sensor (the others differ by their slight
+  // misalignment): the smallest that spans a whole number of cells of two sensor px, to a sixteenth of a cell, also
+  // on reduced outputs (step 3, every 2nd pixel: three sensors 1200 x 900 -> 400 x 300, four
+  // scales, orders 0 to 2: 163, 187 and 272 us taking each pixel in turn, 140, 153 and 224 us so; step 1.5 at order 1,
+  // every 4th: 370 and 317 us); else about two sensor px; beyond 4 (enlargements over 2.25 times) neighbours differ
+  // little: as at 1x
   auto stride = [](double step) {
+    for (int k = 1; k <= 4; k++) {
+      const double cells = 0.5 * k * step, whole = std::round(cells);
+      if (whole >= 1.0 && std::fabs(cells - whole) <= 1.0 / 16) return k;
+    }
     const double n = std::round(2.0 / step);
     return n >= 1.0 && n <= 4.0 ? (int)n : n < 1.0 ? 1 : 2;
   };

@@ -55,3 +55,22 @@ def test_every_stride(ctx, order, sx, sy):
         ctx.check()
         np.testing.assert_array_equal(o2.cpu().numpy(), g)
         np.testing.assert_array_equal(c2.cpu().numpy(), gc)
+
+
+@pytest.mark.parametrize("order", [0, 2])
+@pytest.mark.parametrize("step", [1.5, 2.5, 3.0, 3.5])
+def test_strides_of_reduced_outputs(ctx, order, step):
+    """Reduced outputs whose 2nd or 4th pixels repeat the samples' fractions, ragged and half tiles."""
+    fr = synth.paper_scale(size=120, seed=1601)
+    w, h = round(120 / step) + 1, round(100 / step) - 3
+    p = dataclasses.replace(fr.params, order=order, sigmas=(0.6, 1.1), out_w=w, out_h=h,
+                            out_affine=np.array([[step, 0.0, 0.3], [0.0, step, 0.6]]))
+    ctx.set_rig(0, fr.sensors)
+    ch = torch.full((3, h, w), 77, dtype=torch.uint8, device="cuda")
+    out = ctx.reconstruct(0, p, [torch.from_numpy(s.raw).cuda() for s in fr.sensors], choice=ch)
+    ctx.check()
+    g, gc = out.cpu().numpy(), ch.cpu().numpy()
+    vv, uu = np.mgrid[0:h, 0:w]
+    pix = np.stack([uu.ravel(), vv.ravel()], axis=1)
+    o = oracle.reconstruct(fr.sensors, p, pix, levels=True, kappa=True)
+    parity.compare(g[:, pix[:, 1], pix[:, 0]], gc[:, pix[:, 1], pix[:, 0]], o, pix, 2, order, p.ici_gamma, p.min_pivot)
