@@ -671,11 +671,11 @@ template <int ORDER, int NSP, int MODE, class MOM>
 __device__ __forceinline__ void window_cell_ms(MOM (&m)[NSP], float2 D, float2 fv, const float (&R2)[NSP],
                                                const float (&cexp)[NSP], float taper, float4 Q) {
   constexpr bool STEER = lpa_mode_steered(MODE);
-  constexpr bool LIT = MODE == LPA_LITERAL;
+  static_assert(MODE != LPA_LITERAL, "the printed weight K / s walks one scale at a time");
   const float2 D2 = __fmul2_rn(D, D);
   const float r2 = STEER ? fmaf(Q.x, D2.x, fmaf(Q.z, D2.y, 2.f * Q.y * (D.x * D.y))) : D2.x + D2.y;
-  // Orders 0 and 1: excluded samples (weight 0: they add exact zeros) are only left out of the count, so that
-  // the branch does not wait for the staged value (1.5x order-1 frame 2839 -> 2800 us; at order 2, whose
+  // Orders 0 and 1: excluded samples ((0, 0): they add exact zeros) are only left out of the count, so that
+  // the branch does not wait for the staged value (1.5x order-1 frame 2839 -> 2792 us; at order 2, whose
   // monomials would be formed for them too, +0.7 %)
   constexpr bool LATE = ORDER <= 1;
   if (!(r2 < R2[NSP - 1] && (LATE || sample_ok(fv)))) return;
@@ -704,8 +704,8 @@ __device__ __forceinline__ void window_cell_ms(MOM (&m)[NSP], float2 D, float2 f
       if (q == 1) two(1);
     const float K = PAIRS ? Kq[q] : ex2_approx(r2 * cexp[q]) - taper;
     const float2 W = weights(K, fv);
-    if constexpr (ORDER == 0) m[q].add0(W.x, W.y, (LIT ? K : W.x) * K, one);
-    else m[q].adds(sm, D, D2, W.x, W.y, (LIT ? K : W.x) * K, one);
+    if constexpr (ORDER == 0) m[q].add0(W.x, W.y, W.x * K, one);
+    else m[q].adds(sm, D, D2, W.x, W.y, W.x * K, one);
   }
 }
 
