@@ -30,13 +30,16 @@ struct Group {
 };
 
 // Box origin of a tile in sensor s: x on a multiple of 8 (16-byte loads), y even. FP32 is enough
-// (the box has a margin of a pixel), and every thread forms the same value.
+// (the box has a margin of a pixel). The fetch and the position tables form it each for themselves and must get the
+// same integers, so every rounding is written out: a sum that the compiler fused in one place and not in
+// another could fall on two sides of an integer.
 __device__ __forceinline__ int2 box_origin(const LpaSensorK &S, int u0, int v0, int bh) {
-  float x = S.Gf[0] * (float)(S.Gf[0] < 0.f ? u0 + kBW - 1 : u0) + S.Gf[1] * (float)(S.Gf[1] < 0.f ? v0 + bh - 1 : v0);
-  float y = S.Gf[2] * (float)(S.Gf[2] < 0.f ? u0 + kBW - 1 : u0) + S.Gf[3] * (float)(S.Gf[3] < 0.f ? v0 + bh - 1 : v0);
-  x = fminf(fmaxf(x + S.Gt[0] - S.ext_x, -LPA_FAR_F), LPA_FAR_F);
-  y = fminf(fmaxf(y + S.Gt[1] - S.ext_y, -LPA_FAR_F), LPA_FAR_F);
-  return make_int2((int)floorf(x) & ~7, (int)floorf(y) & ~1);
+  auto origin = [&](float gu, float gv, float gt, float ext) {
+    const float u = (float)(gu < 0.f ? u0 + kBW - 1 : u0), v = (float)(gv < 0.f ? v0 + bh - 1 : v0);
+    const float q = __fsub_rn(__fadd_rn(__fmaf_rn(gv, v, __fmul_rn(gu, u)), gt), ext);
+    return (int)floorf(fminf(fmaxf(q, -LPA_FAR_F), LPA_FAR_F));
+  };
+  return make_int2(origin(S.Gf[0], S.Gf[1], S.Gt[0], S.ext_x) & ~7, origin(S.Gf[2], S.Gf[3], S.Gt[1], S.ext_y) & ~1);
 }
 
 __device__ __forceinline__ Group load_group(const LpaLaunch &L, int s, int g, int u0, int v0, int bh) {

@@ -216,3 +216,19 @@ def test_refused_as_by_the_general_kernel(ctx, n, reduce, rot):
     assert refused[0] == refused[1] and refused[0] in (0, hdr.HDR_E_UNSUPPORTED)
     if (n, reduce) in ((8, 1.0), (8, 3.2)):
         assert (refused[0] == 0) == (reduce == 1.0)
+
+
+@pytest.mark.parametrize("nudge", [-1e-6, 0.0, 1e-6])
+@pytest.mark.parametrize("scale,rot", [(1.0, 0.0), (1.5, 0.0), (1.0, 0.2), (1.3, 0.0)])
+def test_boxes_on_an_alignment_boundary(ctx, scale, rot, nudge):
+    """Sensors displaced by the reach of the staging box, so that its corner falls on a multiple of 8 px, or a
+    rounding to either side, in every tile of an unrotated frame: the fetched samples and the position tables must
+    agree on it."""
+    w, h = round(131 * scale), round(34 * scale)
+    fr = _frame(131, 34, rot, out_w=w, out_h=h, out_affine=np.array([[1 / scale, 0.0, 0.0], [0.0, 1 / scale, 0.0]]))
+    for k, s in enumerate(fr.sensors):
+        s.affine = np.array(s.affine, dtype=np.float64)
+        s.affine[:, 2] = -(3 * 0.7 + 2e-3 + 1.0 + nudge) + 8.0 * k
+        s.raw = synth.simulate_raw(fr.scene, s, 1500, k)
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
