@@ -426,6 +426,14 @@ bool runs_mean(const Rig &rig, const hdr_params *p) {
   return m.size >= 0 && mean_smem(rig, p, m, &bufs, &plane, &tab) > 0;
 }
 
+// Whether the gradient pass of these parameters is planned for lpa_grad, which stages every sensor at once.
+bool runs_grad(const Rig &rig, const hdr_params *p) {
+  const MeanPlan m = grad_plan(rig, p);
+  int bufs = 0;
+  uint32_t plane, tab;
+  return m.size >= 0 && mean_smem(rig, p, m, &bufs, &plane, &tab) > 0 && bufs == rig.n;
+}
+
 bool conv_eligible(const Rig &rig, const hdr_params *p, bool adaptive, bool mean = true) {
   return LPA_FRAME_CONV && !adaptive && (long long)p->out_w * p->out_h >= 152LL * 256 && !(mean && runs_mean(rig, p));
 }
@@ -1895,29 +1903,23 @@ hdr_status lpa_launch_mode(hdr_ctx *ctx, int32_t rig_id, const hdr_params *param
   p.tab_weights = 0;  // the window is searched: offsets or weights differ per pixel
   LpaLaunch L;
   const Rig &rig = ctx->rigs[rig_id];
-  if (mode == LPA_GRADIENTS) {
-    uint32_t plane, tab;
-    int bufs = 0;
-    const MeanPlan m = grad_plan(rig, &p);
-    if (m.size >= 0 && mean_smem(rig, &p, m, &bufs, &plane, &tab) > 0 && bufs == rig.n) {
-      s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, nullptr, true, ahead);
-      if (s) return s;  // (refused where the general kernel refuses)
-      if (L.out_w == 0 || L.out_h == 0) return HDR_OK;
-      L.aux = aux;
-      const bool f64 = p.cond_fallback > 0.0 && (p.min_pivot - 1e-4) * p.cond_fallback < 2.0;
-      cudaError_t e = lpa_launch_grad(L, f64, st);
-      if (e != cudaSuccess) return fail(HDR_E_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
-      return HDR_OK;
-    }
-  }
+  const bool small = mode == LPA_GRADIENTS && runs_grad(rig, &p);  // lpa_grad, which reads the raw frames
   float2 *conv = nullptr;
-  if (ahead) {
+  if (ahead && !small) {
     s = conv_buffer(ctx, rig, &p, true, &conv);
     if (s) return s;
   }
   // (planned as for the level maps: the kernel of `mode` is the general one, with its variance sums)
-  s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, conv);
+  s = plan(ctx, rig, &p, raw_dev, L, reach, true, 1, conv, small, ahead);
   if (s) return s;
+  if (small && L.mode == LPA_GRADIENTS) {  // (a general plan otherwise: refused above, or launched below)
+    if (L.out_w == 0 || L.out_h == 0) return HDR_OK;
+    L.aux = aux;
+    const bool f64 = p.cond_fallback > 0.0 && (p.min_pivot - 1e-4) * p.cond_fallback < 2.0;
+    cudaError_t e = lpa_launch_grad(L, f64, st);
+    if (e != cudaSuccess) return fail(HDR_E_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+    return HDR_OK;
+  }
   if (L.conv) {  // the frame converted once, then the pass
     s = convert_rows(ctx, L, all_rows(L), true, st);
     if (s) return s;
