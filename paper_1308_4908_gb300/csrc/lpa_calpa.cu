@@ -147,7 +147,7 @@ __device__ __forceinline__ void store_matrix(const MetricArgs &A, int r, const D
   float L1 = l1.x * up, L2 = fmaxf(l2.x, 0.f) * up;
   // Nearly rank one: the pairs hold l2 to about 2^-45 l1, less than an FP32 value needs below this
   // ratio (noise keeps it above in camera frames; a lone gradient or a clean ramp is below), so T and
-  // its eigenvalues are formed again in FP64, from the gradients: sums that left FP32's range (not a
+  // its eigenvalues are formed again in FP64, from the gradients: sums and products with the scale that left FP32's range (not a
   // number here) come this way too.
   if (!(l2.x >= 0x1p-18f * l1.x)) {
     double da = 0.0, db = 0.0, dc = 0.0;
@@ -156,21 +156,25 @@ __device__ __forceinline__ void store_matrix(const MetricArgs &A, int r, const D
       const float2 *row = A.grad + (size_t)(v + dj) * A.W + u;
       for (int di = max(-rw, -u); di <= min(rw, A.W - 1 - u); di++) {
         const float2 wp = A.w[di * di + dj * dj], g = row[di];
-        const double w = (double)wp.x + (double)wp.y, gx = (double)(g.x * A.unit), gy = (double)(g.y * A.unit);
+        const double w = (double)wp.x + (double)wp.y, gx = (double)g.x * (double)A.unit, gy = (double)g.y * (double)A.unit;
         da = fma(w, gx * gx, da);
         db = fma(w, gx * gy, db);
         dc = fma(w, gy * gy, dc);
       }
     }
-    const double m2 = ((double)A.m2.x + (double)A.m2.y) * (double)down;
+    const double m2 = (double)A.m2.x + (double)A.m2.y;
     da *= m2;
     db *= m2;
     dc *= m2;
     const double dh = 0.5 * (da + dc), dd = sqrt(0.25 * (da - dc) * (da - dc) + db * db);
-    L1 = (float)(dh + dd) * up;
-    L2 = (float)fmax(dh - dd, 0.0) * up;
-    ux = da > dc ? (float)(dh + dd - dc) : (float)db;
-    uy = da > dc ? (float)db : (float)(dh + dd - da);
+    L1 = (float)(dh + dd);
+    L2 = (float)fmax(dh - dd, 0.0);
+    const double vx = da > dc ? dh + dd - dc : db, vy = da > dc ? db : dh + dd - da;
+    // into FP32's range before the conversion, by a power of two
+    const int vexp = (__double2hiint(fmax(fabs(vx), fabs(vy))) >> 20) & 2047;
+    const double vunit = __hiloint2double(min(max(2046 - vexp, 1), 2046) << 20, 0);
+    ux = (float)(vx * vunit);
+    uy = (float)(vy * vunit);
   }
   const int ex = (__float_as_int(fmaxf(fabsf(ux), fabsf(uy))) >> 23) & 255;  // its exponent removed, exactly
   const float unit = __int_as_float(min(max(253 - ex, 1), 254) << 23);

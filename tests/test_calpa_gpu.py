@@ -341,6 +341,18 @@ def test_metric_of_huge_gradients(ctx, window_sigma, size):
     assert eig.min() >= c.min_eig * (1 - 1e-5) and eig.max() <= c.max_eig * (1 + 1e-5)
 
 
+@pytest.mark.parametrize("window_sigma,size,grad_scale", [(1.0, 1e34, 1e6), (1.06, 1e38, 1e6), (1.0, 1e38, 1.0), (1.0, 1e34, 3e5)])
+def test_metric_of_gradients_scaled_beyond_fp32(ctx, window_sigma, size, grad_scale):
+    """Gradients times grad_scale, or the sums' larger terms, beyond FP32's range: inside the clamp, no NaN."""
+    r = np.random.default_rng(12)
+    g = (size * r.uniform(-1.0, 1.0, (37, 45, 2))).astype(np.float32)
+    g[20:, 20:] = 0.0
+    c = _calpa(window_sigma=window_sigma, grad_scale=grad_scale)
+    q = ctx.calpa_metric(c, torch.from_numpy(g).cuda()).cpu().numpy().astype(np.float64)
+    eig = np.linalg.eigvalsh(np.stack([q[..., [0, 1]], q[..., [1, 2]]], axis=-2))
+    assert eig.min() >= c.min_eig * (1 - 1e-5) and eig.max() <= c.max_eig * (1 + 1e-5)
+
+
 @pytest.mark.parametrize("w,h,scale,grad_sigma", [(1, 1, 1.0, 1.2), (63, 15, 1.0, 0.6), (65, 17, 1.0, 1.2),
                                                    (130, 33, 1.5, 1.8), (96, 48, 2.0, 1.2), (40, 30, 0.6, 1.0),
                                                    (65, 17, 1.0, 2.0)])
