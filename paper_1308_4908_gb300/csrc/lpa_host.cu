@@ -320,7 +320,9 @@ struct MeanPlan {
   double rb = 0, g = 0;  // window radius of R and B, and of G (reference px)
 };
 // Whether a frame runs lpa_mean: order 0, one scale, the inverse-variance weight, and
-// windows of at most 4 x 4 (R, B) and 3 x 3 (G) cells of a colour phase. A fit of one unknown has the
+// windows of at most 4 x 4 (R, B) and 3 x 3 (G) cells of a colour phase, cut at one sigma or further out (the window
+// value is a difference of FP32 exponentials; cut closer in, what it loses shows: at 0.05 sigma 2.3 times the general
+// kernels' error, at 0.3 sigma 1.85 times, from one sigma on the same). A fit of one unknown has the
 // equilibrated pivot 1, so it is usable with any sample (min_pivot below 1) and never solved again
 // in FP64 (cond_fallback at least 1, or none); other parameters keep the general kernel.
 // Rows per thread: four, or eight of half as many threads in the periodic form, once 64 x 32 tiles fill
@@ -329,7 +331,7 @@ struct MeanPlan {
 MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   MeanPlan m;
   // (its grid has a row of tiles per y index: at most 65535 of 8 rows)
-  if (p->out_h > 65535 * 8 || p->order != 0 || p->n_scales != 1 || p->weight_mode != 0 || !(p->min_pivot < 0.99) ||
+  if (p->out_h > 65535 * 8 || p->order != 0 || p->n_scales != 1 || p->weight_mode != 0 || !(p->trunc_k >= 1.0) || !(p->min_pivot < 0.99) ||
       !(p->cond_fallback <= 0.0 || p->cond_fallback >= 1.0))
     return m;
   m.rb = p->trunc_k * p->sigma[0];

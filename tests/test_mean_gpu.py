@@ -232,3 +232,24 @@ def test_boxes_on_an_alignment_boundary(ctx, scale, rot, nudge):
         s.raw = synth.simulate_raw(fr.scene, s, 1500, k)
     out, ch, _ = _run(ctx, fr)
     _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
+def _without_window_rounding(fr, out):
+    """Every pixel within the parity rule's terms for conversion and FP32 sums alone: window values that are exact
+    to one rounding need nothing of the term for their evaluation (ew)."""
+    p = fr.params
+    pix = _every_pixel(p)
+    o = oracle.reconstruct(fr.sensors, p, pix, levels=True)
+    g = out[:, pix[:, 1], pix[:, 0]].T
+    tol = parity.level_tol(o["out"], o["efit"][:, :, 0], 0.0)
+    assert np.array_equal(np.isnan(g), np.isnan(o["out"]))
+    m = ~np.isnan(g)
+    assert (np.abs(g - o["out"])[m] <= tol[m]).all(), float((np.abs(g - o["out"])[m] / tol[m]).max())
+
+
+@pytest.mark.parametrize("trunc_k", [0.05, 0.3, 0.99])
+def test_windows_cut_close_in(ctx, trunc_k):
+    """Windows cut below one sigma, where the window value is the difference of nearly equal exponentials: left to
+    the tabulated windows' general kernel."""
+    fr = _frame(71, 45, 0.0, n=3, sigma=2.0 / trunc_k, trunc_k=trunc_k)
+    _without_window_rounding(fr, _run(ctx, fr)[0])
