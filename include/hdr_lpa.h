@@ -139,7 +139,7 @@ hdr_status hdr_set_rig(hdr_ctx *ctx, int32_t rig_id, int32_t n_sensors, const hd
  * through it by an event), then the reconstruction copies converted footprints; smaller outputs
  * convert each footprint inside one launch. The results are the same either way. Order 0 with one
  * scale whose windows reach less than 4 sensor px (3 for G) runs in one launch of a kernel of its own,
- * which reads the raw frames (weight_mode 0, trunc_k at least 1; tab_weights makes no difference to it).
+ * which reads the raw frames (weight_mode 0, trunc_k at least 1).
  * Asynchronous: returns after queueing the launches. */
 hdr_status hdr_reconstruct(hdr_ctx *ctx, int32_t rig_id, const hdr_params *params,
                            const uint16_t *const *raw_dev, void *out_dev, uint8_t *choice_dev,

@@ -65,11 +65,15 @@ inline const void *lpa_kernel(int order, bool comp, bool diag, int mode, int til
 
 // Order 0 with one window scale (LPA_MEAN). The kernel template for windows that reach reach_rb (R, B) and
 // reach_g (G) sensor px, -1 if they hold more cells than any is built for; its candidate cells per
-// axis; bytes of its position tables for p rows per thread (classes: periodic positions, both axes' classes).
+// axis; bytes of its position tables for p rows per thread (classes: periodic positions, both axes' classes; tab: or
+// of tabulated window weights, whichever the plan takes); the words of the tabulated weights of one sensor, and the place of
+// the first weight of class cls (2 pv + pu) and colour phase ph in them.
 // (sizes 2 and 3 are lpa_grad's: 3 and 4 cells)
 int lpa_mean_size(double reach_rb, double reach_g);
 int lpa_mean_cells(int size, bool green);
-uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors);
+uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, bool tab, int p, int n_sensors);
+int lpa_mean_k_words(int size);
+int lpa_mean_k_word(int size, int cls, int ph);
 // The output rows of `count` unit tiles from tile0 on (whole tile rows) into L.
 void lpa_mean_rows(LpaLaunch &L, int tile0, int count);
 // Its kernel (lpa_mean_threads(L.mean_p) threads), grid and launch over those rows.

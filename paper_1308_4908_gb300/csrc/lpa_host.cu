@@ -116,6 +116,7 @@ struct PlanCache {
   // the inputs a table is built from (sensor count, scales, window constants, scales per pass, each sensor's
   // translation) -> the device table, so that a repeated configuration skips the host build
   std::map<std::vector<double>, void *> by_inputs;
+  cudaStream_t copies = nullptr;  // what tables are uploaded on (upload)
   uint64_t epoch = 0;  // bumped at each eviction (plans holding evicted tables are stale)
   size_t max_tables = 4096;
   // Plans made but not yet launched (a batch plans every frame before its one launch) may hold
@@ -317,6 +318,7 @@ struct MeanPlan {
   bool even = true;   // every sensor's map is a rotation (or reflection) and an even scale
   int tx = 0, ty = 0; // output pixels to a cell of a colour phase where that is exact (2 or 4), else 0
   int p = 1;          // output rows per thread
+  bool tab = false;   // tabulated window weights: an unresampled output of exactly translated sensors
   double rb = 0, g = 0;  // window radius of R and B, and of G (reference px)
 };
 // Whether a frame runs lpa_mean: order 0, one scale, the inverse-variance weight, and
@@ -337,6 +339,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   m.rb = p->trunc_k * p->sigma[0];
   m.g = m.rb * p->green_ratio;
   m.axis = p->out_affine[1] == 0.0 && p->out_affine[3] == 0.0;
+  m.tab = p->tab_weights == 1 && is_identity_linear(p->out_affine);
   double most = 0.0;
   auto period = [](double step) {  // of positions modulo 2 px, to the tolerance of the tabulated weights
     return std::fabs(step - 1.0) <= 1e-12 ? 2 : std::fabs(step - 0.5) <= 1e-12 ? 4 : 0;
@@ -351,6 +354,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
     most = std::max(most, std::max(std::hypot(t[0], t[1]), std::hypot(t[3], t[4])));
     m.axis = m.axis && t[1] == 0.0 && t[3] == 0.0;
     const double *a = rig.s[s].d.affine;
+    m.tab = m.tab && is_identity_linear(a);
     m.even = m.even && std::fabs(a[0] * a[1] + a[3] * a[4]) <= 1e-9 * std::min(a[0] * a[0] + a[3] * a[3], a[1] * a[1] + a[4] * a[4]);
   }
   if (!m.axis || !m.tx || !m.ty) m.tx = m.ty = 0;
@@ -413,7 +417,7 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *
     mean_box(m, G, std::hypot(t[0], t[1]), std::hypot(t[3], t[4]), &bw, &bh, &ex, &ey);
     need = std::max(need, (m.size >= 2 ? 4.0 : 8.0) * bw * bh);  // lpa_grad keeps the green half
   }
-  const double tables = lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.p, rig.n), room = (m.p == 8 ? 73.0 : 110.0) * 1024 - tables;
+  const double tables = lpa_mean_tab_bytes(m.size, m.axis, m.tx + m.ty, m.tab, m.p, rig.n), room = (m.p == 8 ? 73.0 : 110.0) * 1024 - tables;
   if (need > room) return 0;
   *bufs = std::min(rig.n, (int)(room / need));
   *plane = (uint32_t)need;
@@ -456,6 +460,63 @@ size_t conv_elems(const Rig &rig) {
   size_t n = 0;
   for (int s = 0; s < rig.n; s++) n += conv_elems_of(rig.s[s].d.width, rig.s[s].d.height);
   return n;
+}
+
+// Host memory into a new device allocation, also while this thread captures a stream: in relaxed capture mode,
+// by a stream kept for it.
+cudaError_t upload(const void *src, size_t bytes, cudaStream_t st, void **dst) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  void *d = nullptr;
+  e = cudaMalloc(&d, std::max<size_t>(bytes, 16));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) cudaFree(d), d = nullptr;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  *dst = d;
+  return e;
+}
+
+// The device copy of a table built from `inputs`, by its contents (FNV-1a, `tag` apart): the one the
+// context has, or a new one.
+hdr_status device_table(const PlanEnv &env, std::vector<double> inputs, const std::vector<uint8_t> &table, uint64_t tag,
+                        const void **dev) {
+  uint64_t hsh = 1469598103934665603ull;
+  for (uint8_t b : table) hsh = (hsh ^ b) * 1099511628211ull;
+  hsh ^= tag;
+  auto it = env.tabs->dev.find(hsh);
+  if (it == env.tabs->dev.end()) {
+    if (env.tabs->dev.size() >= env.tabs->max_tables) {
+      // every launch made so far may use the tables: wait for the device, then free them, unless
+      // plans that are not launched yet may hold them (then they wait in `retired`)
+      CUDA_TRY(cudaDeviceSynchronize());
+      PlanCache &tc = *env.tabs;
+      size_t keep = 0;
+      for (auto &t : tc.retired) {
+        if (tc.hold > 0 && t.second == tc.scope) tc.retired[keep++] = t;
+        else cudaFree(t.first);
+      }
+      tc.retired.resize(keep);
+      for (auto &t : tc.dev) {
+        if (tc.hold == 0) cudaFree(t.second);
+        else tc.retired.push_back({t.second, tc.scope});
+      }
+      env.tabs->dev.clear();
+      env.tabs->by_inputs.clear();
+      env.tabs->epoch++;
+    }
+    void *d = nullptr;
+    cudaError_t e = upload(table.data(), table.size(), env.tabs->copies, &d);
+    if (e != cudaSuccess)
+      return fail(e == cudaErrorMemoryAllocation ? HDR_E_NOMEM : HDR_E_CUDA, "uploading the weight table failed: %s",
+                  cudaGetErrorString(e));
+    it = env.tabs->dev.emplace(hsh, d).first;
+  }
+  if (env.tabs->by_inputs.size() >= 4 * env.tabs->max_tables) env.tabs->by_inputs.clear();
+  env.tabs->by_inputs.emplace(std::move(inputs), it->second);
+  *dev = it->second;
+  return HDR_OK;
 }
 
 hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p, bool f64_possible, bool one,
@@ -568,55 +629,71 @@ hdr_status build_tables(const PlanEnv &env, const Rig &rig, const hdr_params *p,
   // one padding cell: the kernel loads the cell after each one it reads
   cells.push_back(make_float4(0.f, 0.f, 0.f, 0.f));
   cells.push_back(make_float4(0.f, 0.f, 0.f, 0.f));
-  // content hash (FNV-1a) -> device copy
-  const size_t nb = hdr.size() * sizeof(int4) + cells.size() * sizeof(float4);
-  uint64_t hsh = 1469598103934665603ull;
-  auto mix = [&](const void *ptr, size_t n) {
-    const unsigned char *b = static_cast<const unsigned char *>(ptr);
-    for (size_t i = 0; i < n; i++) hsh = (hsh ^ b[i]) * 1099511628211ull;
-  };
-  mix(hdr.data(), hdr.size() * sizeof(int4));
-  mix(cells.data(), cells.size() * sizeof(float4));
-  hsh ^= (uint64_t)hdr.size() << 40;
-  auto it = env.tabs->dev.find(hsh);
-  if (it == env.tabs->dev.end()) {
-    if (env.tabs->dev.size() >= env.tabs->max_tables) {
-      // every launch made so far may use the tables: wait for the device, then free them, unless
-      // plans that are not launched yet may hold them (then they wait in `retired`)
-      CUDA_TRY(cudaDeviceSynchronize());
-      PlanCache &tc = *env.tabs;
-      size_t keep = 0;
-      for (auto &t : tc.retired) {
-        if (tc.hold > 0 && t.second == tc.scope) tc.retired[keep++] = t;
-        else cudaFree(t.first);
-      }
-      tc.retired.resize(keep);
-      for (auto &t : tc.dev) {
-        if (tc.hold == 0) cudaFree(t.second);
-        else tc.retired.push_back({t.second, tc.scope});
-      }
-      env.tabs->dev.clear();
-      env.tabs->by_inputs.clear();
-      env.tabs->epoch++;
-    }
-    void *d = nullptr;
-    CUDA_TRY(cudaMalloc(&d, std::max<size_t>(nb, 16)));
-    cudaError_t e = cudaMemcpy(d, hdr.data(), hdr.size() * sizeof(int4), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !cells.empty())
-      e = cudaMemcpy(static_cast<int4 *>(d) + hdr.size(), cells.data(), cells.size() * sizeof(float4),
-                     cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      cudaFree(d);
-      return fail(HDR_E_CUDA, "uploading the weight table failed: %s", cudaGetErrorString(e));
-    }
-    it = env.tabs->dev.emplace(hsh, d).first;
-  }
-  if (env.tabs->by_inputs.size() >= 4 * env.tabs->max_tables) env.tabs->by_inputs.clear();
-  env.tabs->by_inputs.emplace(std::move(inputs), it->second);
-  L.tab_hdr = static_cast<const int4 *>(it->second);
-  L.tab_cells = reinterpret_cast<const float4 *>(static_cast<const int4 *>(it->second) + hdr.size());
+  // the header and the cells in one device table
+  std::vector<uint8_t> table(hdr.size() * sizeof(int4) + cells.size() * sizeof(float4));
+  memcpy(table.data(), hdr.data(), hdr.size() * sizeof(int4));
+  memcpy(table.data() + hdr.size() * sizeof(int4), cells.data(), cells.size() * sizeof(float4));
+  const void *dev;
+  hdr_status st = device_table(env, std::move(inputs), table, (uint64_t)hdr.size() << 40, &dev);
+  if (st) return st;
+  L.tab_hdr = static_cast<const int4 *>(dev);
+  L.tab_cells = reinterpret_cast<const float4 *>(static_cast<const int4 *>(dev) + hdr.size());
   L.tab_nsp = nsp;
   L.mode = tab_mode;
+  return HDR_OK;
+}
+
+// Tabulated window weights of lpa_mean (LpaLaunch::mean_k) for a frame whose plan has tab set: per sensor, output
+// parity and colour phase, the window values (Eq. 8, truncated and tapered) of the candidate cells in FP64, rounded
+// once.
+hdr_status mean_weights(const PlanEnv &env, const Rig &rig, const hdr_params *p, const MeanPlan &m, LpaLaunch &L) {
+  std::vector<double> inputs = {-1.0, (double)rig.n, (double)m.size, p->trunc_k, p->green_ratio, p->sigma[0]};
+  for (int s = 0; s < rig.n; s++) {
+    inputs.push_back(L.s[s].G[2]);
+    inputs.push_back(L.s[s].G[5]);
+    L.s[s].ix_shift = (int)std::floor(L.s[s].G[2]);
+    L.s[s].iy_shift = (int)std::floor(L.s[s].G[5]);
+  }
+  auto known = env.tabs->by_inputs.find(inputs);
+  if (known != env.tabs->by_inputs.end()) {
+    L.mean_k = static_cast<const float *>(known->second);
+    return HDR_OK;
+  }
+  const double taper = std::exp(-0.5 * p->trunc_k * p->trunc_k);
+  const size_t words = lpa_mean_k_words(m.size);
+  std::vector<uint8_t> table(rig.n * words * 4, 0);
+  for (int s = 0; s < rig.n; s++) {
+    // by axis, colour phase and output parity: the pixel's distance from the even lattice cell at or below it, in [0, 2),
+    // and the first candidate cell, counted from that one
+    double r[2][4][2];
+    int first[2][4][2];
+    for (int axis = 0; axis < 2; axis++)
+      for (int ph = 0; ph < 4; ph++)
+        for (int par = 0; par < 2; par++) {
+          const double t = L.s[s].G[axis ? 5 : 2], fl = std::floor(t);
+          r[axis][ph][par] = floor_div2_parity((long long)par + (long long)fl - (axis ? ph >> 1 : ph & 1)) + (t - fl);
+          const double R = p->trunc_k * p->sigma[0] * (ph == 1 || ph == 2 ? p->green_ratio : 1.0);
+          first[axis][ph][par] = (int)std::floor((r[axis][ph][par] - R) / 2) + 1;
+          memcpy(&table[(s * words + 8 * axis + 2 * ph + par) * 4], &first[axis][ph][par], 4);
+        }
+    for (int cls = 0; cls < 4; cls++)
+      for (int ph = 0; ph < 4; ph++) {
+        const bool green = ph == 1 || ph == 2;
+        const int pu = cls & 1, pv = cls >> 1, n = lpa_mean_cells(m.size, green);
+        const double sg = p->sigma[0] * (green ? p->green_ratio : 1.0), R = p->trunc_k * sg;
+        for (int j = 0; j < n; j++)
+          for (int i = 0; i < n; i++) {
+            const double dx = 2.0 * (first[0][ph][pu] + i) - r[0][ph][pu], dy = 2.0 * (first[1][ph][pv] + j) - r[1][ph][pv];
+            const double r2 = dx * dx + dy * dy;
+            const float k = r2 < R * R ? (float)(std::exp(-r2 / (2.0 * sg * sg)) - taper) : 0.f;
+            memcpy(&table[(s * words + lpa_mean_k_word(m.size, cls, ph) + j * n + i) * 4], &k, 4);
+          }
+      }
+  }
+  const void *dev;
+  hdr_status st = device_table(env, std::move(inputs), table, 1ull << 63, &dev);
+  if (st) return st;
+  L.mean_k = static_cast<const float *>(dev);
   return HDR_OK;
 }
 
@@ -848,7 +925,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     L.mean_ly = mean.ty / 2;
     if (L.tiles_x > 0 && L.tiles_y > 0) lpa_mean_rows(L, 0, L.tiles_x * L.tiles_y);
     L.stages = 1;
-    return HDR_OK;
+    return mean.tab && env.tabs && env.tabulate ? mean_weights(env, rig, p, mean, L) : HDR_OK;
   }
   L.tx_bytes = tx;
   // a usable fit's equilibrated pivots lie in (min_pivot, 1]: when min_pivot * cond_fallback >= 2
@@ -1082,10 +1159,11 @@ hdr_status hdr_create(int device, hdr_ctx **out) {
   }
   e = cudaMalloc(&c->status, sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->tabs.copies, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     cudaFree(c->status);
     delete c;
-    return fail(HDR_E_NOMEM, "status word allocation failed: %s", cudaGetErrorString(e));
+    return fail(HDR_E_NOMEM, "status word or copy stream allocation failed: %s", cudaGetErrorString(e));
   }
   *out = c;
   return HDR_OK;
@@ -1102,6 +1180,7 @@ void hdr_destroy(hdr_ctx *ctx) {
   cudaFree(ctx->calpa);
   for (auto &t : ctx->tabs.dev) cudaFree(t.second);
   for (auto &t : ctx->tabs.retired) cudaFree(t.first);
+  if (ctx->tabs.copies) cudaStreamDestroy(ctx->tabs.copies);
   if (ctx->h2d) cudaStreamDestroy(ctx->h2d);
   if (ctx->d2h) cudaStreamDestroy(ctx->d2h);
   if (ctx->band2) cudaStreamDestroy(ctx->band2);
@@ -1688,7 +1767,7 @@ hdr_status batch_run_frames(hdr_ctx *ctx, int n, const hdr_frame *frames, const 
                   L.order, L.mode, L.tile_h, L.px, L.stages);
     CUDA_TRY(lpa_opt_in(fn));
     // grid size and shared memory are set on each replay: graphs are kept per sequence of kernels
-    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 8 * L.mean_size + 64 * L.mean_axis + 256 * (L.mean_lx != 0) + 512 * L.mean_comp : L.px,
+    key.push_back({L.order * 64 + L.mode, comp ? 1 : 0, L.tile_h, mean ? L.mean_p + 16 * L.mean_size + 64 * L.mean_axis + 256 * (L.mean_lx != 0) + 512 * L.mean_comp + 1024 * (L.mean_k != nullptr) : L.px,
                    L.stages + 4 * (d >= 0 ? 1 : 0)});
     args.push_back({&plans[f], nullptr});
     cudaKernelNodeParams r{};

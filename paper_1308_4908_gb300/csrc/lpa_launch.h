@@ -116,6 +116,11 @@ struct LpaLaunch {
   int mean_comp;                 // compensated sums
   int mean_y0, mean_y1;          // output rows of the launch (lpa_mean_rows)
   uint32_t mean_plane, mean_tab;
+  // Tabulated window weights of LPA_MEAN (NULL: formed in the kernel), per sensor 16 words and 4 classes of
+  // output parity (2 pv + pu): words 2 ph + pu and 8 + 2 ph + pv are the first candidate column and row of
+  // colour phase ph = ox + 2 oy, in cells from the pixel's even lattice cell; a class holds the weights
+  // of its four phases' candidate cells, row by row, where lpa_mean_k_word puts them.
+  const float *mean_k;
 };
 
 // LPA_SEARCHED_F32, LPA_STEERED_F32, LPA_TABULATED_F32: the searched, steered or tabulated window

@@ -16,10 +16,17 @@ int lpa_mean_size(double reach_rb, double reach_g) {
 int lpa_mean_cells(int size, bool green) {
   return size >= 2 ? size + 1 : size == 0 ? (green ? 2 : 3) : (green ? 3 : 4);
 }
-uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, int p, int n_sensors) {
+int lpa_mean_k_words(int size) { return size == 0 ? lpa::Layout<3, 2>::kTab : lpa::Layout<4, 3>::kTab; }
+int lpa_mean_k_word(int size, int cls, int ph) {
+  using A = lpa::Layout<3, 2>;
+  using B = lpa::Layout<4, 3>;
+  return 16 + (size == 0 ? cls * A::kClass + A::phase_words(ph) : cls * B::kClass + B::phase_words(ph));
+}
+uint32_t lpa_mean_tab_bytes(int size, bool axis, int classes, bool tab, int p, int n_sensors) {
   if (!axis) return (uint32_t)(n_sensors * lpa_mean_tile_h(p) * 16);
   const int words = size == 0 ? lpa::Layout<3, 2>::kWords : lpa::Layout<4, 3>::kWords;
   const int row = size == 0 ? lpa::Layout<3, 2>::kRow : lpa::Layout<4, 3>::kRow;
+  if (tab) return (uint32_t)(n_sensors * 4 * lpa_mean_k_words(size));  // (more than the classes' tables)
   if (classes) return (uint32_t)(n_sensors * 4 * row * classes);
   return (uint32_t)(n_sensors * 4 * (words * lpa::kBW + row * lpa_mean_tile_h(p)));
 }

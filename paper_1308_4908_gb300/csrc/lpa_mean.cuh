@@ -27,7 +27,9 @@
 // class, forms the K of its cells once per sensor and slides the window down one cell a row, each
 // loaded cell serving up to N rows. kFactored: the output is rotated against a sensor whose map is a
 // rotation and an even scale, so |d|^2 still separates in the sensor's axes; the 2 N factors of a window are
-// formed per pixel. kGeneral: each cell forms its offset and one exponential.
+// formed per pixel. kGeneral: each cell forms its offset and one exponential. kTabulated: kPeriodic at 1x on
+// exactly translated sensors, whose window weights the caller may have tabulated (tab_weights): formed by the
+// host in FP64 and rounded once, they are copied into shared memory instead of the factors.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -46,6 +48,13 @@ struct Layout {
   static constexpr int kE = 2 * (NR + NG);       // factors: RB phase 0, RB phase 1, G phase 0, G phase 1
   static constexpr int kWords = 4 + kE;          // four first cells, then the factors
   static constexpr int kRow = (kWords + 3) / 4 * 4;
+  // tabulated positions: words of a phase's weights (16-byte loads), the first of phase ph = ox + 2 oy in
+  // a class, of a class (columns of unequal parity read different banks) and of a sensor (LpaLaunch::mean_k)
+  static constexpr int kR = (NR * NR + 3) / 4 * 4, kG = (NG * NG + 3) / 4 * 4;
+  __host__ __device__ static constexpr int phase_words(int ph) { return ph == 0 ? 0 : kR + (ph - 1) * kG; }
+  static constexpr int kClass = (2 * (kR + kG) + 31) / 32 * 32 == 2 * (kR + kG) ? 2 * (kR + kG) + 4 : 2 * (kR + kG);
+  static constexpr int kTab = 16 + 4 * kClass;
+  static_assert(kTab >= 4 * kRow, "the tables of two classes per axis fit in the same place");
 };
 
 __device__ __forceinline__ void store_group(const LpaLaunch &L, const Group &r, float2 *planes) {
@@ -97,7 +106,7 @@ struct Sums<true> {
   __device__ __forceinline__ float2 value() const { return __fadd2_rn(h, l); }
 };
 
-enum { kGeneral = 0, kAxis = 1, kFactored = 2, kPeriodic = 3 };
+enum { kGeneral = 0, kAxis = 1, kFactored = 2, kPeriodic = 3, kTabulated = 4 };
 
 // The cells and factors of one position along one axis for every (window, phase): words of Layout at
 // t[0], t[stride], ... `last`: how many cells further the last position served by the entry lies. Returns
@@ -150,7 +159,24 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
   float *yt = xt + S * T::kWords * kBW;
   int4 *anchor = reinterpret_cast<int4 *>(smem + L.mean_tab);
   const int lx = L.mean_lx, ly = L.mean_ly, tx = 1 << lx, ty = 1 << ly;  // kPeriodic: pixels to a cell
-  if constexpr (FORM == kPeriodic) {
+  if constexpr (FORM == kTabulated) {
+    for (int w = kThreads - 1 - tid; w < S * T::kTab; w += kThreads) {  // the last threads first: the others fetch samples
+      const int s = w / T::kTab, r = w - s * T::kTab;
+      float v = __ldg(L.mean_k + w);
+      if (r < 16) {  // a first column or row, from the pixel's cell to the box
+        const LpaSensorK &Sk = L.s[s];
+        const int2 o = box_origin(Sk, u0, v0, BH);
+        const bool col = r < 8;
+        const int ph = (r >> 1) & 3, c = r & 1, N = ph == 1 || ph == 2 ? NG : NR;
+        const int l = (col ? u0 + Sk.ix_shift - o.x - (ph & 1) : v0 + Sk.iy_shift - o.y - (ph >> 1)) + c;
+        const int i = (l >> 1) + __float_as_int(v), last = col ? (kBW - 1) >> 1 : (BH - 1) >> 1;
+        const int at = max(min(i, ((col ? Sk.box_w : Sk.box_h) >> 1) - N - last), 0);
+        if (at != i && (col ? u0 + c < L.out_w : v0 + c < y_end)) atomicOr(L.status, LPA_ERR_BOUNDS);
+        v = __int_as_float(col ? at : at * (Sk.box_w >> 1));
+      }
+      xt[w] = v;
+    }
+  } else if constexpr (FORM == kPeriodic) {
     // one entry per sensor, axis and class of positions: class c starts at G c + G_t, and the n-th
     // pixel of a class lies exactly 2 n px further, whatever the tile
     const int entry = kThreads - 1 - tid;  // by the last threads: the first ones fetch samples
@@ -197,7 +223,8 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
 
   // this thread's column and its P rows: row0 + k, or (kPeriodic) row0 + ty k
   const int col = (tid & 31) + 32 * ((tid >> 5) & 1), group = tid >> 6;
-  const int row0 = FORM == kPeriodic ? (group >> ly) * (P << ly) + (group & (ty - 1)) : group * P;
+  constexpr bool kClasses = FORM == kPeriodic || FORM == kTabulated;
+  const int row0 = kClasses ? (group >> ly) * (P << ly) + (group & (ty - 1)) : group * P;
   const int u = u0 + col;
   Sums<COMP> acc[P][3];  // per row and channel
 
@@ -215,19 +242,35 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
     const LpaSensorK &Sk = L.s[s];
     const float2 *planes = reinterpret_cast<const float2 *>(smem + (s - s0) * L.mean_plane);
     const int PW = Sk.box_w >> 1, PP = PW * (Sk.box_h >> 1);
-    if constexpr (FORM == kPeriodic) {
+    if constexpr (kClasses) {
       const float *ex = xt + (s * (tx + ty) + (col & (tx - 1))) * T::kRow;
       const float *ey = xt + (s * (tx + ty) + tx + (group & (ty - 1))) * T::kRow;
       const int shift = (col >> lx) + (group >> ly) * P * PW;  // whole cells from the class's first pixel
       auto phase = [&](auto N_, auto c_, int ox, int oy, int g) {
         constexpr int N = decltype(N_)::value, c = decltype(c_)::value;
-        const float *fx = ex + 4 + 2 * NR * g + N * ox, *fy = ey + 4 + 2 * NR * g + N * oy;
         float K[N][N];
+        const float2 *pl;
+        if constexpr (FORM == kTabulated) {
+          const int pu = col & 1, pv = group & 1, ph = ox + 2 * oy;
+          const float *t = xt + s * T::kTab;
+          const float4 *k = reinterpret_cast<const float4 *>(t + 16 + (2 * pv + pu) * T::kClass + T::phase_words(ph));
 #pragma unroll
-        for (int j = 0; j < N; j++)
+          for (int j = 0; j < N * N; j += 4) {
+            const float4 q = k[j / 4];
+            const float e[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-          for (int i = 0; i < N; i++) K[j][i] = fmaxf(fmaf(fx[i], fy[j], -L.taper), 0.f);
-        const float2 *pl = planes + (ox + 2 * oy) * PP + shift + __float_as_int(ex[2 * g + ox]) + __float_as_int(ey[2 * g + oy]);
+            for (int i = 0; i < 4; i++)
+              if (j + i < N * N) K[(j + i) / N][(j + i) % N] = e[i];
+          }
+          pl = planes + ph * PP + shift + __float_as_int(t[2 * ph + pu]) + __float_as_int(t[8 + 2 * ph + pv]);
+        } else {
+          const float *fx = ex + 4 + 2 * NR * g + N * ox, *fy = ey + 4 + 2 * NR * g + N * oy;
+#pragma unroll
+          for (int j = 0; j < N; j++)
+#pragma unroll
+            for (int i = 0; i < N; i++) K[j][i] = fmaxf(fmaf(fx[i], fy[j], -L.taper), 0.f);
+          pl = planes + (ox + 2 * oy) * PP + shift + __float_as_int(ex[2 * g + ox]) + __float_as_int(ey[2 * g + oy]);
+        }
 #pragma unroll
         for (int r = 0; r < N + P - 1; r++)
 #pragma unroll
@@ -344,7 +387,7 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
   if (u >= L.out_w || (status & LPA_ERR_TIMEOUT)) return;
   // per channel: a pointer to the first row's pixel and the step to the next
   const size_t plane = (size_t)L.out_w * L.out_h, first = (size_t)(v0 + row0) * L.out_w + u;
-  const int step = FORM == kPeriodic ? ly : 0;
+  const int step = kClasses ? ly : 0;
   const uint32_t next = (uint32_t)L.out_w << step;
   const int rows = v0 + row0 < y_end ? ((y_end - v0 - row0 - 1) >> step) + 1 : 0;
 #pragma unroll
@@ -375,19 +418,21 @@ __global__ void __launch_bounds__(lpa_mean_threads(P), P == 8 ? 3 : 2) lpa_mean(
   }
 }
 
-// The kernel of plan L for window size (NR, NG), plain (any rows per thread) or compensated (two).
+// The kernel of plan L for window size (NR, NG), plain (one, two or the most rows per thread) or compensated (two).
 template <int NR, int NG, int FORM, bool COMP>
 const void *pick_rows(int p) {
   if constexpr (COMP) return (const void *)lpa_mean<NR, NG, FORM, 2, true>;
-  else
+  else {
+    constexpr int kMost = FORM == kPeriodic || FORM == kTabulated ? 8 : 4;
     return p == 1   ? (const void *)lpa_mean<NR, NG, FORM, 1, false>
            : p == 2 ? (const void *)lpa_mean<NR, NG, FORM, 2, false>
-           : p == 8 && FORM == kPeriodic ? (const void *)lpa_mean<NR, NG, kPeriodic, 8, false>
-                    : (const void *)lpa_mean<NR, NG, FORM, 4, false>;
+                    : (const void *)lpa_mean<NR, NG, FORM, kMost, false>;
+  }
 }
 template <int NR, int NG, bool COMP>
 const void *pick(const LpaLaunch &L) {
-  return L.mean_lx           ? pick_rows<NR, NG, kPeriodic, COMP>(L.mean_p)
+  return L.mean_k            ? pick_rows<NR, NG, kTabulated, COMP>(L.mean_p)
+         : L.mean_lx         ? pick_rows<NR, NG, kPeriodic, COMP>(L.mean_p)
          : L.mean_axis == 1 ? pick_rows<NR, NG, kAxis, COMP>(L.mean_p)
          : L.mean_axis == 2 ? pick_rows<NR, NG, kFactored, COMP>(L.mean_p)
                             : pick_rows<NR, NG, kGeneral, COMP>(L.mean_p);

@@ -8,6 +8,7 @@ sensors, one and eight sensors, and the larger tiles of big frames on sampled pi
 rule of tests/parity.py, unchanged.
 """
 import dataclasses
+import math
 
 import numpy as np
 import pytest
@@ -234,6 +235,16 @@ def test_boxes_on_an_alignment_boundary(ctx, scale, rot, nudge):
     _against_oracle(fr, out, ch, _every_pixel(fr.params))
 
 
+def _edge_frame(**over):
+    """Three exactly translated sensors whose red samples lie within 1e-5 px of the edge of every even pixel's
+    window, so that their window values are a few 1e-7 of the centre's."""
+    fr = _frame(70, 41, 0.0, n=3, sigma=1.3 / 3, **over)
+    for k, s in enumerate(fr.sensors):
+        s.affine = np.array([[1.0, 0.0, 1.0], [0.0, 1.0, math.sqrt((1.3 - 1e-5 * (k + 1)) ** 2 - 1.0)]])
+        s.raw = synth.simulate_raw(fr.scene, s, 1500, k)
+    return fr
+
+
 def _without_window_rounding(fr, out):
     """Every pixel within the parity rule's terms for conversion and FP32 sums alone: window values that are exact
     to one rounding need nothing of the term for their evaluation (ew)."""
@@ -247,9 +258,64 @@ def _without_window_rounding(fr, out):
     assert (np.abs(g - o["out"])[m] <= tol[m]).all(), float((np.abs(g - o["out"])[m] / tol[m]).max())
 
 
+def test_tabulated_weights_at_the_window_edge(ctx):
+    """tab_weights 1: window values formed in FP64. In FP32 they are off by parts in a thousand at the edge of
+    a window, and so are the estimates there."""
+    fr = _edge_frame()
+    _without_window_rounding(fr, _run(ctx, fr)[0])
+
+
+@pytest.mark.parametrize("w,h", [(832, 380), (832, 760), (1250, 1010)])  # one, two and eight rows per thread
+@pytest.mark.parametrize("sigma,accum", [(0.7, 0), (1.2, 0), (1.2, 1)])
+def test_tabulated_weights_in_every_entry_point(ctx, w, h, sigma, accum):
+    """Sampled pixels against the oracle, and the same bits from a batch, the host-buffer bands and a first call
+    under stream capture, whose table is not there yet."""
+    from paper_1308_4908_gb300 import hdr
+    fr = _frame(w, h, 0.0, n=3, sigma=sigma, accum=accum)
+    out, ch, raws = _run(ctx, fr)
+    p = fr.params
+    r = np.random.default_rng(w)
+    pix = np.concatenate([np.stack([r.integers(0, w, 1500), r.integers(0, h, 1500)], 1),
+                          [[0, 0], [w - 1, 0], [0, h - 1], [w - 1, h - 1]]])
+    _against_oracle(fr, out, ch, pix)
+    o = torch.full((3, h, w), -7.0, device="cuda")
+    keep = [raws]
+    ctx.reconstruct_batch([ctx.frame(0, p, raws, o, None, keep)])
+    ctx.check()
+    np.testing.assert_array_equal(o.cpu().numpy(), out)
+    host = np.full((3, h, w), -7.0, np.float32)
+    ctx.reconstruct_host(0, p, [np.ascontiguousarray(s.raw) for s in fr.sensors], host)
+    np.testing.assert_array_equal(host, out)
+    own = hdr.Context(0)
+    try:
+        own.set_rig(0, fr.sensors)
+        o.fill_(-7.0)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            own.reconstruct(0, p, raws, out=o)
+        g.replay()
+        torch.cuda.synchronize()
+        own.check()
+    finally:
+        own.close()
+    np.testing.assert_array_equal(o.cpu().numpy(), out)
+
+
 @pytest.mark.parametrize("trunc_k", [0.05, 0.3, 0.99])
 def test_windows_cut_close_in(ctx, trunc_k):
     """Windows cut below one sigma, where the window value is the difference of nearly equal exponentials: left to
     the tabulated windows' general kernel."""
     fr = _frame(71, 45, 0.0, n=3, sigma=2.0 / trunc_k, trunc_k=trunc_k)
     _without_window_rounding(fr, _run(ctx, fr)[0])
+
+
+@pytest.mark.parametrize("sigma,rot,n", [(1.2, 0.0, 2), (1.2, 0.2, 2), (0.7, 0.0, 4), (1.2, 0.0, 4)])
+def test_largest_tiles_enlarged(ctx, sigma, rot, n):
+    """Twofold output of at least four tiles of 64 x 32 per SM and CTA: the largest tiles of each form and window size,
+    sampled pixels and the border."""
+    fr = _frame(625, 505, rot, n=n, sigma=sigma, out_w=1250, out_h=1010, out_affine=synth.output_affine(625, 505, 1250, 1010))
+    out, ch, _ = _run(ctx, fr)
+    r = np.random.default_rng(n)
+    pix = np.concatenate([np.stack([r.integers(0, 1250, 2000), r.integers(0, 1010, 2000)], 1),
+                          np.stack([np.arange(1250), np.full(1250, 1009)], 1), np.stack([np.full(1010, 1249), np.arange(1010)], 1)])
+    _against_oracle(fr, out, ch, pix)
