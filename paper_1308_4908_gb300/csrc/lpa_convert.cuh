@@ -37,8 +37,8 @@ __device__ __forceinline__ float2 convert_sample(const LpaSensorK &Sk, bool plai
     if (y < sat) {
       const float a = Sk.prnu ? Sk.prnu[px] : 1.f;
       const float e0 = y - b;
-      f = div_approx(e0 * Sk.inv_gtn, a);
-      iv = div_approx(Sk.gtn2 * a * a, fmaf(Sk.gain, fmaxf(e0, 0.f), rv));
+      f = __fdividef(e0 * Sk.inv_gtn, a);  // (denormal divisors too, unlike div_approx)
+      iv = __fdividef(Sk.gtn2 * a * a, fmaf(Sk.gain, fmaxf(e0, 0.f), rv));
       if (LIT) iv = sqrtf(iv);
       if (!(iv > 0.f && fabsf(iv * f) <= 3.402823466e38f)) f = iv = 0.f;
     }

@@ -57,6 +57,7 @@ struct RigSensor {
 
 struct Rig {
   int n = 0;
+  int weight_exp = 0;  // weight_exponent() of its sensors
   RigSensor s[HDR_MAX_SENSORS];
 };
 
@@ -252,6 +253,33 @@ hdr_status check_sensors(int32_t n_sensors, const hdr_sensor_desc *sensors) {
         return fail(HDR_E_INVALID, "sensor %d: read_var_frame must be finite and > 0", s);
   }
   return HDR_OK;
+}
+
+// An even exponent k: the kernels stage inverse variances times 2^k. Values and choices do not depend on a
+// common factor of the weights, and a power of two changes no rounding, so k is 0 unless the rig's units would take
+// FP32 sums near the ends of its range: a sensor's smallest weights (its brightest samples') below 2^-90 (their
+// sums over small windows, and pivots of higher orders, are smaller yet, and rcp_approx gives infinity below
+// 2^-126) or above 2^80. The largest of the sensors' smallest weights then comes to about 1. Per-pixel frames count
+// by their median (of at most 4096 pixels): single pixels may hold anything.
+int weight_exponent(int32_t n_sensors, const hdr_sensor_desc *sensors) {
+  auto typical = [](const float *frame, size_t n, double scalar) {
+    if (!frame) return scalar;
+    std::vector<float> v;
+    for (size_t i = 0, step = (n + 4095) / 4096; i < n; i += step) v.push_back(frame[i]);
+    std::nth_element(v.begin(), v.begin() + v.size() / 2, v.end());
+    return (double)v[v.size() / 2];
+  };
+  double lo = HUGE_VAL, hi = 0.0;
+  for (int s = 0; s < n_sensors; s++) {
+    const hdr_sensor_desc &d = sensors[s];
+    const size_t n = (size_t)d.width * d.height;
+    const double gtn = d.gain * d.exposure * d.nd * typical(d.prnu_frame, n, 1.0);
+    const double w = gtn * gtn / (d.gain * 65535.0 + typical(d.read_var_frame, n, d.read_var));
+    lo = std::min(lo, w);
+    hi = std::max(hi, w);
+  }
+  if ((lo >= 0x1p-90 && hi <= 0x1p80) || !(hi > 0.0) || !std::isfinite(hi)) return 0;
+  return std::min(std::max(-std::ilogb(hi) / 2 * 2, -240), 240);
 }
 
 hdr_status check_params(const hdr_params *p) {
@@ -762,7 +790,8 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   for (int j = 0; j < p->n_scales; j++) L.sigma[j] = (float)p->sigma[j];
   L.green_ratio = (float)p->green_ratio;
   L.trunc_k = (float)p->trunc_k;
-  L.ici_gamma = (float)p->ici_gamma;
+  L.weight_exp = rig.weight_exp;
+  L.ici_gamma = (float)std::ldexp(p->ici_gamma, rig.weight_exp / 2);  // (Var C_0 comes out times 2^-weight_exp)
   L.min_pivot = (float)p->min_pivot;
   L.cond_fallback = (float)p->cond_fallback;
   L.taper = (float)std::exp(-0.5 * p->trunc_k * p->trunc_k);
@@ -811,7 +840,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     K.hy_unit = (float)hyu;
     const double gtn = d.gain * d.exposure * d.nd;
     K.inv_gtn = (float)(1.0 / gtn);
-    K.gtn2 = (float)(gtn * gtn);
+    K.gtn2 = (float)std::ldexp(gtn * gtn, rig.weight_exp);
     K.gain = (float)d.gain;
     K.read_var = (float)d.read_var;
     K.black = (float)d.black;
@@ -1222,6 +1251,7 @@ hdr_status hdr_set_rig(hdr_ctx *ctx, int32_t rig_id, int32_t n_sensors, const hd
   }
   Rig fresh;
   fresh.n = n_sensors;
+  fresh.weight_exp = weight_exponent(n_sensors, sensors);
   for (int s = 0; s < n_sensors; s++) {
     RigSensor &rs = fresh.s[s];
     rs.d = sensors[s];
@@ -2156,6 +2186,7 @@ extern "C" hdr_status hdr_reconstruct_noalloc(int device, int32_t n_sensors, con
   CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned int), stream));
   Rig rig;
   rig.n = n_sensors;
+  rig.weight_exp = weight_exponent(n_sensors, sensors);
   size_t off = kScratchHeader;
   for (int s = 0; s < n_sensors; s++) {
     RigSensor &rs = rig.s[s];

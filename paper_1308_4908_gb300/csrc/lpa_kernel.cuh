@@ -1147,7 +1147,7 @@ __device__ __forceinline__ bool process_tile(const LpaLaunch &L, const LpaLaunch
       if (DIAG && pix) {
         float *o = L.levels + (((size_t)c * NL + level) * plane_px + index()) * 2;
         o[0] = f.valid ? f.c0 : __int_as_float(0x7fffffff);
-        o[1] = f.valid ? f.var : __int_as_float(0x7fffffff);
+        o[1] = f.valid ? ldexpf(f.var, L.weight_exp) : __int_as_float(0x7fffffff);
       }
     };
     // order fallback at the largest scale (m holds its moments when any lane needs it), then the store

@@ -121,6 +121,7 @@ struct LpaLaunch {
   // colour phase ph = ox + 2 oy, in cells from the pixel's even lattice cell; a class holds the weights
   // of its four phases' candidate cells, row by row, where lpa_mean_k_word puts them.
   const float *mean_k;
+  int weight_exp;                // inverse variances are staged times 2^weight_exp (ici_gamma allows for it)
 };
 
 // LPA_SEARCHED_F32, LPA_STEERED_F32, LPA_TABULATED_F32: the searched, steered or tabulated window

@@ -15,9 +15,9 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// 1 / x as the FP32 reciprocal unit gives it: __fdividef(1, x) for every normal x. That function also
-// scales denormal x (four instructions for one), of which it can return only the reciprocals of [2^-128,
-// 2^-126) as finite numbers; here these are infinite too.
+// 1 / x as the FP32 reciprocal unit gives it: __fdividef(1, x) for every normal x. Denormal x, whose reciprocals
+// that function takes care of, give infinity here: callers' divisors are normal (weights are kept
+// away from the ends of the range by LpaLaunch::weight_exp, conversions by LpaSensorK::plain).
 __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
