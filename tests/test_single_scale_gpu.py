@@ -88,3 +88,28 @@ def test_window_sizes_of_the_fixed_walk(ctx, order, sigma, green, zoom):
         got.append((out.cpu().numpy(), ch.cpu().numpy()))
     np.testing.assert_array_equal(got[0][0], got[1][0])
     np.testing.assert_array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("sigma,green", [(0.79, 1.0), (0.81, 0.9), (0.99, 0.7), (1.0, 0.8), (1.12, 1.0), (1.14, 0.7), (1.33, 0.6), (1.34, 0.6)])
+def test_fixed_walk_at_order_0(ctx, sigma, green):
+    """Order 0 outside its own kernel (a pivot threshold next to 1), on both sides of the reaches from which its
+    windows take a fixed block of cells (2.4 to 3 and 3.4 to 4 px): the same bits as the kernels that search."""
+    from paper_1308_4908_gb300 import hdr
+    fr = _frame(False, 1)
+    p = dataclasses.replace(fr.params, order=0, sigmas=(sigma,), green_ratio=green, min_pivot=0.995, out_w=50, out_h=47)
+    ctx.set_rig(0, fr.sensors)
+    raws = [torch.from_numpy(s.raw).cuda() for s in fr.sensors]
+    got = []
+    for batch in (False, True):
+        out = torch.full((3, 47, 50), -7.0, device="cuda")
+        ch = torch.empty((3, 47, 50), dtype=torch.uint8, device="cuda")
+        if batch:
+            keep = [raws]
+            ctx.reconstruct_batch([ctx.frame(0, p, raws, out, ch, keep)], hdr.hdr_batch_config(16, 0, 1, 0, 2, 1))
+        else:
+            ctx.reconstruct(0, p, raws, out=out, choice=ch)
+        ctx.check()
+        got.append((out.cpu().numpy(), ch.cpu().numpy()))
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    np.testing.assert_array_equal(got[0][1], got[1][1])
+    assert np.isfinite(got[0][0]).mean() > 0.5
