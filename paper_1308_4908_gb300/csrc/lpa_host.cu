@@ -358,7 +358,8 @@ struct MeanPlan {
 // Rows per thread: four, or eight of half as many threads in the periodic form, once 64 x 32 tiles fill
 // the SMs' two resident CTAs twice (less halo converted per pixel), fewer for smaller frames (more CTAs);
 // two of compensated sums (24 registers of sums a row).
-MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
+// tables: weights may be tabulated (the entry point has the context's caches).
+MeanPlan mean_plan(const Rig &rig, const hdr_params *p, bool tables) {
   MeanPlan m;
   // (its grid has a row of tiles per y index: at most 65535 of 8 rows)
   if (p->out_h > 65535 * 8 || p->order != 0 || p->n_scales != 1 || p->weight_mode != 0 || !(p->trunc_k >= 1.0) || !(p->min_pivot < 0.99) ||
@@ -367,7 +368,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
   m.rb = p->trunc_k * p->sigma[0];
   m.g = m.rb * p->green_ratio;
   m.axis = p->out_affine[1] == 0.0 && p->out_affine[3] == 0.0;
-  m.tab = p->tab_weights == 1 && is_identity_linear(p->out_affine);
+  m.tab = tables && p->tab_weights == 1 && is_identity_linear(p->out_affine);
   double most = 0.0;
   auto period = [](double step) {  // of positions modulo 2 px, to the tolerance of the tabulated weights
     return std::fabs(step - 1.0) <= 1e-12 ? 2 : std::fabs(step - 0.5) <= 1e-12 ? 4 : 0;
@@ -386,6 +387,7 @@ MeanPlan mean_plan(const Rig &rig, const hdr_params *p) {
     m.even = m.even && std::fabs(a[0] * a[1] + a[3] * a[4]) <= 1e-9 * std::min(a[0] * a[0] + a[3] * a[3], a[1] * a[1] + a[4] * a[4]);
   }
   if (!m.axis || !m.tx || !m.ty) m.tx = m.ty = 0;
+  if (m.tab) m.axis = true, m.tx = m.ty = 2;  // (to the tolerance of is_identity_linear)
   m.size = lpa_mean_size(m.rb * most + 2e-3, m.g * most + 2e-3);
   const long long px = (long long)p->out_w * p->out_h;
   m.p = p->accum ? 2 : px >= 4LL * 152 * 64 * 32 ? (m.tx ? 8 : 4) : px >= 4LL * 152 * 64 * 16 ? 2 : 1;
@@ -454,7 +456,7 @@ uint32_t mean_smem(const Rig &rig, const hdr_params *p, const MeanPlan &m, int *
 }
 
 bool runs_mean(const Rig &rig, const hdr_params *p) {
-  const MeanPlan m = mean_plan(rig, p);
+  const MeanPlan m = mean_plan(rig, p, true);
   int bufs;
   uint32_t plane, tab;
   return m.size >= 0 && mean_smem(rig, p, m, &bufs, &plane, &tab) > 0;
@@ -809,7 +811,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
   int max_smem = 0;
   CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, env.device));
   MeanPlan mean;
-  if (env.mean) mean = mean_plan(rig, p);
+  if (env.mean) mean = mean_plan(rig, p, env.tabs && env.tabulate);
   if (env.grad) mean = grad_plan(rig, p);
   if (mean.size >= 0) {
     L.smem_bytes = mean_smem(rig, p, mean, &L.mean_bufs, &L.mean_plane, &L.mean_tab);
@@ -954,7 +956,7 @@ hdr_status plan_env(const PlanEnv &env, const Rig &rig, const hdr_params *p, con
     L.mean_ly = mean.ty / 2;
     if (L.tiles_x > 0 && L.tiles_y > 0) lpa_mean_rows(L, 0, L.tiles_x * L.tiles_y);
     L.stages = 1;
-    return mean.tab && env.tabs && env.tabulate ? mean_weights(env, rig, p, mean, L) : HDR_OK;
+    return mean.tab ? mean_weights(env, rig, p, mean, L) : HDR_OK;
   }
   L.tx_bytes = tx;
   // a usable fit's equilibrated pivots lie in (min_pivot, 1]: when min_pivot * cond_fallback >= 2

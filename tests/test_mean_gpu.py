@@ -265,6 +265,16 @@ def test_tabulated_weights_at_the_window_edge(ctx):
     _without_window_rounding(fr, _run(ctx, fr)[0])
 
 
+@pytest.mark.parametrize("scale,shear", [(5e-13, 0.0), (0.0, 5e-13), (-4e-13, -3e-13)])
+def test_nearly_exact_translations(ctx, scale, shear):
+    """Sensors whose linear part is the identity to the tolerance of the tabulated weights, but not exactly."""
+    fr = _frame(131, 34, 0.0)
+    for s in fr.sensors:
+        s.affine = np.array(s.affine) + np.array([[scale, shear, 0.0], [-shear, scale, 0.0]])
+    out, ch, _ = _run(ctx, fr)
+    _against_oracle(fr, out, ch, _every_pixel(fr.params))
+
+
 @pytest.mark.parametrize("w,h", [(832, 380), (832, 760), (1250, 1010)])  # one, two and eight rows per thread
 @pytest.mark.parametrize("sigma,accum", [(0.7, 0), (1.2, 0), (1.2, 1)])
 def test_tabulated_weights_in_every_entry_point(ctx, w, h, sigma, accum):
