@@ -17,7 +17,7 @@ constexpr int kThreads = 256;
 constexpr int kMaxFrames = 4096;      // exact integer sums: n * sum y^2 < 2^63
 constexpr int kReduceBlocks = 304;    // fixed grid: the summation order does not depend on timing
 
-// num / den correctly rounded to FP32 for integers num = hi + lo (|lo| below 2^16, hi 0 or above
+// num / den correctly rounded to FP32 for integers num = hi + lo (|lo| at most 2^32, hi 0 or above
 // |lo|) and den in [1, 2^24) (rden: its FP32 reciprocal). The quotient is formed as a pair qh + ql
 // with an error below 2^-20 ulp of qh: qh is the answer unless the exact quotient lies within 2^-15
 // ulp of the midpoint of two floats, where `exact` (an FP64 division) decides.

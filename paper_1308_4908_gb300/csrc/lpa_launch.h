@@ -102,16 +102,16 @@ struct LpaLaunch {
   const int4 *tab_hdr;           // bounds packed as (min & 0xffff) | (max << 16)
   const float4 *tab_cells;
   int tab_nsp;                   // scales per pass the table was built for
-  // Kernel mode (LPA_SEARCHED .. LPA_TABULATED_F32 below). Adaptive reconstruction (Sections 5.4-5.5):
+  // Kernel mode (LPA_SEARCHED .. LPA_MEAN below). Adaptive reconstruction (Sections 5.4-5.5):
   // LPA_STEERED reads the steering matrix of each output pixel from aux ([out_h][out_w][3]: C11,
   // C12, C22); LPA_GRADIENTS writes the gradient of the green fit to aux ([out_h][out_w][2]).
   // LPA_LITERAL: the searched window with the noise weight printed in Eq. 6 (K / s, not K / s2).
   int mode;
   float *aux;
-  // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, its form (1: every
-  // sensor's axes parallel to the output's, 2: every sensor's map a rotation and an even scale, 0: any), the pixels that span one cell of a colour phase where that is exact for
-  // every sensor (as powers of two, 1 or 2 on each axis, else both 0), sensors staged at a time, bytes of one sensor's
-  // colour-phase planes (from offset 0) and the offset of the position tables
+  // LPA_MEAN (lpa_mean.cu): rows per thread, the candidate cells' template, its form (1: every sensor's axes parallel
+  // to the output's, 2: every sensor's map a rotation and an even scale, 0: any), the pixels that span one cell of a
+  // colour phase where that is exact for every sensor (as powers of two, 1 or 2 on each axis, else both 0), sensors
+  // staged at a time, bytes of one sensor's colour-phase planes (from offset 0) and the offset of the position tables
   int mean_p, mean_size, mean_axis, mean_lx, mean_ly, mean_bufs;
   int mean_comp;                 // compensated sums
   int mean_y0, mean_y1;          // output rows of the launch (lpa_mean_rows)

@@ -15,9 +15,9 @@
 // two in flight per thread) and converted once per sample (Eqs. 18 and 20) into colour-phase planes of
 // (1 / s2, f / s2) in shared memory; one barrier later the sums of every sensor follow. Each cell is
 // then one shared load and one paired FMA into (sum K / s2, sum K f / s2). No conversion pass goes
-// ahead of the kernel: with 64 x 32 tiles a sample is converted about 1.5 times, and the pass cost
-// 47 us of 517 on four 2336 x 1752 sensors. Measured against the general kernel with that pass: 2 x 2048^2 ->
-// 4096^2 FP16 1226 -> 136 us, the four sensors (tabulated windows before) 517 -> 87 us, 64^2 14.4 -> 6.3 us a call (2.9
+// ahead of the kernel: with 64 x 32 tiles (boxes of 80 x 42 samples at 1x) a sample is converted 1.64 times, and the
+// pass cost 47 us of 517 on four 2336 x 1752 sensors. Measured against the general kernel with that pass: 2 x 2048^2 ->
+// 4096^2 FP16 1226 -> 136 us, the four sensors (tabulated windows) 517 -> 84 us, 64^2 14.4 -> 6.3 us a call (2.9
 // of it in the binding); 1024 x 900, three rotated sensors 147 -> 58 us, compensated 201 -> 106 us.
 //
 // kAxis: every sensor's axes are parallel to the output's, so the Gaussian factors into a column and
