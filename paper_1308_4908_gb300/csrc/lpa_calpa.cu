@@ -23,6 +23,8 @@ struct MetricArgs {
   int cells;                       // cells of the disc (pixels whose disc lies inside the image)
   int rw[2 * kRmax + 1];           // half width of the disc in row offset dj (|di| <= rw)
   float2 w[2 * kRmax * kRmax + 1];  // Gaussian weight by di^2 + dj^2, as a pair
+  double w64[2 * kRmax * kRmax + 1];  // and in FP64
+  double scale2;                     // grad_scale^2
   // grad_scale = unit m with unit a power of two (the gradients are staged times it, exactly) and
   // m in [1, 2): T of the scaled gradients is m^2 (a pair) times the sums
   float unit;
@@ -140,41 +142,63 @@ __device__ __forceinline__ void store_matrix(const MetricArgs &A, int r, const D
   const float2 h = make_float2(0.5f * sum.x, 0.5f * sum.y), t = make_float2(0.5f * dif.x, 0.5f * dif.y);
   const float2 d = pair_sqrt(pair_add(pair_mul(t, t), pair_mul(b, b)));
   const float2 l1 = pair_add(h, d), l2 = pair_add(h, pair_neg(d));
-  // the eigenvector's longer form: |l1 - c| > |l1 - a| where a > c
-  float ux = b.x, uy = b.x;
-  if (dif.x > 0.f) ux = pair_add(l1, pair_neg(c)).x;
-  else uy = pair_add(l1, pair_neg(a)).x;
+  // the eigenvector of l1 in its longer form: |l1 - c| > |l1 - a| where a > c
+  const bool wide = dif.x > 0.f;
+  const float2 Ux = wide ? pair_add(l1, pair_neg(c)) : b, Uy = wide ? b : pair_add(l1, pair_neg(a));
+  float ux = Ux.x, uy = Uy.x;
   float L1 = l1.x * up, L2 = fmaxf(l2.x, 0.f) * up;
-  // Nearly rank one: the pairs hold l2 to about 2^-45 l1, less than an FP32 value needs below this
-  // ratio (noise keeps it above in camera frames; a lone gradient or a clean ramp is below), so T and
-  // its eigenvalues are formed again in FP64, from the gradients: sums and products with the scale that left FP32's range (not a
-  // number here) come this way too.
   if (!(l2.x >= 0x1p-18f * l1.x)) {
-    double da = 0.0, db = 0.0, dc = 0.0;
-    for (int dj = max(-r, -v); dj <= min(r, A.H - 1 - v); dj++) {
-      const int rw = A.rw[dj + r];
-      const float2 *row = A.grad + (size_t)(v + dj) * A.W + u;
-      for (int di = max(-rw, -u); di <= min(rw, A.W - 1 - u); di++) {
-        const float2 wp = A.w[di * di + dj * dj], g = row[di];
-        const double w = (double)wp.x + (double)wp.y, gx = (double)g.x * (double)A.unit, gy = (double)g.y * (double)A.unit;
-        da = fma(w, gx * gx, da);
-        db = fma(w, gx * gy, db);
-        dc = fma(w, gy * gy, dc);
+    if (l1.x <= 3.402823466e38f) {
+      // Nearly rank one: the pairs hold l2 to about 2^-45 l1, less than an FP32 value needs below this ratio (noise keeps
+      // it above in camera frames; clean edges and ramps, and lone gradients, are below). Their eigenvector is good to
+      // 2^-44 all the same, so l2 is summed again as w (g . v)^2 over the disc, v across it: g . v from exact products,
+      // no cancellation after it. 1920 x 1080 clean gradients with the default disc: 0.13 ms; FP64 sums there 1.37 ms (0.55 ms
+      // where every pixel is summed in FP64, from staged products), and these hold l2 to 2^-52 l1 only.
+      const int eh = (127 - et) >> 1;
+      const float half = __int_as_float((127 + eh) << 23), back = __int_as_float((127 - eh) << 23);
+      float sum = 0.f, rest = 0.f;  // and what its additions rounded away
+      for (int dj = max(-r, -v); dj <= min(r, A.H - 1 - v); dj++) {
+        const int rw = A.rw[dj + r];
+        const float2 *row = A.grad + (size_t)(v + dj) * A.W + u;
+        for (int di = max(-rw, -u); di <= min(rw, A.W - 1 - u); di++) {
+          const float2 g = row[di];
+          const float gx = g.x * A.unit * half, gy = g.y * A.unit * half;
+          const float px = __fmul_rn(gy, Ux.x), py = __fmul_rn(gx, Uy.x);
+          const float low = (__fmaf_rn(gy, Ux.x, -px) - __fmaf_rn(gx, Uy.x, -py)) + (gy * Ux.y - gx * Uy.y);
+          const float q = __fadd_rn(__fsub_rn(px, py), low);
+          const float term = A.w[di * di + dj * dj].x * q * q, next = __fadd_rn(sum, term);
+          rest += __fsub_rn(term, __fsub_rn(next, sum));
+          sum = next;
+        }
       }
+      L2 = (sum + rest) / fmaf(ux, ux, uy * uy) * A.m2.x * back * back;
+    } else {
+      // sums, or products with the scale, that left FP32's range: in FP64 from the gradients
+      double da = 0.0, db = 0.0, dc = 0.0;
+      for (int dj = max(-r, -v); dj <= min(r, A.H - 1 - v); dj++) {
+        const int rw = A.rw[dj + r];
+        const float2 *row = A.grad + (size_t)(v + dj) * A.W + u;
+        for (int di = max(-rw, -u); di <= min(rw, A.W - 1 - u); di++) {
+          const float2 g = row[di];
+          const double w = A.w64[di * di + dj * dj], gx = g.x, gy = g.y;
+          da = fma(w, gx * gx, da);
+          db = fma(w, gx * gy, db);
+          dc = fma(w, gy * gy, dc);
+        }
+      }
+      da *= A.scale2;
+      db *= A.scale2;
+      dc *= A.scale2;
+      const double dh = 0.5 * (da + dc), dd = sqrt(0.25 * (da - dc) * (da - dc) + db * db);
+      L1 = (float)(dh + dd);
+      L2 = (float)fmax(dh - dd, 0.0);
+      const double vx = da > dc ? dh + dd - dc : db, vy = da > dc ? db : dh + dd - da;
+      // into FP32's range before the conversion, by a power of two
+      const int vexp = (__double2hiint(fmax(fabs(vx), fabs(vy))) >> 20) & 2047;
+      const double vunit = __hiloint2double(min(max(2046 - vexp, 1), 2046) << 20, 0);
+      ux = (float)(vx * vunit);
+      uy = (float)(vy * vunit);
     }
-    const double m2 = (double)A.m2.x + (double)A.m2.y;
-    da *= m2;
-    db *= m2;
-    dc *= m2;
-    const double dh = 0.5 * (da + dc), dd = sqrt(0.25 * (da - dc) * (da - dc) + db * db);
-    L1 = (float)(dh + dd);
-    L2 = (float)fmax(dh - dd, 0.0);
-    const double vx = da > dc ? dh + dd - dc : db, vy = da > dc ? db : dh + dd - da;
-    // into FP32's range before the conversion, by a power of two
-    const int vexp = (__double2hiint(fmax(fabs(vx), fabs(vy))) >> 20) & 2047;
-    const double vunit = __hiloint2double(min(max(2046 - vexp, 1), 2046) << 20, 0);
-    ux = (float)(vx * vunit);
-    uy = (float)(vy * vunit);
   }
   const int ex = (__float_as_int(fmaxf(fabsf(ux), fabsf(uy))) >> 23) & 255;  // its exponent removed, exactly
   const float unit = __int_as_float(min(max(253 - ex, 1), 254) << 23);
@@ -360,7 +384,8 @@ hdr_status hdr_calpa_metric(hdr_ctx *ctx, int32_t out_w, int32_t out_h, const hd
   auto pair = [](double x) { return make_float2((float)x, (float)(x - (double)(float)x)); };
   A.cells = 0;
   for (int dj = -A.r; dj <= A.r; dj++) A.cells += 2 * A.rw[dj + A.r] + 1;
-  for (int k = 0; k <= 2 * A.r * A.r; k++) A.w[k] = pair(std::exp(-(double)k / (2.0 * ws * ws)));
+  for (int k = 0; k <= 2 * A.r * A.r; k++) A.w[k] = pair(A.w64[k] = std::exp(-(double)k / (2.0 * ws * ws)));
+  A.scale2 = calpa->grad_scale * calpa->grad_scale;
   A.unit = (float)std::ldexp(1.0, std::max(std::ilogb(calpa->grad_scale), -100));
   const double m = calpa->grad_scale / (double)A.unit;
   A.m2 = pair(m * m);

@@ -341,6 +341,37 @@ def test_metric_of_huge_gradients(ctx, window_sigma, size):
     assert eig.min() >= c.min_eig * (1 - 1e-5) and eig.max() <= c.max_eig * (1 + 1e-5)
 
 
+@pytest.mark.parametrize("size", [1e-3, 7.0, 900.0, 1e6, 1e15])
+@pytest.mark.parametrize("window_sigma", [0.2, 0.34, 1.0, 1.06, 3.6])
+def test_metric_of_one_gradient_everywhere(ctx, window_sigma, size):
+    """A plane of one oblique gradient g: T = (sum w) g g^T exactly, its small eigenvalue 0, so the matrix is known in
+    closed form. The small eigenvalue may be off by 2^-40 of the large one's square root without moving an FP32
+    matrix here; FP64 sums leave 2^-26, which moves the power by parts in ten for large gradients. The rest is
+    a dozen FP32 operations and a power of at most 0.3: 4e-6 of the larger eigenvalue."""
+    c = _calpa(window_sigma=window_sigma)
+    H, W = 37, 45
+    gx, gy = np.float32(size * 0.83), np.float32(size * -0.41)
+    g = np.empty((H, W, 2), np.float32)
+    g[...] = (gx, gy)
+    q = ctx.calpa_metric(c, torch.from_numpy(g).cuda()).cpu().numpy().astype(np.float64)
+    r = int(3 * window_sigma)
+    sw, M = np.zeros((H, W)), np.zeros((H, W))
+    for dj in range(-r, r + 1):
+        for di in range(-r, r + 1):
+            if di * di + dj * dj > (3 * window_sigma) ** 2:
+                continue
+            y0, y1, x0, x1 = max(0, -dj), min(H, H - dj), max(0, -di), min(W, W - di)
+            sw[y0:y1, x0:x1] += np.exp(-(di * di + dj * dj) / (2 * window_sigma ** 2))
+            M[y0:y1, x0:x1] += 1
+    n = np.hypot(np.float64(gx), np.float64(gy))
+    s1 = np.sqrt(sw) * n * c.grad_scale
+    e, gamma = (s1 + c.lambda1) / c.lambda1, (c.lambda2 / M) ** c.alpha
+    ea, eb = np.clip(gamma * e, c.min_eig, c.max_eig), np.clip(gamma / e, c.min_eig, c.max_eig)
+    ux, uy = np.float64(gx) / n, np.float64(gy) / n
+    want = np.stack([ea * ux * ux + eb * uy * uy, (ea - eb) * ux * uy, ea * uy * uy + eb * ux * ux], 2)
+    assert (np.abs(q - want) <= 4e-6 * ea[..., None]).all(), np.abs(q - want).max()
+
+
 @pytest.mark.parametrize("window_sigma,size,grad_scale", [(1.0, 1e34, 1e6), (1.06, 1e38, 1e6), (1.0, 1e38, 1.0), (1.0, 1e34, 3e5)])
 def test_metric_of_gradients_scaled_beyond_fp32(ctx, window_sigma, size, grad_scale):
     """Gradients times grad_scale, or the sums' larger terms, beyond FP32's range: inside the clamp, no NaN."""
